@@ -26,7 +26,7 @@ static int cuda_fail(cudaError_t e, const char* where) {
 template <typename T>
 KTab<T> make_ktab(const HostProblem& hp) {
   KTab<T> t;
-  std::memset(&t, 0, sizeof(t));
+  std::memset((void*)&t, 0, sizeof(t));
   const Tables1D& tb = hp.tab;
   const int n = hp.n;
   const double hd2 = std::pow(hp.h, hp.d - 2);
@@ -82,6 +82,10 @@ KTab<T> make_ktab(const HostProblem& hp) {
       }
     for (int k = 0; k < n; ++k) t.hlam[k] = (T)(hd2 * tb.lam[k]);
   }
+  if constexpr (std::is_same<T, double>::value) {
+    t.xVt = hp.fx.Vt;
+    t.xV = hp.fx.V;
+  }
   return t;
 }
 template KTab<double> make_ktab<double>(const HostProblem&);
@@ -117,6 +121,7 @@ static cudaError_t upload(T** dst, const T* src, size_t count) {
 
 static void free_device(DeviceData* dd) {
   cudaFree(dd->lines);
+  cudaFree(dd->xfix);
   cudaFree(dd->reg_cell_chunk);
   cudaFree(dd->reg_block_first);
   cudaFree(dd->reg_mask);
@@ -317,6 +322,9 @@ static int build_device(const HostProblem& hp, DeviceData* dd) {
   }
   cudaError_t e;
   if ((e = upload(&dd->nbr, nbr.data(), nbr.size())) != cudaSuccess) goto err;
+  if (d == 3 &&
+      (e = upload(&dd->xfix, hp.fx.xline.data(), hp.fx.xline.size())) != cudaSuccess)
+    goto err;
   if ((e = upload(&dd->lines, lines_o.data(), lines_o.size())) != cudaSuccess) goto err;
   if ((e = upload(&dd->cell_rank, dd->order.data(), dd->order.size())) != cudaSuccess) goto err;
   if ((e = upload(&dd->face_start, fstart.data(), fstart.size())) != cudaSuccess) goto err;
@@ -857,7 +865,9 @@ int sbm_autotune(sbm_problem* prob, int* shape64, int* shape32) {
   void *x = nullptr, *y = nullptr;
   cudaError_t e = cudaMalloc(&x, n * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&y, n * sizeof(double));
-  if (e == cudaSuccess) e = cudaMemset(x, 0, n * sizeof(double));
+  // an ordinary vector (0.00048 in FP64, 0.75 in FP32): the FP64 cell term
+  // takes its careful conversions on zeros
+  if (e == cudaSuccess) e = cudaMemset(x, 0x3f, n * sizeof(double));
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (e == cudaSuccess) e = cudaEventCreate(&e0);
   if (e == cudaSuccess) e = cudaEventCreate(&e1);
@@ -868,7 +878,7 @@ int sbm_autotune(sbm_problem* prob, int* shape64, int* shape32) {
     for (int vo = 0; vo < 8 && e == cudaSuccess; ++vo) {
       const int v = vo / 2;
       const bool o = vo % 2;
-      if ((v == 2 && !cell_reg_available(prob->hp, prec == 1)) || (v == 3 && prob->hp.d != 3) ||
+      if ((v == 2 && (prec == 0 || !cell_reg_available(prob->hp, true))) || (v == 3 && prob->hp.d != 3) ||
           (o && (v == 1 || v == 2 || !prob->dd.chunks[0].ordered)))
         continue;
       prob->dd.variant[prec] = v;

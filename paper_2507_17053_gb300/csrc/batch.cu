@@ -296,6 +296,8 @@ void make_table(const sbm_batch* B, const LaunchPlan& L, const T* const* x, T* c
     q.ca.ycol = yc;
     q.ca.run_bits = ct.run_bits;
     q.ca.bit_words = ct.bit_words;
+    q.ca.xfix = dd.xfix;
+    q.ca.eoff = p->hp.fx.eoff;
     q.ca.lines = dd.lines;
     q.ca.face_start = dd.face_start;
     q.ca.face_kind = dd.face_kind;
@@ -474,7 +476,7 @@ int autotune(sbm_batch* B) {
     return sbm_fail_detail(SBM_ERR_OOM, "autotune buffers");
   }
   int status = SBM_OK;
-  if ((e = cudaMemsetAsync(xbuf, 0, most * sizeof(T), B->cap)) != cudaSuccess)
+  if ((e = cudaMemsetAsync(xbuf, 0x3f, most * sizeof(T), B->cap)) != cudaSuccess)
     status = sbm_cuda_fail_detail(e, "autotune buffers");
   for (auto& [deg, ks] : by_deg) {
     if (status != SBM_OK) break;

@@ -141,7 +141,7 @@ __device__ SBM_BK_ITEM void face_item(const Prob<T>& P, const KTab<T>& tu, const
 template <typename T, int D, int N, int R>
 __device__ SBM_BK_ITEM void chunk_item(const Prob<T>& P, const KTab<T>& tu, const Item& it,
                                         int rhs) {
-  chunk_xline_build<T, D, N, R>(bk_smem, *P.kt, threadIdx.x);
+  chunk_xline_build<T, D, N, R>(bk_smem, *P.kt, P.ca.xfix, threadIdx.x);
   chunk_loop<T, D, N, R, true, kThreads>(P.ca, tu, bk_smem, rhs, it.b, it.e, 1);
 }
 
@@ -408,15 +408,20 @@ size_t smem_dn(int v, int fh, int ext, int tc) {
 
 // The persistent kernel.  U::tab<N>() is the constant-memory unit table of
 // degree N - 1 (one per translation unit and precision).
-// Resident blocks per SM the register budget is sized for: FP64 5 (48
-// registers, no spills in the item loops), FP32 6 (40; its kernels are
-// latency-bound and gain from the extra warps).
+// Resident blocks per SM the register budget is sized for: FP64 4 (64
+// registers; the fixed-point cell term, 9 problems x 3 right-hand sides: 2
+// blocks 1.48 ms, 3 1.26 ms, 4 1.19 ms; item functions compiled apart 1.25
+// ms), FP32 6 (40; its kernels are latency-bound and gain from the extra
+// warps).
 #ifndef SBM_BK_F32_MINB
 #define SBM_BK_F32_MINB 6
 #endif
+#ifndef SBM_BK_F64_MINB
+#define SBM_BK_F64_MINB 4
+#endif
 template <typename T>
 constexpr int min_blocks() {
-  return sizeof(T) == 4 ? SBM_BK_F32_MINB : 5;
+  return sizeof(T) == 4 ? SBM_BK_F32_MINB : SBM_BK_F64_MINB;
 }
 
 // TC: the variant with the tensor-core face items (FP32).  It is a separate

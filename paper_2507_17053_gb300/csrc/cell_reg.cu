@@ -1,6 +1,9 @@
 // Cell term of the continuous Galerkin apply with one thread per cell and
-// the cell's whole (p+1)^3 tile in registers (3D; FP32 for p <= 4, FP64 for
-// p <= 3): tile shape 2 of the single applies.
+// the cell's whole (p+1)^3 tile in registers (3D, FP32, p <= 4): tile shape 2
+// of the single applies.  (FP64 applies accept shape 2 for p <= 3 and run it
+// as shape 0, which gives the same bits: the register form's cell term took
+// 0.56 ms against 0.38 ms at p = 3 in double precision, and the fixed-point
+// cell term needs two registers per node and more.)
 //
 // The chunk kernel (cg_apply.cu) spends most of its issue slots outside the
 // arithmetic: staging runs in shared memory, splitting run indices, five
@@ -44,11 +47,11 @@ constexpr int reg_threads(int n) { return n == 5 ? 96 : (n == 2 ? 64 : 32); }
 
 // Resident blocks asked of the compiler, as warps per SM: FP32 p <= 3, 16
 // (128 registers, no spills; p = 3 cell term 41.2 -> 37.9 us against 12 at
-// 148 registers); p = 4 and FP64, 12 (168 registers; 14 or 16 warps spill
-// the p = 4 tile: 83 -> 102 us).
+// 148 registers); p = 4, 12 (168 registers; 14 or 16 warps spill the tile:
+// 83 -> 102 us).
 template <typename T, int N>
 constexpr int reg_min_blocks() {
-  return ((std::is_same<T, float>::value && N <= 4) ? 16 : 12) * 32 / reg_threads(N);
+  return (N <= 4 ? 16 : 12) * 32 / reg_threads(N);
 }
 
 template <int N>
@@ -387,27 +390,16 @@ cudaError_t build_cell_reg_tables(const HostProblem& hp, const std::vector<int32
   return e;
 }
 
-template <typename T>
-cudaError_t launch_cell_reg(const HostProblem& hp, const DeviceData& dd, const T* x, T* y,
-                            const T* fo, T* ycol, cudaStream_t st, bool pdl) {
-  if (!cell_reg_available(hp, std::is_same<T, float>::value) || !dd.reg_mask)
-    return cudaErrorInvalidValue;
+cudaError_t launch_cell_reg(const HostProblem& hp, const DeviceData& dd, const float* x, float* y,
+                            const float* fo, float* ycol, cudaStream_t st, bool pdl) {
+  if (!cell_reg_available(hp, true) || !dd.reg_mask) return cudaErrorInvalidValue;
   switch (hp.n) {
-    case 2: return launch_reg<T, 2>(hp, dd, x, y, fo, ycol, st, pdl);
-    case 3: return launch_reg<T, 3>(hp, dd, x, y, fo, ycol, st, pdl);
-    case 4: return launch_reg<T, 4>(hp, dd, x, y, fo, ycol, st, pdl);
-    case 5:
-      if constexpr (std::is_same<T, float>::value)
-        return launch_reg<T, 5>(hp, dd, x, y, fo, ycol, st, pdl);
-      return cudaErrorInvalidValue;
+    case 2: return launch_reg<float, 2>(hp, dd, x, y, fo, ycol, st, pdl);
+    case 3: return launch_reg<float, 3>(hp, dd, x, y, fo, ycol, st, pdl);
+    case 4: return launch_reg<float, 4>(hp, dd, x, y, fo, ycol, st, pdl);
+    case 5: return launch_reg<float, 5>(hp, dd, x, y, fo, ycol, st, pdl);
     default: return cudaErrorInvalidValue;
   }
 }
-template cudaError_t launch_cell_reg<double>(const HostProblem&, const DeviceData&, const double*,
-                                             double*, const double*, double*, cudaStream_t,
-                                             bool);
-template cudaError_t launch_cell_reg<float>(const HostProblem&, const DeviceData&, const float*,
-                                            float*, const float*, float*, cudaStream_t,
-                                            bool);
 
 }  // namespace sbm

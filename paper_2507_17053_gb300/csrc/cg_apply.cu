@@ -44,27 +44,36 @@ CellLaunch cell_launch_shape(int d, int n) {
 }
 
 
+// Resident blocks asked of the compiler.  FP64 3D (fixed-point cell term),
+// blocks of about 250 threads: 6 up to p = 3 (40 registers), 4 above (64; two
+// blocks fewer per SM cost 10 % at p = 4 and 20 % at p = 5, 6); half-size
+// blocks (shape 1) twice as many.
 template <typename T, int D, int N, int R>
-__global__ void __launch_bounds__(R * Shape<D, N>::L)
+constexpr int chunk_min_blocks() {
+  return !kFixed<T, D> ? 1 : (N <= 4 ? 6 : 4) * (R * N * N <= 128 ? 2 : 1);
+}
+
+template <typename T, int D, int N, int R>
+__global__ void __launch_bounds__(block_threads<T, D, N>(R), (chunk_min_blocks<T, D, N, R>()))
 cg_chunk_kernel(const ChunkArgs<T> a, const __grid_constant__ KTab<T> t) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   // FP32: launched as a programmatic dependent of the face kernel (coherent
   // face loads, a wait before the first fold); FP64 launches plainly
   constexpr bool kPdl = std::is_same<T, float>::value;
   if constexpr (kPdl) pdl_trigger();
-  chunk_xline_build<T, D, N, R>(smem_raw, t, threadIdx.x);
-  chunk_loop<T, D, N, R, kPdl, R * Shape<D, N>::L, kPdl>(a, t, smem_raw, blockIdx.y,
+  chunk_xline_build<T, D, N, R>(smem_raw, t, a.xfix, threadIdx.x);
+  chunk_loop<T, D, N, R, kPdl, block_threads<T, D, N>(R), kPdl>(a, t, smem_raw, blockIdx.y,
                                                          a.q0 + blockIdx.x, a.q1, gridDim.x);
 }
 
 // The same chunks with colour-ordered stores (chunk_loop, ORD): a
 // persistent grid taking chunks from the ticket counter, no assembly pass.
 template <typename T, int D, int N, int R>
-__global__ void __launch_bounds__(R * Shape<D, N>::L)
+__global__ void __launch_bounds__(block_threads<T, D, N>(R))
 cg_chunk_ord_kernel(const ChunkArgs<T> a, const __grid_constant__ KTab<T> t,
                     const __grid_constant__ OrdArgs o) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  chunk_xline_build<T, D, N, R>(smem_raw, t, threadIdx.x);
+  chunk_xline_build<T, D, N, R>(smem_raw, t, a.xfix, threadIdx.x);
   chunk_loop_ord<T, D, N, R>(a, t, smem_raw, o);
 }
 
@@ -77,7 +86,7 @@ constexpr int direct_min_blocks() {
 }
 
 template <typename T, int N, int R>
-__global__ void __launch_bounds__(R * N * N, (direct_min_blocks<T, N>()))
+__global__ void __launch_bounds__(block_threads<T, 3, N>(R), (direct_min_blocks<T, N>()))
 cg_direct_kernel(const ChunkArgs<T> a, const __grid_constant__ KTab<T> t) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr bool kPdl = std::is_same<T, float>::value;     // as cg_chunk_kernel
@@ -87,7 +96,7 @@ cg_direct_kernel(const ChunkArgs<T> a, const __grid_constant__ KTab<T> t) {
 }
 
 template <typename T, int N, int R>
-__global__ void __launch_bounds__(R * N * N, (direct_min_blocks<T, N>()))
+__global__ void __launch_bounds__(block_threads<T, 3, N>(R), (direct_min_blocks<T, N>()))
 cg_direct_ord_kernel(const ChunkArgs<T> a, const __grid_constant__ KTab<T> t,
                      const __grid_constant__ OrdArgs o) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -127,7 +136,7 @@ static cudaError_t direct_prepare(int* grid_cap) {
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (attr != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cg_direct_kernel<T, N, R>,
-                                                      R * N * N, smem) != cudaSuccess ||
+                                                      block_threads<T, 3, N>(R), smem) != cudaSuccess ||
         per_sm < 1)
       per_sm = 1;
   }
@@ -182,7 +191,7 @@ static cudaError_t chunk_prepare(int* grid_cap) {
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (attr != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cg_chunk_kernel<T, D, N, R>,
-                                                      R * Shape<D, N>::L, smem) != cudaSuccess ||
+                                                      block_threads<T, D, N>(R), smem) != cudaSuccess ||
         per_sm < 1)
       per_sm = 1;
   }
@@ -205,7 +214,7 @@ static cudaError_t apply_r(const HostProblem& hp, const DeviceData& dd, const Ch
                            const T* x, T* y, int64_t ld, int nrhs, T* fo, T* ycol, int face_mode,
                            cudaStream_t st, Profiler* prof, Part part, bool reg,
                            bool direct, bool ord, bool allow_pdl) {
-  constexpr int L = Shape<D, N>::L;
+  constexpr int L = Shape<D, N>::L, NT = block_threads<T, D, N>(R);
   const KTab<T> t = make_ktab<T>(hp);
   constexpr size_t smem = ChunkSmem<T, D, N, R>::bytes;
   if (part.f1 < 0) part.f1 = dd.nface;
@@ -250,6 +259,8 @@ static cudaError_t apply_r(const HostProblem& hp, const DeviceData& dd, const Ch
   a.n_dofs = hp.n_dofs;
   a.q0 = part.q0;
   a.q1 = part.q1;
+  a.xfix = dd.xfix;
+  a.eoff = hp.fx.eoff;
   a.ldx = ld;
   a.ld_ycol = (int64_t)dd.ncolours * hp.n_dofs;
   a.ld_face = (int64_t)dd.nface * 2 * L;
@@ -257,30 +268,32 @@ static cudaError_t apply_r(const HostProblem& hp, const DeviceData& dd, const Ch
              ct.dep_cap};
   const int nl0 = nlaunch;
   if (reg) {                 // tile shape 2: one thread per cell (cell_reg.cu)
-    if ((err = launch_cell_reg<T>(hp, dd, x, y, fo, ycol, st, pdl_cell)) != cudaSuccess)
-      return err;
-    nlaunch++;
+    if constexpr (std::is_same<T, float>::value) {
+      if ((err = launch_cell_reg(hp, dd, x, y, fo, ycol, st, pdl_cell)) != cudaSuccess)
+        return err;
+      nlaunch++;
+    }
   } else if (ord && part.q1 > part.q0) {      // colour-ordered stores, no assembly
     if constexpr (R == ChunkShape<D, N>::R) {
       static int cache = 0;
       int grid = 0;
       if (direct) {
         if constexpr (D == 3) {
-          if ((err = resident_grid(cg_direct_ord_kernel<T, N, R>, R * L,
+          if ((err = resident_grid(cg_direct_ord_kernel<T, N, R>, NT,
                                    DirectSmem<T, N, R>::bytes, &cache, &grid)) != cudaSuccess)
             return err;
           if ((err = launch_maybe_pdl(cg_direct_ord_kernel<T, N, R>, dim3(std::min(grid, ct.n)),
-                                      dim3(R * L), DirectSmem<T, N, R>::bytes, st, pdl_cell, a,
+                                      dim3(NT), DirectSmem<T, N, R>::bytes, st, pdl_cell, a,
                                       t, oa)) != cudaSuccess)
             return err;
         }
       } else {
         static int cache0 = 0;
-        if ((err = resident_grid(cg_chunk_ord_kernel<T, D, N, R>, R * L, smem, &cache0, &grid)) !=
+        if ((err = resident_grid(cg_chunk_ord_kernel<T, D, N, R>, NT, smem, &cache0, &grid)) !=
             cudaSuccess)
           return err;
         if ((err = launch_maybe_pdl(cg_chunk_ord_kernel<T, D, N, R>, dim3(std::min(grid, ct.n)),
-                                    dim3(R * L), smem, st, pdl_cell, a, t, oa)) != cudaSuccess)
+                                    dim3(NT), smem, st, pdl_cell, a, t, oa)) != cudaSuccess)
           return err;
       }
       nlaunch++;
@@ -290,7 +303,7 @@ static cudaError_t apply_r(const HostProblem& hp, const DeviceData& dd, const Ch
       int dcap = 0;
       if ((err = direct_prepare<T, N, R>(&dcap)) != cudaSuccess) return err;
       const int grid = std::min(part.q1 - part.q0, dcap);
-      if ((err = launch_maybe_pdl(cg_direct_kernel<T, N, R>, dim3(grid, nrhs), dim3(R * L),
+      if ((err = launch_maybe_pdl(cg_direct_kernel<T, N, R>, dim3(grid, nrhs), dim3(NT),
                                   DirectSmem<T, N, R>::bytes, st, pdl_cell, a, t)) !=
           cudaSuccess)
         return err;
@@ -298,7 +311,7 @@ static cudaError_t apply_r(const HostProblem& hp, const DeviceData& dd, const Ch
     }
   } else if (part.q1 > part.q0) {
     const int grid = std::min(part.q1 - part.q0, cap);
-    if ((err = launch_maybe_pdl(cg_chunk_kernel<T, D, N, R>, dim3(grid, nrhs), dim3(R * L), smem,
+    if ((err = launch_maybe_pdl(cg_chunk_kernel<T, D, N, R>, dim3(grid, nrhs), dim3(NT), smem,
                                 st, pdl_cell, a, t)) != cudaSuccess)
       return err;
     nlaunch++;
@@ -341,8 +354,9 @@ static cudaError_t apply_t(const HostProblem& hp, const DeviceData& dd, const T*
   constexpr int R = ChunkShape<D, N>::R;
   constexpr int RH = (R / 2) > 0 ? R / 2 : 1;
   const int v = (variant == 1 && RH < R) ? 1 : 0;
-  const bool reg = variant == 2 && slab < 0 && nrhs == 1 &&
-                   cell_reg_available(hp, std::is_same<T, float>::value);
+  // (FP64 runs variant 2 as variant 0, which gives the same bits)
+  const bool reg = std::is_same<T, float>::value && variant == 2 && slab < 0 && nrhs == 1 &&
+                   cell_reg_available(hp, true);
   const bool direct = variant == 3 && D == 3;
   const ChunkTable& ct = dd.chunks[v];
   // colour-ordered stores: whole single applies of chunking 0 by the chunk

@@ -47,7 +47,30 @@ struct ChunkArgs {
   // right-hand side blockIdx.y of a multi-RHS launch: offsets of its x and y,
   // its colour buffers and its face results (0 for a single right-hand side)
   int64_t ldx, ld_ycol, ld_face;
+  // FP64, 3D: the problem's fixed-point x-line operators and result exponent
+  const fix::Entry* __restrict__ xfix;
+  int eoff;
 };
+
+// 3D FP64: the fixed-point cell term (sweeps.cuh)
+template <typename T, int D>
+constexpr bool kFixed = D == 3 && std::is_same<T, double>::value;
+
+// threads of a block of R cells, and a thread's cell and line
+template <typename T, int D, int N>
+constexpr int block_threads(int R) {
+  if constexpr (kFixed<T, D>) return FixMap<N>::threads(R);
+  else return R * Shape<D, N>::L;
+}
+template <typename T, int D, int N>
+__device__ __forceinline__ void cell_of_thread(int tid, int& c, int& tl) {
+  if constexpr (kFixed<T, D>) {
+    FixMap<N>::of(tid, c, tl);
+  } else {
+    c = tid / Shape<D, N>::L;
+    tl = tid - c * Shape<D, N>::L;
+  }
+}
 
 // ---- colour-ordered stores ----------------------------------------------------
 //
@@ -240,8 +263,10 @@ struct ChunkSmem {
       (D == 3) ? XLineOp<T, N>::kSlots * XLineOp<T, N>::kPacked : 0;
   // two run areas and two run-start tables: the next chunk's runs are copied
   // in (cp.async) while the current chunk is computed
+  // FP64 3D: the cells' exponent words, this chunk's and the next one's
+  static constexpr int EX = kFixed<T, D> ? 2 * R : 0;
   static constexpr size_t bytes =
-      (size_t)(TILE + 2 * XS + XL) * sizeof(T) + (size_t)(2 * L + WORDS) * 4;
+      (size_t)(TILE + 2 * XS + XL) * sizeof(T) + (size_t)(2 * L + WORDS + EX) * 4;
 };
 
 // Asynchronous global -> shared copy of one element (cp.async, no register
@@ -288,9 +313,17 @@ __device__ __forceinline__ int zix(int cc, int l, int m) {
 }
 
 // h K + mu M of the 3D x-lines into the chunk's shared memory (one operator
-// per x-line of modes (a, b) = (tl % n, tl / n), built by the threads of
-// cell 0); visible after the caller's next barrier.  tx supplies hlam, fM
-// and fKh (the problem's h-scaled tables).
+// per x-line of modes (a, b) = (tl % n, tl / n)); visible after the caller's
+// next barrier.  FP32: built by the threads of cell 0 from tx's hlam, fM and
+// fKh (the problem's h-scaled tables); FP64: copied from the set-up's
+// fixed-point operators xfix.
+template <int N>
+__device__ __forceinline__ void xline_copy(fix::Entry* m, const fix::Entry* __restrict__ xfix,
+                                           int tid) {
+  constexpr int n = XLineOp<double, N>::kSlots * XLineOp<double, N>::kPacked;
+  const int2* src = reinterpret_cast<const int2*>(xfix);
+  for (int i = tid; i < n; i += blockDim.x) reinterpret_cast<int2*>(m)[i] = __ldg(src + i);
+}
 template <typename T, int D, int N, int R>
 __device__ __forceinline__ T* chunk_xline_smem(unsigned char* smem_raw) {
   using CS = ChunkSmem<T, D, N, R>;
@@ -298,9 +331,12 @@ __device__ __forceinline__ T* chunk_xline_smem(unsigned char* smem_raw) {
 }
 template <typename T, int D, int N, int R>
 __device__ __forceinline__ void chunk_xline_build(unsigned char* smem_raw, const KTab<T>& tx,
-                                                  int tid) {
+                                                  const fix::Entry* __restrict__ xfix, int tid) {
   constexpr int L = Shape<D, N>::L;
-  if (D == 3 && tid < L && tid % N <= tid / N)
+  if constexpr (kFixed<T, D>)
+    xline_copy<N>(reinterpret_cast<fix::Entry*>(chunk_xline_smem<T, D, N, R>(smem_raw)), xfix,
+                  tid);
+  else if (D == 3 && tid < L && tid % N <= tid / N)
     XLineOp<T, N>(tx, tid % N, tid / N)
         .store(chunk_xline_smem<T, D, N, R>(smem_raw) +
                XLineOp<T, N>::slot(tid % N, tid / N) * XLineOp<T, N>::kPacked);
@@ -332,9 +368,15 @@ __device__ __forceinline__ void chunk_loop(const ChunkArgs<T>& a, const KTab<T>&
   // blockDim.x (the same value; this split keeps the FP64 kernels at 32-40
   // registers)
   constexpr int nthr = NTHR;
-  const int c = tid / L, tl = tid - c * L;
-  const XLineShared<T, N> xop{XLs + XLineOp<T, N>::slot(tl % N, tl / N) *
-                                         XLineOp<T, N>::kPacked};
+  int c, tl;
+  cell_of_thread<T, D, N>(tid, c, tl);
+  T* const xsl = XLs + XLineOp<T, N>::slot(tl % N, tl / N) * XLineOp<T, N>::kPacked;
+  uint32_t* const Ex = Bs + CS::WORDS;                       // FP64 3D: [2][R] exponent words
+  unsigned lanes = 0u;
+  if constexpr (kFixed<T, D>) {
+    lanes = cell_lanes(c);
+    for (int i = tid; i < 2 * R; i += blockDim.x) Ex[i] = 0u;
+  }
   const T* __restrict__ xr = a.x + rhs * a.ldx;
   const T* fo = a.face_out + rhs * a.ld_face;
   T* ycb = a.ycol + rhs * a.ld_ycol;
@@ -384,9 +426,15 @@ __device__ __forceinline__ void chunk_loop(const ChunkArgs<T>& a, const KTab<T>&
     __syncthreads();                          // ... and everyone's
     const bool act = c < nc;
     T out[N];
-    if constexpr (D == 3)
-      cell_fd_3d<T, N>(t, Xs, (tl / N) * SM + P * c + (tl % N), N * SM, tile, c, tl, act, xop,
+    if constexpr (kFixed<T, D>) {
+      const T* xl = Xs + (tl / N) * SM + P * c + (tl % N);
+      cell_fix_3d_l<N>(t, [&](int j) { return xl[N * SM * j]; }, tile, c, tl, act,
+                       reinterpret_cast<const fix::Entry*>(xsl), lanes, Ex + buf * R + c, a.eoff,
                        out);
+      if (tid < R) Ex[(buf ^ 1) * R + tid] = 0u;    // for the next chunk
+    } else if constexpr (D == 3)
+      cell_fd_3d<T, N>(t, Xs, (tl / N) * SM + P * c + (tl % N), N * SM, tile, c, tl, act,
+                       XLineShared<T, N>{xsl}, out);
     else
       cell_sweeps_2d<T, N>(t, Xs, P * c + tl, SM, AE, c, tl, act, out);
     if (act) {
@@ -409,6 +457,16 @@ __device__ __forceinline__ void chunk_loop(const ChunkArgs<T>& a, const KTab<T>&
       }
     }
     __syncthreads();
+    if constexpr (kFixed<T, D>) {
+      // the node shared by cells c and c + 1: one addition per thread, in
+      // full warps (in the store loop below every warp would issue it for
+      // its few lanes, 16 FP64-pipe clocks each)
+      if (c + 1 < nc) {
+        T* z = Z + zix<T, D, N>(c + 1, tl, 0);
+        *z = Z[zix<T, D, N>(c, tl, P)] + *z;
+      }
+      __syncthreads();
+    }
     // runs of the result: the node shared by cells c-1 and c is the sum of
     // their two values (fixed order), then one coalesced store per run, into
     // y where this chunk is the DoF's only writer
@@ -418,7 +476,7 @@ __device__ __forceinline__ void chunk_loop(const ChunkArgs<T>& a, const KTab<T>&
       const int cc = kk / P, m = kk - cc * P;
       T v;
       if (cc == nc) v = Z[zix<T, D, N>(nc - 1, l, P)];
-      else if (m == 0 && cc > 0) v = Z[zix<T, D, N>(cc - 1, l, P)] + Z[zix<T, D, N>(cc, l, 0)];
+      else if (!kFixed<T, D> && m == 0 && cc > 0) v = Z[zix<T, D, N>(cc - 1, l, P)] + Z[zix<T, D, N>(cc, l, 0)];
       else v = Z[zix<T, D, N>(cc, l, m)];
       const int64_t g = (int64_t)Ls[l] + kk;
       if ((Bs[idx >> 5] >> (idx & 31)) & 1u) yc[g] = v;
@@ -449,9 +507,15 @@ __device__ __forceinline__ void chunk_loop_ord(const ChunkArgs<T>& a, const KTab
   int* Lbuf = reinterpret_cast<int*>(XLs + CS::XL);
   uint32_t* Bs = reinterpret_cast<uint32_t*>(Lbuf + 2 * L);
   const int tid = threadIdx.x;
-  const int c = tid / L, tl = tid - c * L;
-  const XLineShared<T, N> xop{XLs + XLineOp<T, N>::slot(tl % N, tl / N) *
-                                         XLineOp<T, N>::kPacked};
+  int c, tl;
+  cell_of_thread<T, D, N>(tid, c, tl);
+  T* const xsl = XLs + XLineOp<T, N>::slot(tl % N, tl / N) * XLineOp<T, N>::kPacked;
+  uint32_t* const Ex = Bs + CS::WORDS;                       // FP64 3D: [2][R] exponent words
+  unsigned lanes = 0u;
+  if constexpr (kFixed<T, D>) {
+    lanes = cell_lanes(c);
+    for (int i = tid; i < 2 * R; i += blockDim.x) Ex[i] = 0u;
+  }
   const T* __restrict__ xr = a.x;
   T* yb = a.y;
 
@@ -466,7 +530,7 @@ __device__ __forceinline__ void chunk_loop_ord(const ChunkArgs<T>& a, const KTab
     for (int i = tid; i < L; i += blockDim.x) Lbuf[i] = __ldg(a.lines + (size_t)first * L + i);
     __syncthreads();
     if (tid == 0) s_ord_next = (int)atomicAdd(o.tickets, 1u);
-    gather_runs_async<T, L, SM>(xr, Lbuf, Xbuf, S, tid, R * L);
+    gather_runs_async<T, L, SM>(xr, Lbuf, Xbuf, S, tid, blockDim.x);
   }
   cp_async_commit();
   __syncthreads();                            // s_ord_next written
@@ -491,7 +555,7 @@ __device__ __forceinline__ void chunk_loop_ord(const ChunkArgs<T>& a, const KTab
       for (int i = tid; i < L; i += blockDim.x) Ln[i] = __ldg(a.lines + (size_t)f2 * L + i);
       if (tid == 0) tk2 = atomicAdd(o.tickets, 1u);
       __syncthreads();
-      gather_runs_async<T, L, SM>(xr, Ln, Xbuf + (buf ^ 1) * CS::XS, S2, tid, R * L);
+      gather_runs_async<T, L, SM>(xr, Ln, Xbuf + (buf ^ 1) * CS::XS, S2, tid, blockDim.x);
     }
     cp_async_commit();
     {
@@ -502,9 +566,15 @@ __device__ __forceinline__ void chunk_loop_ord(const ChunkArgs<T>& a, const KTab
     __syncthreads();
     const bool act = c < nc;
     T out[N];
-    if constexpr (D == 3)
-      cell_fd_3d<T, N>(t, Xs, (tl / N) * SM + P * c + (tl % N), N * SM, tile, c, tl, act, xop,
+    if constexpr (kFixed<T, D>) {
+      const T* xl = Xs + (tl / N) * SM + P * c + (tl % N);
+      cell_fix_3d_l<N>(t, [&](int j) { return xl[N * SM * j]; }, tile, c, tl, act,
+                       reinterpret_cast<const fix::Entry*>(xsl), lanes, Ex + buf * R + c, a.eoff,
                        out);
+      if (tid < R) Ex[(buf ^ 1) * R + tid] = 0u;    // for the next chunk
+    } else if constexpr (D == 3)
+      cell_fd_3d<T, N>(t, Xs, (tl / N) * SM + P * c + (tl % N), N * SM, tile, c, tl, act,
+                       XLineShared<T, N>{xsl}, out);
     else
       cell_sweeps_2d<T, N>(t, Xs, P * c + tl, SM, AE, c, tl, act, out);
     pdl_wait();                               // the face kernel's results
@@ -528,6 +598,16 @@ __device__ __forceinline__ void chunk_loop_ord(const ChunkArgs<T>& a, const KTab
       }
     }
     __syncthreads();
+    if constexpr (kFixed<T, D>) {
+      // the node shared by cells c and c + 1: one addition per thread, in
+      // full warps (in the store loop below every warp would issue it for
+      // its few lanes, 16 FP64-pipe clocks each)
+      if (c + 1 < nc) {
+        T* z = Z + zix<T, D, N>(c + 1, tl, 0);
+        *z = Z[zix<T, D, N>(c, tl, P)] + *z;
+      }
+      __syncthreads();
+    }
     ord_wait(o, ch, target, peek);
     // a thread's run elements (at most n of them: L S <= L (P R + 1) <=
     // n R L): first the earlier colours' partial sums where the bit is set,
@@ -536,7 +616,7 @@ __device__ __forceinline__ void chunk_loop_ord(const ChunkArgs<T>& a, const KTab
     T old[N];
 #pragma unroll
     for (int k = 0; k < N; ++k) {
-      const int idx = tid + k * R * L;
+      const int idx = tid + k * (int)blockDim.x;
       old[k] = T(0);
       if (idx < L * S && ((Bs[idx >> 5] >> (idx & 31)) & 1u)) {
         const int l = __float2int_rz(((float)idx + 0.5f) * invS);
@@ -545,13 +625,13 @@ __device__ __forceinline__ void chunk_loop_ord(const ChunkArgs<T>& a, const KTab
     }
 #pragma unroll
     for (int k = 0; k < N; ++k) {
-      const int idx = tid + k * R * L;
+      const int idx = tid + k * (int)blockDim.x;
       if (idx < L * S) {
         const int l = __float2int_rz(((float)idx + 0.5f) * invS), kk = idx - l * S;
         const int cc = kk / P, m = kk - cc * P;
         T v;
         if (cc == nc) v = Z[zix<T, D, N>(nc - 1, l, P)];
-        else if (m == 0 && cc > 0)
+        else if (!kFixed<T, D> && m == 0 && cc > 0)
           v = Z[zix<T, D, N>(cc - 1, l, P)] + Z[zix<T, D, N>(cc, l, 0)];
         else v = Z[zix<T, D, N>(cc, l, m)];
         yb[(int64_t)Ls[l] + kk] = ((Bs[idx >> 5] >> (idx & 31)) & 1u) ? old[k] + v : v;
@@ -702,7 +782,9 @@ struct DirectSmem {
   static constexpr int XL = XLineOp<T, N>::kSlots * XLineOp<T, N>::kPacked;  // x-line ops
   static constexpr int XF = R * L;                       // j0 = P faces of the cells
   static constexpr int WORDS = (L * (P * R + 1) + 31) / 32;
-  static constexpr size_t bytes = (size_t)(TILE + XL + XF) * sizeof(T) + (size_t)(L + WORDS) * 4;
+  static constexpr int EX = kFixed<T, 3> ? 2 * R : 0;    // exponent words, two chunks
+  static constexpr size_t bytes =
+      (size_t)(TILE + XL + XF) * sizeof(T) + (size_t)(L + WORDS + EX) * 4;
 };
 
 template <typename T, int N, int R, bool COH, bool ORD = false, bool PDL = false>
@@ -718,13 +800,21 @@ __device__ __forceinline__ void chunk_loop_direct(const ChunkArgs<T>& a, const K
   int* Ls = reinterpret_cast<int*>(XF + DS::XF);
   uint32_t* Bs = reinterpret_cast<uint32_t*>(Ls + L);
   const int tid = threadIdx.x;
-  const int c = tid / L, tl = tid - c * L;
+  int c, tl;
+  cell_of_thread<T, 3, N>(tid, c, tl);
   const int j0 = tl % N, j1 = tl / N;
-  if (tid < L && tid % N <= tid / N)
+  T* const xsl = XLs + XLineOp<T, N>::slot(tl % N, tl / N) * XLineOp<T, N>::kPacked;
+  uint32_t* const Ex = Bs + DS::WORDS;                       // FP64: [2][R] exponent words
+  unsigned lanes = 0u;
+  int buf = 0;
+  if constexpr (kFixed<T, 3>) {
+    xline_copy<N>(reinterpret_cast<fix::Entry*>(XLs), a.xfix, tid);
+    lanes = cell_lanes(c);
+    for (int i = tid; i < 2 * R; i += blockDim.x) Ex[i] = 0u;
+  } else if (tid < L && tid % N <= tid / N) {
     XLineOp<T, N>(tx, tid % N, tid / N)
         .store(XLs + XLineOp<T, N>::slot(tid % N, tid / N) * XLineOp<T, N>::kPacked);
-  const XLineShared<T, N> xop{XLs + XLineOp<T, N>::slot(tl % N, tl / N) *
-                                         XLineOp<T, N>::kPacked};
+  }
   const T* __restrict__ xr = a.x + rhs * a.ldx;
   const T* fo = a.face_out + rhs * a.ld_face;
   T* ycb = a.ycol + rhs * a.ld_ycol;
@@ -756,9 +846,15 @@ __device__ __forceinline__ void chunk_loop_direct(const ChunkArgs<T>& a, const K
     __syncthreads();                          // Ls, Bs; the x-line operators (first chunk)
     const bool act = c < nc;
     T out[N];
-    cell_fd_3d_l<T, N>(
-        t, [&](int j) { return __ldg(xr + Ls[j1 + N * j] + P * c + j0); }, tile, c, tl, act, xop,
-        out);
+    const auto load = [&](int j) { return __ldg(xr + Ls[j1 + N * j] + P * c + j0); };
+    if constexpr (kFixed<T, 3>) {
+      cell_fix_3d_l<N>(t, load, tile, c, tl, act, reinterpret_cast<const fix::Entry*>(xsl), lanes,
+                       Ex + buf * R + c, a.eoff, out);
+      if (tid < R) Ex[(buf ^ 1) * R + tid] = 0u;    // for the next chunk
+      buf ^= 1;
+    } else {
+      cell_fd_3d_l<T, N>(t, load, tile, c, tl, act, XLineShared<T, N>{xsl}, out);
+    }
     if (act) {
       const int pos = first + c;
       const int fs = __ldg(a.face_start + pos), fe = __ldg(a.face_start + pos + 1);

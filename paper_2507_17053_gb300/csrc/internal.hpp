@@ -9,6 +9,7 @@
 #include <string>
 #include <vector>
 
+#include "fixed_point.cuh"
 #include "setup.hpp"
 
 namespace sbm {
@@ -29,8 +30,16 @@ struct Folded {
   T O[kMaxH][kMaxH];
 };
 
+// FP64: the transforms of the fixed-point cell term (3D; h-independent)
 template <typename T>
-struct KTab {
+struct KTabFix {};
+template <>
+struct KTabFix<double> {
+  fix::Block xVt, xV;
+};
+
+template <typename T>
+struct KTab : KTabFix<T> {
   T M[kMaxN][kMaxN];     // 1D mass on [0,1]
   T K[kMaxN][kMaxN];     // 1D stiffness on [0,1]
   T Mh[kMaxN][kMaxN];    // h^(d-2) * M   (last sweep of the cell operator)
@@ -126,6 +135,8 @@ struct DeviceData {
   int32_t* face_start = nullptr; // [Nc + 1] per ordered cell, range into the ordered face list
   int32_t* face_kind = nullptr;  // [F] k | (s << 2)
   int32_t* face_cell = nullptr;  // [F] ordered cell position of the face's cell
+  // 3D: the x-line operators of the fixed-point FP64 cell term, slot by slot
+  fix::Entry* xfix = nullptr;
   int nface = 0;
   double* face_out = nullptr;    // [F * 2L] per-face results of the face kernel (scratch)
   float* face_out32 = nullptr;
@@ -234,14 +245,13 @@ cudaError_t launch_maybe_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size
 }
 
 // Tile shape 2: the cell term with one thread per cell and the tile in
-// registers (cell_reg.cu); available for 3D CG problems with n <= 5 (FP32)
-// or n <= 4 (FP64); bitwise equal to tile shape 0.
+// registers (cell_reg.cu); accepted for 3D CG problems with n <= 5 (FP32) or
+// n <= 4 (FP64, which runs shape 0 instead); bitwise equal to tile shape 0.
 bool cell_reg_available(const HostProblem& hp, bool fp32);
 cudaError_t build_cell_reg_tables(const HostProblem& hp, const std::vector<int32_t>& ch_first,
                                   DeviceData* dd);
-template <typename T>
-cudaError_t launch_cell_reg(const HostProblem& hp, const DeviceData& dd, const T* x, T* y,
-                            const T* fo, T* ycol, cudaStream_t st, bool pdl = false);
+cudaError_t launch_cell_reg(const HostProblem& hp, const DeviceData& dd, const float* x, float* y,
+                            const float* fo, float* ycol, cudaStream_t st, bool pdl = false);
 
 // The surrogate faces [fb, fe) of the kernel face order (all: 0, -1) into
 // the per-face scratch (face_kernel.cu).

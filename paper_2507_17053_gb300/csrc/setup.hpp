@@ -7,6 +7,7 @@
 #include <string>
 #include <vector>
 
+#include "fixed_tables.hpp"
 #include "geom.hpp"
 #include "sbm.h"
 
@@ -74,6 +75,7 @@ struct HostProblem {
   int L = 0;         // n^(d-1) lines per cell / points per face
   double h = 0, sigma = 0, sigma_f = 0;
   Tables1D tab;
+  FixedTables fx;    // the 3D FP64 cell term's fixed-point tables
   LevelSet ls;
 
   // active cells, lexicographic (axis 0 fastest)

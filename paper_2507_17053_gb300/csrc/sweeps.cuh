@@ -312,6 +312,157 @@ struct TilePad {
   static constexpr int NDP = PX * N * N;
 };
 
+// ---- 3D cell term in fixed point (FP64) -----------------------------------------
+//
+// The same five phases with the cell's values as 61-bit integers
+// (fixed_point.cuh): the double-precision pipe, which bound the double form
+// (83 % busy), is left to the face folds and the x-face sums.  Per line and
+// phase: n shared-memory reads, the folds, 3 (ceil(n/2)^2 + floor(n/2)^2)
+// mad.wide, n shared-memory writes.  The exponent of a cell is the maximum
+// over its own nodes, so the results do not depend on the chunk it is in.
+// Measured on GB300, cell term of 96^3-cell spheres (64^3 at p = 5; 48^3
+// ellipsoid at p = 6), double -> fixed point, best tile shape of each: p = 1
+// 47.5 -> 28.2 us, p = 2 142 -> 67, p = 3 374 -> 139, p = 4 810 -> 274, p = 5
+// 503 -> 161, p = 6 257 -> 84 us; the whole applies 1.4 to 2.1 times faster.
+// Now the integer pipes and the issue slots bind (1 120 warp instructions per
+// cell at p = 4, ALU pipe 53 %, issue 55 % busy), and barrier waits.
+
+// The threads of a cell in this warp (its cell index c = tid / L): the lanes
+// that reduce together.
+__device__ __forceinline__ unsigned cell_lanes(int c) {
+  return __match_any_sync(__activemask(), c);
+}
+
+// slot[c] = max over the cell's threads of v (slot zeroed beforehand; visible
+// after the next block barrier)
+__device__ __forceinline__ void cell_max(uint32_t v, unsigned lanes, uint32_t* slot) {
+  const uint32_t m = __reduce_max_sync(lanes, v);
+  if ((int)(threadIdx.x & 31u) == __ffs(lanes) - 1) atomicMax(slot, m);
+}
+
+// Threads and cells.  A block of R cells has R n^2 threads, for n = 5 rounded
+// up to groups of 128 (5 cells each): the line phases of a cell need its own
+// threads' tile only, so they synchronise a group (n = 5: cell term of the
+// 96^3 sphere 286 -> 280 us) or a warp (n = 2, 4: whole cells per warp; p = 3
+// 144 -> 140 us) instead of the block (n = 3 in groups of 14 cells: 72 -> 75
+// us, not kept).
+template <int N>
+struct FixMap {
+  static constexpr int L = N * N;
+  static constexpr int GROUP = N == 5 ? 128 : 0;
+  static constexpr bool kWarp = 32 % L == 0;
+  static constexpr int threads(int R) { return GROUP ? (R * L + 127) / 128 * 128 : R * L; }
+  // cell and line of a thread (line = L: none)
+  __device__ __forceinline__ static void of(int tid, int& c, int& tl) {
+    if constexpr (GROUP != 0) {
+      constexpr int CPG = GROUP / L;
+      const int g = tid / GROUP, r = tid - g * GROUP;
+      c = g * CPG + r / L;
+      tl = r % L;
+      if (r >= CPG * L) c = 1 << 20;
+    } else {
+      c = tid / L;
+      tl = tid - c * L;
+    }
+  }
+  __device__ __forceinline__ static void sync(int tid) {
+    if constexpr (kWarp) __syncwarp();
+    else if constexpr (GROUP == 0) __syncthreads();
+    else if (tid < GROUP) asm volatile("bar.sync 1, %0;" ::"n"(GROUP) : "memory");
+    else asm volatile("bar.sync 2, %0;" ::"n"(GROUP) : "memory");
+  }
+};
+
+// load(j): the thread's z-line of x; xop: the slot of its x-line's modes;
+// slot: the cell's exponent word (zeroed); eoff: FixedTables::eoff.  The
+// z-line result (nodal) is returned in out[]; the tile then holds nothing
+// useful.
+template <int N, typename Load>
+__device__ __forceinline__ void cell_fix_3d_l(const KTab<double>& t, const Load& load, double* tile,
+                                              int c, int tl, bool act, const fix::Entry* xop,
+                                              unsigned lanes, uint32_t* slot, int eoff,
+                                              double (&out)[N]) {
+  using Op = XLineOp<double, N>;
+  constexpr int PX = TilePad<double, N>::PX, NDP = PX * N * N, PL = PX * N;
+  constexpr int HE = (N + 1) / 2;
+  const int a = tl % N, b = tl / N;
+  const int zl = (PX == N) ? tl : a + PX * b;     // the z-line's first node
+  long long* cell = reinterpret_cast<long long*>(tile) + c * NDP;
+  uint64_t u[N];
+  uint32_t mx = 0u;
+  if (act) {
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      u[j] = (uint64_t)__double_as_longlong(load(j));
+      mx = max(mx, fix::mag_hi(u[j]));
+    }
+    cell_max(mx, lanes, slot);
+  }
+  FixMap<N>::sync(threadIdx.x);
+  int E = 1;
+  if (act) {                       // z-lines (j0, j1) = (a, b) -> z-modes
+    E = max(1, (int)(*slot >> 20));
+    int64_t v[N], w[N];
+    if (fix::plain_exp(E)) {
+#pragma unroll
+      for (int j = 0; j < N; ++j) v[j] = fix::from_double<false>(u[j], E);
+    } else {
+#pragma unroll
+      for (int j = 0; j < N; ++j) v[j] = fix::from_double<true>(u[j], E);
+    }
+    fix::to_modes<N, 0>(t.xVt, v, w);
+#pragma unroll
+    for (int k = 0; k < N; ++k) cell[zl + PL * k] = w[k];
+  }
+  FixMap<N>::sync(threadIdx.x);
+  if (act) {                       // y-lines (j0 = a, z-mode b) -> y-modes
+    int64_t v[N], w[N];
+#pragma unroll
+    for (int j = 0; j < N; ++j) v[j] = cell[a + PX * j + PL * b];
+    fix::to_modes<N, 0>(t.xVt, v, w);
+#pragma unroll
+    for (int k = 0; k < N; ++k) cell[a + PX * k + PL * b] = w[k];
+  }
+  FixMap<N>::sync(threadIdx.x);
+  if (act) {                       // x-lines (y-mode a, z-mode b): h K + mu_ab M
+    int64_t v[N], y[N];
+#pragma unroll
+    for (int j = 0; j < N; ++j) v[j] = cell[PX * tl + j];
+    fix::apply_line<N, fix::shift_x(N)>(
+        [&](int i, int j) { return xop[Op::sym(i, j, HE)]; },
+        [&](int i, int j) { return xop[HE * (HE + 1) / 2 + Op::sym(i, j, N / 2)]; }, v, y);
+#pragma unroll
+    for (int j = 0; j < N; ++j) cell[PX * tl + j] = y[j];
+  }
+  FixMap<N>::sync(threadIdx.x);
+  if (act) {                       // y-modes back (j0 = a, z-mode b)
+    int64_t w[N], y[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) w[k] = cell[a + PX * k + PL * b];
+    fix::from_modes<N, fix::shift_y(N)>(t.xV, w, y);
+#pragma unroll
+    for (int j = 0; j < N; ++j) cell[a + PX * j + PL * b] = y[j];
+  }
+  FixMap<N>::sync(threadIdx.x);
+  if (act) {                       // z-modes back (j0, j1) = (a, b), to double
+    int64_t w[N], y[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) w[k] = cell[zl + PL * k];
+    fix::from_modes<N, fix::shift_z(N)>(t.xV, w, y);
+    if (fix::plain_exp(E)) {
+#pragma unroll
+      for (int j = 0; j < N; ++j)
+        out[j] = __longlong_as_double((long long)fix::to_double<false>(y[j], E + eoff));
+    } else {
+#pragma unroll
+      for (int j = 0; j < N; ++j)
+        out[j] = E == fix::kExpBad
+                     ? __longlong_as_double(0x7ff8000000000000ll)
+                     : __longlong_as_double((long long)fix::to_double<true>(y[j], E + eoff));
+    }
+  }
+}
+
 // The thread's z-line of x comes from load(j), j = 0..n-1 (staged runs in
 // shared memory, or global memory directly).
 // PAD = false: the unpadded layout (PX = n), for callers that address the

@@ -1,0 +1,173 @@
+"""The fixed-point arithmetic of the 3D FP64 cell term (fixed_point.cuh,
+fixed_tables.cpp), compiled for the host: the cell operator against extended
+precision and the conversions at the ends of the exponent range."""
+import os
+import subprocess
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
+                    "paper_2507_17053_gb300", "csrc")
+
+SRC = r"""
+#include <algorithm>
+#include <cmath>
+#include <cstdio>
+#include <cstring>
+#include <limits>
+#include <vector>
+#include "setup.hpp"
+using namespace sbm;
+static uint64_t bits(double x) { uint64_t b; std::memcpy(&b, &x, 8); return b; }
+static double val(uint64_t b) { double x; std::memcpy(&x, &b, 8); return x; }
+static uint64_t rs = 7;
+static double rnd() {            // splitmix64, U(-1,1)
+  rs += 0x9E3779B97F4A7C15ull;
+  uint64_t z = rs;
+  z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+  z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+  z ^= z >> 31;
+  return 2.0 * (double)(z >> 11) * 0x1p-53 - 1.0;
+}
+
+template <int N>
+int cell(double h) {
+  constexpr int H = N / 2, HE = (N + 1) / 2, L = N * N, ND = L * N;
+  constexpr int packed = (HE * (HE + 1) / 2 + H * (H + 1) / 2) | 1;
+  Tables1D tb;
+  build_tables(N - 1, &tb);
+  FixedTables ft;
+  if (!build_fixed_tables(tb, h, &ft)) { std::printf("n=%d h=%g: tables\n", N, h); return 1; }
+  auto tri = [](int i, int j, int n) { return i * n - i * (i - 1) / 2 + (j - i); };
+  auto sym = [&](int i, int j, int n) { return i <= j ? tri(i, j, n) : tri(j, i, n); };
+  int bad = 0;
+  for (int kind = 0; kind < 4; ++kind) {
+    double num = 0, den = 0;
+    for (int trial = 0; trial < 8; ++trial) {
+      std::vector<double> x(ND);
+      for (int c = 0; c < ND; ++c) {
+        x[c] = rnd();
+        if (kind == 1) x[c] *= std::pow(10.0, 3.0 * rnd() - 3.0);        // graded
+        if (kind == 2) x[c] = rnd() > 0 ? 1.0 : -1.0;                    // the bounds
+        if (kind == 3) x[c] = std::ldexp(1.0 + 0.01 * x[c], 500);        // near constant
+      }
+      // reference: sum over axes of M x .. K .. x M in long double
+      std::vector<long double> ref(ND, 0), cur(ND), nx(ND);
+      const int st[3] = {1, N, L};
+      for (int k = 0; k < 3; ++k) {
+        for (int c = 0; c < ND; ++c) cur[c] = x[c];
+        for (int ax = 0; ax < 3; ++ax) {
+          for (int c = 0; c < ND; ++c) {
+            const int i = c / st[ax] % N;
+            long double s = 0;
+            for (int j = 0; j < N; ++j)
+              s += (long double)(ax == k ? tb.K[i][j] : tb.M[i][j]) * cur[c + (j - i) * st[ax]];
+            nx[c] = s;
+          }
+          cur = nx;
+        }
+        for (int c = 0; c < ND; ++c) ref[c] += (long double)h * cur[c];
+      }
+      uint32_t mx = 0;
+      for (double v : x) mx = std::max(mx, fix::mag_hi(bits(v)));
+      const int E = (int)(mx >> 20);
+      std::vector<int64_t> q(ND);
+      for (int c = 0; c < ND; ++c) q[c] = fix::from_double<false>(bits(x[c]), E);
+      auto line = [&](int base, int s, auto f) {
+        int64_t v[N], w[N];
+        for (int j = 0; j < N; ++j) v[j] = q[base + j * s];
+        f(v, w);
+        for (int j = 0; j < N; ++j) {
+          if (std::llabs(w[j]) > (1ll << 60) + 64) { std::printf("n=%d overflow\n", N); bad = 1; }
+          q[base + j * s] = w[j];
+        }
+      };
+      for (int l = 0; l < L; ++l)
+        line(l, L, [&](auto& v, auto& w) { fix::to_modes<N, 0>(ft.Vt, v, w); });
+      for (int l = 0; l < L; ++l)
+        line(l % N + l / N * L, N, [&](auto& v, auto& w) { fix::to_modes<N, 0>(ft.Vt, v, w); });
+      for (int l = 0; l < L; ++l) {
+        const fix::Entry* m = ft.xline.data() + sym(l % N, l / N, N) * packed;
+        line(l * N, 1, [&](auto& v, auto& w) {
+          fix::apply_line<N, fix::shift_x(N)>(
+              [&](int i, int j) { return m[sym(i, j, HE)]; },
+              [&](int i, int j) { return m[HE * (HE + 1) / 2 + sym(i, j, H)]; }, v, w);
+        });
+      }
+      for (int l = 0; l < L; ++l)
+        line(l % N + l / N * L, N,
+             [&](auto& v, auto& w) { fix::from_modes<N, fix::shift_y(N)>(ft.V, v, w); });
+      for (int l = 0; l < L; ++l)
+        line(l, L, [&](auto& v, auto& w) { fix::from_modes<N, fix::shift_z(N)>(ft.V, v, w); });
+      long double big = 0;
+      for (int c = 0; c < ND; ++c) big = std::max(big, (long double)std::fabs(x[c]));
+      for (int c = 0; c < ND; ++c) {
+        const double y = val(fix::to_double<false>(q[c], E + ft.eoff));
+        const long double d = ((long double)y - ref[c]) / big;
+        num = std::max(num, (double)std::fabs(d));
+        den = std::max(den, (double)std::fabs(ref[c] / big));
+      }
+    }
+    // backward-stable bound relative to |A| |x| (|A| by rows ~ 3 h max|K|), with the 1D
+    // double tables' own rounding (about n ulps) that the reference shares
+    double kmax = 0;
+    for (int i = 0; i < N; ++i)
+      for (int j = 0; j < N; ++j) kmax = std::max(kmax, std::fabs(tb.K[i][j]));
+    const double tol = 8.0 * N * 0x1p-53 * 3.0 * h * kmax;
+    if (!(num <= tol)) { std::printf("n=%d kind %d err %g tol %g\n", N, kind, num, tol); bad = 1; }
+  }
+  return bad;
+}
+
+static int conversions() {
+  int bad = 0;
+  const double inf = std::numeric_limits<double>::infinity();
+  const double xs[] = {0.0, -0.0, 1.0, -1.0, 1.9999999999999998, -0x1.8p-7, 0x1.fffffffffffffp-3,
+                       0x1.fffffffffffffp+1023, -0x1p-1022, 0x0.0000000000001p-1022,
+                       -0x0.8000000000001p-1022, 0x1.23456789abcdep-1000, 0x1p+1000};
+  for (double x : xs) {
+    const int E = std::max(1, (int)(fix::mag_hi(bits(x)) >> 20));
+    for (int d = 0; d < 8 && E + d < 0x7ff; ++d) {       // the cell's largest is 2^d larger
+      const int64_t q = fix::from_double<true>(bits(x), E + d);
+      const double y = val(fix::to_double<true>(q, E + d - 59));
+      if (y != x) { std::printf("round trip %a (+%d): %a\n", x, d, y); bad = 1; }
+      if (fix::plain_exp(E + d)) {
+        const int64_t p = fix::from_double<false>(bits(x), E + d);
+        if (p != q || val(fix::to_double<false>(p, E + d - 59)) != x) {
+          std::printf("plain %a (+%d)\n", x, d);
+          bad = 1;
+        }
+      }
+    }
+  }
+  // values far below the largest round down; overflow gives infinity; ties away are nearest
+  bad |= fix::from_double<false>(bits(1.0), 1023 + 60) != 0;
+  bad |= fix::from_double<false>(bits(-1.0), 1023 + 200) != -1;
+  bad |= fix::from_double<false>(bits(1.0), 1023 + 59) != 1;
+  bad |= val(fix::to_double<true>(-(1ll << 60), 2046)) != -inf;
+  bad |= val(fix::to_double<true>((1ll << 60), 1986)) != 0x1p+1023;
+  bad |= val(fix::to_double<true>((1ll << 61) - 1, 1986)) != inf;
+  bad |= val(fix::to_double<false>((1ll << 61) - 1, 963)) != 2.0;
+  return bad;
+}
+
+int main() {
+  int bad = conversions();
+  for (double h : {2.0, 2.0 / 3, 2.0 / 96, 2.0 / 1000}) {
+    bad |= cell<2>(h) | cell<3>(h) | cell<4>(h) | cell<5>(h) | cell<6>(h) | cell<7>(h);
+  }
+  return bad;
+}
+"""
+
+
+def test_fixed_point_cell_term_and_conversions(tmp_path):
+    src = tmp_path / "fixed.cpp"
+    src.write_text(SRC)
+    exe = str(tmp_path / "fixed")
+    inc = [f"-I{CSRC}", f"-I{os.path.join(CSRC, '..', '..', 'include')}"]
+    subprocess.run(["g++", "-O1", "-std=c++17", "-ffp-contract=off",
+                    "-fsanitize=signed-integer-overflow", "-fno-sanitize-recover=all",
+                    "-static-libubsan", *inc, str(src),
+                    os.path.join(CSRC, "setup.cpp"), os.path.join(CSRC, "fixed_tables.cpp"),
+                    "-o", exe], check=True)
+    r = subprocess.run([exe], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout + r.stderr
