@@ -150,7 +150,10 @@ static void free_device(DeviceData* dd) {
   cudaFree(dd->ycol32);
   cudaFree(dd->face_phi);
   cudaFree(dd->face_phi32);
-  cudaFree(dd->face_pp);
+  cudaFree(dd->fix_pp);
+  cudaFree(dd->fix_p0);
+  cudaFree(dd->fix_exp);
+  cudaFree(dd->fix_tab);
   cudaFree(dd->nbr);
   cudaFree(dd->stage_x);
   cudaFree(dd->stage_y);
@@ -381,8 +384,9 @@ static int build_device(const HostProblem& hp, DeviceData* dd) {
   }
   if ((e = device_face_phi(hp, fsrc, &dd->face_phi, &dd->face_phi32)) != cudaSuccess) goto err;
   if (d == 3 && hp.desc.extension == SBM_EXT_EXACT &&
-      (e = device_face_pp((int64_t)fsrc.size(), L, n, dd->face_phi, &dd->face_pp)) !=
-          cudaSuccess)
+      ((e = device_face_fix((int64_t)fsrc.size(), L, n, dd->face_phi, make_ktab<double>(hp).W,
+                            &dd->fix_pp, &dd->fix_p0, &dd->fix_exp)) != cudaSuccess ||
+       (e = upload(&dd->fix_tab, hp.fx.face.data(), hp.fx.face.size())) != cudaSuccess))
     goto err;
   if (dd->nslab > 1) {
     // copy streams and events of the pipelined host-buffer apply

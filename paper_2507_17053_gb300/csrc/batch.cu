@@ -316,7 +316,7 @@ void make_table(const sbm_batch* B, const LaunchPlan& L, const T* const* x, T* c
     q.fa.face_cell = dd.face_cell;
     q.fa.face_kind = dd.face_kind;
     q.fa.face_phi = face_phi_of<T>(dd);
-    q.fa.face_pp = face_pp_of<T>(dd);
+    q.fa.fix = face_fix_of(p->hp, dd);
     q.fa.out = fo;
     q.fa.face0 = 0;
     q.fa.nface = dd.nface;

@@ -33,7 +33,7 @@
 #pragma once
 
 #include "chunk_body.cuh"
-#include "face_body.cuh"
+#include "face_fixed.cuh"
 #include "tc_common.cuh"
 
 namespace sbm {
@@ -134,8 +134,14 @@ extern __shared__ __align__(16) unsigned char bk_smem[];
 template <typename T, int D, int N, int EXT, int FPB>
 __device__ SBM_BK_ITEM void face_item(const Prob<T>& P, const KTab<T>& tu, const Item& it,
                                        int rhs) {
-  for (int f0 = it.b; f0 < it.e; f0 += FPB)
-    face_group<T, D, N, EXT, FPB>(P.fa, tu, *P.kt, bk_smem, f0, it.e, rhs);
+  if constexpr (kFaceFixed<T, D, EXT>) {
+    face_fix_begin<N, FPB>(P.fa, bk_smem);
+    for (int f0 = it.b; f0 < it.e; f0 += FPB)
+      face_group_fix<N, FPB>(P.fa, *P.kt, bk_smem, f0, it.e, rhs);
+  } else {
+    for (int f0 = it.b; f0 < it.e; f0 += FPB)
+      face_group<T, D, N, EXT, FPB>(P.fa, tu, *P.kt, bk_smem, f0, it.e, rhs);
+  }
 }
 
 template <typename T, int D, int N, int R>
@@ -398,9 +404,12 @@ size_t smem_dn(int v, int fh, int ext, int tc) {
   if constexpr (D == 3) {
     if (v == 3) c = DirectSmem<T, N, R>::bytes;
   }
-  const size_t f = ext ? face_group_smem<T, D, N, 1, FF>()
-                       : (fh ? face_group_smem<T, D, N, 0, FHALF>()
-                             : face_group_smem<T, D, N, 0, FF>());
+  size_t f = ext ? face_group_smem<T, D, N, 1, FF>()
+                 : (fh ? face_group_smem<T, D, N, 0, FHALF>()
+                       : face_group_smem<T, D, N, 0, FF>());
+  if constexpr (kFaceFixed<T, D, 0>) {
+    if (!ext) f = fh ? FaceFixSmem<N, FHALF>::bytes : FaceFixSmem<N, FF>::bytes;
+  }
   const size_t g = tc ? tc_item_smem<N>() : 0;
   return std::max(std::max(c, f), g);
 }

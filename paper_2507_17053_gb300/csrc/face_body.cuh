@@ -1,6 +1,7 @@
 // Surrogate-boundary faces (Algorithm 3): the per-face device routine shared
 // by the single-problem face kernel (face_kernel.cu) and the persistent
-// batched apply.  See face_kernel.cu for the method.
+// batched apply.  See face_kernel.cu for the method, face_fixed.cuh for the
+// 3D FP64 faces with the exact extension.
 #pragma once
 
 #include <type_traits>
@@ -8,6 +9,23 @@
 #include "sweeps.cuh"
 
 namespace sbm {
+
+// Tables of the fixed-point faces (face_fixed.cuh; 3D FP64, exact extension).
+struct FaceFix {
+  const fix::Entry* __restrict__ pp;       // [F][n^2][L] products of axes 1, 2 (j1 + n j2)
+  const fix::Entry* __restrict__ p0;       // [F][n][L] weighted values of axis 0
+  const int32_t* __restrict__ exp;         // [F] exponent of the weighted extension
+  const fix::Entry* __restrict__ tab;      // D0, M, S
+  int eq, etm;                             // result exponents of q (plus exp[f]) and tm
+};
+
+inline FaceFix face_fix_of(const HostProblem& hp, const DeviceData& dd) {
+  return FaceFix{dd.fix_pp, dd.fix_p0, dd.fix_exp, dd.fix_tab, hp.fx.face_eq, hp.fx.face_etm};
+}
+
+// 3D exact FP64 faces run in fixed point
+template <typename T, int D, int EXT>
+constexpr bool kFaceFixed = D == 3 && EXT == 0 && std::is_same<T, double>::value;
 
 template <typename T>
 struct FaceArgs {
@@ -17,7 +35,7 @@ struct FaceArgs {
   const int32_t* __restrict__ face_cell;   // face -> ordered cell position
   const int32_t* __restrict__ face_kind;   // k | (s << 2)
   const T* __restrict__ face_phi;          // [F][L][D][N], or the shifts [F][L][D] (Taylor)
-  const T* __restrict__ face_pp;           // 3D exact, FP64: [F][N^2][L] products of axes 1, 2
+  FaceFix fix;                             // 3D exact, FP64
   T* __restrict__ out;                     // [F][2L]
   int face0, nface;                        // this launch: faces [face0, nface)
   int dg;
@@ -45,6 +63,7 @@ template <typename T, int D, int N, int EXT, int FPB>
 __device__ __forceinline__ void face_group(const FaceArgs<T>& a, const KTab<T>& t,
                                            const KTab<T>& ts, unsigned char* smem_raw, int f0,
                                            int fend, int rhs) {
+  static_assert(!kFaceFixed<T, D, EXT>, "face_group_fix");
   constexpr int L = Shape<D, N>::L, ND = Shape<D, N>::ND;
   constexpr int NS = FaceScratch<EXT>::n;
   const T* __restrict__ xr = a.x + rhs * a.ldx;
@@ -130,18 +149,15 @@ __device__ __forceinline__ void face_group(const FaceArgs<T>& a, const KTab<T>& 
 #pragma unroll
       for (int j = 0; j < N; ++j) tm = fma(t.M[tl][j], Td[j], tm);
     }
-    // 3. E u at the shifted point of Gauss point tl, weighted.  3D FP64:
-    //    E u = sum_j0 phi_j0 sum_{j1,j2} P[j1 + n j2] u[j0, j1, j2] with the
-    //    stored products P of the other two axes' values: n^3 + n FMAs
-    //    instead of n^3 + n^2 + n (FP32: the products cost less than their
-    //    loads, the 1D values are contracted axis by axis)
+    // 3. E u at the shifted point of Gauss point tl, weighted; the 1D values
+    //    are contracted axis by axis
     if (act) {
       const T* pq = a.face_phi + ((size_t)f * L + tl) * D * N;
       T p0[N];
 #pragma unroll
       for (int j = 0; j < N; ++j) p0[j] = __ldg(pq + j);
       T e = T(0);
-      if (D == 3 && !std::is_same<T, double>::value) {
+      if (D == 3) {
         T p1[N], p2[N];
 #pragma unroll
         for (int j = 0; j < N; ++j) {
@@ -160,19 +176,6 @@ __device__ __forceinline__ void face_group(const FaceArgs<T>& a, const KTab<T>& 
           }
           e = fma(p2[j2], s1, e);
         }
-      } else if (D == 3) {
-        const T* pp = a.face_pp + (size_t)f * N * N * L + tl;
-        T acc[N];
-#pragma unroll
-        for (int j0 = 0; j0 < N; ++j0) acc[j0] = T(0);
-#pragma unroll
-        for (int j12 = 0; j12 < N * N; ++j12) {
-          const T w = __ldg(pp + (size_t)j12 * L);
-#pragma unroll
-          for (int j0 = 0; j0 < N; ++j0) acc[j0] = fma(w, Xf[j0 + N * j12], acc[j0]);
-        }
-#pragma unroll
-        for (int j0 = 0; j0 < N; ++j0) e = fma(p0[j0], acc[j0], e);
       } else {
         T p1[N];
 #pragma unroll

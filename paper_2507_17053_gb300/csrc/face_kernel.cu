@@ -19,7 +19,7 @@
 //   R[node (kend, jt)] += rv[jt],  R[node (j, jt)] += phi_j'(s) rg[jt].
 // Output: out[f * 2L + jt] = rv[jt], out[f * 2L + L + jt] = rg[jt].  Faces
 // write disjoint slots, so there is no ordering hazard and no atomics.
-#include "face_body.cuh"
+#include "face_fixed.cuh"
 
 namespace sbm {
 
@@ -32,6 +32,20 @@ sface_kernel(const FaceArgs<T> a, const __grid_constant__ KTab<T> t) {
   face_group<T, D, N, EXT, Shape<D, N>::CPB>(a, t, t, smem_raw,
                                               a.face0 + blockIdx.x * Shape<D, N>::CPB, a.nface,
                                               blockIdx.y);
+}
+
+// Fixed-point faces (3D FP64, exact extension): 256 / L faces per block, 4
+// blocks per SM up to n = 5 (64 registers), 3 above (80; with 3 blocks n = 4
+// is 12 % slower, with 2 n = 5 22 %, n = 7 3 % faster).
+template <int N>
+constexpr int fix_faces() { return 256 / (N * N); }
+template <int N>
+__global__ void __launch_bounds__(fix_faces<N>() * N * N, N <= 5 ? 4 : 3)
+sface_fix_kernel(const FaceArgs<double> a, const __grid_constant__ KTab<double> t) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  constexpr int FPB = fix_faces<N>();
+  face_fix_begin<N, FPB>(a, smem_raw);
+  face_group_fix<N, FPB>(a, t, smem_raw, a.face0 + blockIdx.x * FPB, a.nface, blockIdx.y);
 }
 
 template <typename T, int D, int N, int EXT>
@@ -47,15 +61,22 @@ static cudaError_t face_t(const HostProblem& hp, const DeviceData& dd, const T* 
   a.face_cell = dd.face_cell;
   a.face_kind = dd.face_kind;
   a.face_phi = face_phi_of<T>(dd);
-  a.face_pp = face_pp_of<T>(dd);
+  a.fix = face_fix_of(hp, dd);
   a.out = out;
   a.face0 = fb;
   a.nface = fe;
   a.dg = hp.desc.dg;
   a.ldx = ldx;
   a.ld_out = (int64_t)dd.nface * 2 * L;
-  const size_t smem = face_group_smem<T, D, N, EXT, FPB>();
-  sface_kernel<T, D, N, EXT><<<dim3((fe - fb + FPB - 1) / FPB, nrhs), FPB * L, smem, st>>>(a, t);
+  if constexpr (kFaceFixed<T, D, EXT>) {
+    constexpr int FX = fix_faces<N>();
+    sface_fix_kernel<N><<<dim3((fe - fb + FX - 1) / FX, nrhs), FX * L,
+                          FaceFixSmem<N, FX>::bytes, st>>>(a, t);
+  } else {
+    const size_t smem = face_group_smem<T, D, N, EXT, FPB>();
+    sface_kernel<T, D, N, EXT><<<dim3((fe - fb + FPB - 1) / FPB, nrhs), FPB * L, smem, st>>>(a,
+                                                                                             t);
+  }
   return cudaGetLastError();
 }
 

@@ -38,6 +38,7 @@ namespace sbm {
 namespace fix {
 
 constexpr int kMaxHalf = 4;          // ceil(7 / 2)
+constexpr int kFaceExpBad = -0x40000000;   // exponent of a face with non-finite tables
 
 // the output shifts K of the phases for n nodes: x-lines, y-modes back,
 // z-modes back (the transforms to the modes need none)
@@ -58,7 +59,7 @@ struct Block {
 };
 
 // a value split for the products
-struct Split {
+struct alignas(8) Split {
   int32_t h, l;                      // q = h 2^31 + l, 0 <= l < 2^31
 };
 SBM_FIX Split split(int64_t q) { return Split{(int32_t)(q >> 31), (int32_t)(q & 0x7fffffff)}; }

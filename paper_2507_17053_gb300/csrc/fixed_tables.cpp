@@ -60,6 +60,7 @@ void legendre(int m, const DD& t, DD* P, DD* dP) {
 struct Pencil {
   int n;
   DD M[kMaxN][kMaxN], K[kMaxN][kMaxN], V[kMaxN][kMaxN], lam[kMaxN];
+  DD S[kMaxN][kMaxN], D0[kMaxN];     // phi_j at Gauss point q, phi_j'(0)
 };
 
 // 1D mass and stiffness matrices from double-double nodes and Gauss points
@@ -93,19 +94,25 @@ void mass_stiffness(const Tables1D& t, Pencil* P) {
   }
   for (int i = 0; i < n; ++i)
     for (int j = 0; j < n; ++j) P->M[i][j] = P->K[i][j] = DD();
-  for (int q = 0; q < n; ++q) {
-    DD v[kMaxN], dv[kMaxN];
+  auto lagrange = [&](const DD& s, DD* v, DD* dv) {
     for (int j = 0; j < n; ++j) {
       DD a = 1.0, b;
       for (int m = 0; m < n; ++m) {
         if (m == j) continue;
         const DD f = DD(1.0) / (x[j] - x[m]);
-        b = (b * (g[q] - x[m]) + a) * f;
-        a = a * (g[q] - x[m]) * f;
+        b = (b * (s - x[m]) + a) * f;
+        a = a * (s - x[m]) * f;
       }
       v[j] = a;
       dv[j] = b;
     }
+  };
+  DD ends[kMaxN];
+  lagrange(DD(0.0), ends, P->D0);
+  for (int q = 0; q < n; ++q) {
+    DD v[kMaxN], dv[kMaxN];
+    lagrange(g[q], v, dv);
+    for (int j = 0; j < n; ++j) P->S[q][j] = v[j];
     for (int i = 0; i < n; ++i)
       for (int j = 0; j < n; ++j) {
         P->M[i][j] = P->M[i][j] + w[q] * v[i] * v[j];
@@ -317,6 +324,29 @@ bool build_fixed_tables(const Tables1D& tb, double scale, FixedTables* out) {
       }
     }
   out->eoff = -59 - S5 + eh;
+  // faces: t = 61 - ceil(log2) of the largest absolute sum; the trace of D0
+  // is taken of 57-bit values and leaves at 60 bits (K = 3)
+  double cD = 0.0, cM = 0.0, cS = 0.0;
+  for (int j = 0; j < n; ++j) {
+    double m = 0.0, s = 0.0;
+    for (int i = 0; i < n; ++i) {
+      m += mag(P.M[i][j]);
+      s += mag(P.S[i][j]);
+    }
+    cD += mag(P.D0[j]);
+    cM = std::max(cM, m);
+    cS = std::max(cS, s);
+  }
+  auto fit = [](double c) { return 61 - (int)std::ceil(std::log2(c * (1.0 + 1e-6))); };
+  const int tD = fit(cD), tM = fit(cM), tS = fit(cS);
+  out->face.clear();
+  for (int j = 0; j < n; ++j) out->face.push_back(entry(P.D0[j], tD));
+  for (int i = 0; i < n; ++i)
+    for (int j = 0; j < n; ++j) out->face.push_back(entry(P.M[i][j], tM));
+  for (int q = 0; q < n; ++q)
+    for (int j = 0; j < n; ++j) out->face.push_back(entry(P.S[q][j], tS));
+  out->face_eq = 2 + 2 * (61 - tS);
+  out->face_etm = 2 - tD + 2 * (61 - tM);
   return true;
 }
 

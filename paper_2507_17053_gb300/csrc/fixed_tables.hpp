@@ -14,6 +14,10 @@ struct FixedTables {
   fix::Block Vt, V;                  // nodal line -> scaled modes; modes -> nodal line
   std::vector<fix::Entry> xline;     // x-line operators, slot by slot (XLineOp's packed layout)
   int eoff = 0;                      // result unit: biased exponent E + eoff (to_double's eb)
+  // faces (face_fixed.cuh): D0 [n], M [n][n], S [n][n] (phi_j'(0), the mass
+  // matrix, phi_j at the Gauss points), the result exponents of q and tm
+  std::vector<fix::Entry> face;
+  int face_eq = 0, face_etm = 0;
 };
 
 // Tables of the pencil of t for the cell operator scaled by scale = h^(d-2);

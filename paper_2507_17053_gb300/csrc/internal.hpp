@@ -117,10 +117,10 @@ cudaError_t device_chunk_tables(const int32_t* lines, int64_t nc, int L, int n, 
 // face index of kernel face k), FP64 and FP32, allocated here.
 cudaError_t device_face_phi(const HostProblem& hp, const std::vector<int64_t>& fsrc,
                             double** phi, float** phi32);
-// 3D exact extension: the per-point products of the two non-first axes'
-// values from the FP64 table phi ([F][Q][3][n]) into pp ([F][n^2][Q]),
-// allocated here.
-cudaError_t device_face_pp(int64_t F, int L, int n, const double* phi, double** pp);
+// 3D exact extension: the fixed-point tables of the FP64 faces from the FP64
+// table phi ([F][Q][3][n]) and the face weights W ([Q]), allocated here.
+cudaError_t device_face_fix(int64_t F, int L, int n, const double* phi, const double* W,
+                            fix::Entry** pp, fix::Entry** p0, int32_t** exp);
 
 // Device-resident set-up data of one problem.
 struct DeviceData {
@@ -159,10 +159,14 @@ struct DeviceData {
   // at the shifted point; first-order Taylor: [F * Q * d] the shift d_q
   double* face_phi = nullptr;
   float* face_phi32 = nullptr;   // the same table rounded to FP32
-  // 3D exact extension (FP64 face kernel): [F][n^2][Q] the products
-  // phi_j1(xi_{q,1}) phi_j2(xi_{q,2}) of the two non-first axes, index
-  // j1 + n j2 (point index fastest)
-  double* face_pp = nullptr;
+  // 3D exact extension, FP64 faces (face_fixed.cuh), point index fastest:
+  // [F][n^2][Q] the products phi_j1(xi_{q,1}) phi_j2(xi_{q,2}) of the two
+  // non-first axes, index j1 + n j2; [F][n][Q] W_q phi_j0(xi_{q,0}); [F] the
+  // exponents; the 1D tables
+  fix::Entry* fix_pp = nullptr;
+  fix::Entry* fix_p0 = nullptr;
+  int32_t* fix_exp = nullptr;
+  fix::Entry* fix_tab = nullptr;
   int32_t* nbr = nullptr;        // DG [Nc * 2d] neighbour rank per (k, s), -1 = surrogate
   double* stage_x = nullptr;     // host-apply staging buffers (allocated on first use)
   double* stage_y = nullptr;
@@ -261,9 +265,6 @@ cudaError_t launch_face_kernel(const HostProblem& hp, const DeviceData& dd, cons
 template <typename T> inline const T* face_phi_of(const DeviceData& dd);
 template <> inline const double* face_phi_of<double>(const DeviceData& dd) { return dd.face_phi; }
 template <> inline const float* face_phi_of<float>(const DeviceData& dd) { return dd.face_phi32; }
-template <typename T> inline const T* face_pp_of(const DeviceData& dd);
-template <> inline const double* face_pp_of<double>(const DeviceData& dd) { return dd.face_pp; }
-template <> inline const float* face_pp_of<float>(const DeviceData&) { return nullptr; }
 
 // Surrogate faces on the tensor cores (3D, FP32 apply): face_mode
 // SBM_FACE_TF32 or SBM_FACE_BF16; same output as launch_face_kernel.

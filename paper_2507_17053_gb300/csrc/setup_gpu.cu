@@ -665,29 +665,85 @@ cudaError_t device_chunk_tables(const int32_t* lines, int64_t nc, int L, int n, 
   return cudaDeviceSynchronize();
 }
 
-// pp[(f n^2 + j12) L + q] = phi[f][q][1][j1] phi[f][q][2][j2], j12 = j1 + n j2
-__global__ void k_face_pp(int64_t F, int L, int n, const double* __restrict__ phi,
-                          double* __restrict__ pp) {
-  const int64_t nn = (int64_t)n * n;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < F * nn * L;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int q = (int)(t % L);
-    const int64_t fj = t / L;
-    const int j12 = (int)(fj % nn);
-    const int64_t f = fj / nn;
-    const int j1 = j12 % n, j2 = j12 / n;
-    const double* pq = phi + ((size_t)f * L + q) * 3 * n;
-    pp[t] = pq[n + j1] * pq[2 * n + j2];
+// a b 2^t as an entry (the product's rounding error included)
+__device__ __forceinline__ fix::Entry fix_product(double a, double b, int t) {
+  const double p = a * b, err = fma(a, b, -p);
+  const double s = ldexp(p, t);
+  const long long i1 = __double2ll_rn(s);
+  const long long I = i1 + __double2ll_rn((s - (double)i1) + ldexp(err, t));
+  const long long h = (I + (1ll << 29)) >> 30;
+  return fix::Entry{(int32_t)h, (int32_t)(2 * (I - h * (1ll << 30)))};
+}
+
+struct FaceWeights {
+  double W[kMaxN * kMaxN];
+};
+
+// One face per block of 64 threads, one point per thread: pp = phi1 phi2 2^t
+// with absolute row sum in (2^60, 2^61), p0 = W phi0 2^(61 - t - exp[f]).
+__global__ void __launch_bounds__(64)
+k_face_fix(int64_t F, int L, int n, const double* __restrict__ phi,
+           const __grid_constant__ FaceWeights fw, fix::Entry* __restrict__ pp,
+           fix::Entry* __restrict__ p0, int32_t* __restrict__ exp) {
+  __shared__ int s_exp, s_bad;
+  const int q = threadIdx.x;
+  for (int64_t f = blockIdx.x; f < F; f += gridDim.x) {
+    if (q == 0) {
+      s_exp = INT_MIN;
+      s_bad = 0;
+    }
+    __syncthreads();
+    const double* ph = phi + ((size_t)f * L + (q < L ? q : 0)) * 3 * n;
+    const double W = fw.W[q < L ? q : 0];
+    int t = 0;
+    if (q < L) {
+      double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+      for (int j = 0; j < n; ++j) {
+        s0 += fabs(ph[j]);
+        s1 += fabs(ph[n + j]);
+        s2 += fabs(ph[2 * n + j]);
+      }
+      const double b12 = s1 * s2 * (1.0 + 1e-6), b0 = s0 * W * (1.0 + 1e-6);
+      if (isfinite(b12) && isfinite(b0)) {
+        int e12, e0;
+        frexp(b12, &e12);
+        frexp(b0, &e0);
+        t = 61 - e12;
+        atomicMax(&s_exp, e0 - t);
+      } else {
+        atomicOr(&s_bad, 1);
+      }
+    }
+    __syncthreads();
+    const int ef = s_exp;
+    const bool bad = s_bad != 0;
+    if (q == 0) exp[f] = bad ? fix::kFaceExpBad : ef;
+    if (q < L) {
+      for (int j2 = 0; j2 < n; ++j2)
+        for (int j1 = 0; j1 < n; ++j1)
+          pp[((size_t)f * n * n + j1 + n * j2) * L + q] =
+              bad ? fix::Entry{0, 0} : fix_product(ph[n + j1], ph[2 * n + j2], t);
+      for (int j = 0; j < n; ++j)
+        p0[((size_t)f * n + j) * L + q] =
+            bad ? fix::Entry{0, 0} : fix_product(W, ph[j], 61 - t - ef);
+    }
+    __syncthreads();               // s_exp, s_bad are reused
   }
 }
 
-cudaError_t device_face_pp(int64_t F, int L, int n, const double* phi, double** pp) {
-  *pp = nullptr;
+cudaError_t device_face_fix(int64_t F, int L, int n, const double* phi, const double* W,
+                            fix::Entry** pp, fix::Entry** p0, int32_t** exp) {
+  *pp = *p0 = nullptr;
+  *exp = nullptr;
   if (F == 0) return cudaSuccess;
-  const size_t cnt = (size_t)F * n * n * L;
+  FaceWeights fw = {};
+  for (int q = 0; q < L; ++q) fw.W[q] = W[q];
   cudaError_t e;
-  if ((e = cudaMalloc((void**)pp, cnt * 8)) != cudaSuccess) return e;
-  k_face_pp<<<grid_for((int64_t)cnt), 256>>>(F, L, n, phi, *pp);
+  if ((e = cudaMalloc((void**)pp, (size_t)F * n * n * L * sizeof(fix::Entry))) != cudaSuccess ||
+      (e = cudaMalloc((void**)p0, (size_t)F * n * L * sizeof(fix::Entry))) != cudaSuccess ||
+      (e = cudaMalloc((void**)exp, (size_t)F * sizeof(int32_t))) != cudaSuccess)
+    return e;
+  k_face_fix<<<(unsigned)std::min<int64_t>(F, 1 << 16), 64>>>(F, L, n, phi, fw, *pp, *p0, *exp);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   return cudaDeviceSynchronize();
 }

@@ -1,4 +1,4 @@
-"""The fixed-point arithmetic of the 3D FP64 cell term (fixed_point.cuh,
+"""The fixed-point arithmetic of the 3D FP64 cell term and faces (fixed_point.cuh,
 fixed_tables.cpp), compiled for the host: the cell operator against extended
 precision and the conversions at the ends of the exponent range."""
 import os
@@ -149,8 +149,72 @@ static int conversions() {
   return bad;
 }
 
+// The faces' sums at their bounds (absolute sum of the products 2^61, values of +-2^57;
+// overflow stops the program) against 128-bit sums, and the 1D face tables.
+template <int N>
+int faces() {
+  int bad = 0;
+  Tables1D tb;
+  build_tables(N - 1, &tb);
+  FixedTables ft;
+  if (!build_fixed_tables(tb, 0.1, &ft)) return 1;
+  for (int kind = 0; kind < 4; ++kind) {
+    fix::Entry w[N * N];
+    fix::Split x[N * N];
+    int64_t A[N * N], q[N * N];
+    for (int j = 0; j < N * N; ++j) {
+      // equal magnitudes with the low part at its largest, or one dominant product
+      const double m = std::ldexp(1.0 / (1.0 + 1e-6), 61);
+      int64_t a = kind == 3 ? (j ? 1 : (int64_t)m - N * N) : (int64_t)(m / (N * N));
+      if (kind < 3) a = ((a >> 30) << 30) - ((int64_t)1 << 29);
+      if (kind == 1 && rnd() < 0) a = -a;
+      A[j] = a;
+      const int64_t h = (a + ((int64_t)1 << 29)) >> 30;
+      w[j] = fix::Entry{(int32_t)h, (int32_t)(2 * (a - h * ((int64_t)1 << 30)))};
+      const double v = kind == 2 ? -1.9999999999999998 : (A[j] < 0 ? -1.0 : 1.9999999999999998);
+      q[j] = fix::from_double<false>(bits(v), 1023) >> 3;
+      x[j] = fix::split(q[j]);
+    }
+    int64_t hi = 0, mid = (int64_t)1 << 27;
+    __int128 ref = 0;
+    for (int j = 0; j < N * N; ++j) {
+      hi = fix::mad_wide(w[j].h, x[j].h, hi);
+      mid = fix::mad_wide(w[j].h, x[j].l, mid);
+      mid = fix::mad_wide(w[j].l, x[j].h, mid);
+      ref += (__int128)A[j] * q[j];
+    }
+    const int64_t r = fix::shl_add<3>(hi, mid >> 28), e = (int64_t)(ref >> 58);
+    // the dropped products l ql: below 2^61 N^2 in units of 2^-59 of r's
+    if (std::llabs(r - e) > 2 + 8 * N * N || std::llabs(r) > (1ll << 60)) {
+      std::printf("faces n=%d kind %d: %lld %lld\n", N, kind, (long long)r, (long long)e);
+      bad = 1;
+    }
+    fix::Split y[N];
+    for (int j = 0; j < N; ++j) y[j] = fix::split(j & 1 ? -(1ll << 60) : (1ll << 60));
+    for (int i = 0; i < N; ++i) {
+      // columns of S and of M, the row of D0 on 57-bit values
+      auto S = [&](int j) { return ft.face[N + N * N + N * j + i]; };
+      auto M = [&](int j) { return ft.face[N + N * j + i]; };
+      bad |= std::llabs(fix::dot<0, N>(S, y)) > (1ll << 60);
+      bad |= std::llabs(fix::dot<0, N>(M, y)) > (1ll << 60);
+      for (int j = 0; j < N; ++j) {
+        const int tS = 61 - (ft.face_eq - 2) / 2;
+        const fix::Entry a = S(j);
+        const double s = std::ldexp((double)a.h * 0x1p30 + 0.5 * a.l, -tS);
+        // the double table: N - 1 factors of three roundings, |phi| <= 1
+        if (std::fabs(s - tb.S[j][i]) > 3 * N * 0x1p-53) { std::printf("S n=%d %d %d\n", N, j, i); bad = 1; }
+      }
+    }
+    fix::Split z[N];
+    for (int j = 0; j < N; ++j) z[j] = fix::split(ft.face[j].h < 0 ? -(1ll << 57) : (1ll << 57));
+    bad |= std::llabs(fix::dot<3, N>([&](int j) { return ft.face[j]; }, z)) > (1ll << 60);
+  }
+  return bad;
+}
+
 int main() {
   int bad = conversions();
+  bad |= faces<2>() | faces<3>() | faces<4>() | faces<5>() | faces<6>() | faces<7>();
   for (double h : {2.0, 2.0 / 3, 2.0 / 96, 2.0 / 1000}) {
     bad |= cell<2>(h) | cell<3>(h) | cell<4>(h) | cell<5>(h) | cell<6>(h) | cell<7>(h);
   }
