@@ -10,8 +10,10 @@
 //    iterations of a chunk into no-ops, and the host reads the state once
 //    per chunk;
 //  * GMRES(m) orthogonalises with classical Gram-Schmidt applied twice
-//    (CGS2) and keeps the small Hessenberg least-squares problem (Givens
-//    rotations) on the host, one short read per Arnoldi step.
+//    (CGS2), three kernels per Arnoldi step; each writes its column of the
+//    Hessenberg matrix to page-locked memory, and the host (Givens rotations)
+//    follows one step behind, so the device never waits for it.
+#include <algorithm>
 #include <cmath>
 #include <functional>
 #include <vector>
@@ -220,28 +222,6 @@ __global__ void k_residual(const T* __restrict__ b, T* __restrict__ y, int64_t n
     y[i] = b[i] - y[i];
 }
 
-// v = w * (1 / nrm[0]) with nrm a device scalar holding the squared norm
-template <typename T>
-__global__ void k_scale_inv_sqrt(T* __restrict__ v, const T* __restrict__ w,
-                                 const double* __restrict__ nrm2, int64_t n) {
-  const double s = 1.0 / sqrt(*nrm2);
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    v[i] = (T)((double)w[i] * s);
-}
-
-// w -= sum_j h[j] V_j  (j < m)
-template <typename T>
-__global__ void k_multi_axpy(T* __restrict__ w, const T* __restrict__ V, int64_t ldv,
-                             const double* __restrict__ h, int m, int64_t n) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    double acc = (double)w[i];
-    for (int j = 0; j < m; ++j) acc = fma(-h[j], (double)V[j * ldv + i], acc);
-    w[i] = (T)acc;
-  }
-}
-
 // x += sum_j y[j] V_j, accumulated in double (x may be T or double)
 template <typename TX, typename T>
 __global__ void k_update_x(TX* __restrict__ x, const T* __restrict__ V, int64_t ldv,
@@ -402,6 +382,241 @@ SolveStatus solve_cg(const ApplyFn<double>& apply, int64_t n, const double* b, d
   return ret;
 }
 
+// ---- Arnoldi step (GMRES) ----------------------------------------------------
+//
+// Basis vectors are kept unnormalised, v_i = s_i U_i (s_i = 1 / |U_i|), so no
+// kernel only scales.  q = A U_j; one step is
+//   kDot1   h1_i = s_j s_i (U_i, q)
+//   kDot2   U_{j+1} = s_j q - sum_i h1_i s_i U_i,  h2_i = s_i (U_i, U_{j+1})
+//   kNorm   U_{j+1} -= sum_i h2_i s_i U_i,  column h1 + h2, |U_{j+1}|
+// A block owns gm_rows rows and walks them in tiles of tr rows: 256 / tr
+// threads share a row's sum over i, a warp takes four dot products over the
+// tile at a time.  The last block to finish sums the blocks' partials in
+// block order, so results do not depend on the schedule.  Few rows: tiles of
+// 64 rows and up to 8 blocks (gridDim.y) that split the dot products of the
+// same rows (each repeats the rows' axpy; the double-precision pipe of one SM
+// would bind, 2 operations per clock).
+// Residual norm: with phi the left null vector of the (k+1) x k Hessenberg
+// matrix, phi_0 = 1, it is beta / |phi|; one dot product per step ends the
+// cycle on the device (ctl->done), where Givens rotations would be a chain of
+// j dependent operations.
+// Measured, disk of 1 801 DoFs, restart 100, 625 steps (18 us apply each):
+// whole solve 341 -> 26.6 ms (1 216 blocks per dot product, eleven stream
+// operations and a host round trip per step before).
+constexpr int GM_MAXB = 304;       // row blocks at most, 2 per SM
+constexpr int GM_SLICES = 8;       // blocks sharing the dot products of the same rows, at most
+constexpr int GM_RING = 4;         // columns in flight to the host
+constexpr int GM_AHEAD = 2;        // steps enqueued ahead of the host's test
+enum { kDot1 = 0, kDot2 = 1, kNorm = 2 };
+
+struct GmCtl {
+  double sumphi2, beta, tol;       // |phi|^2, |r_0|, absolute residual to stop at
+  int done;
+  unsigned cnt[3][GM_SLICES];      // finished blocks (reset by the last one)
+};
+
+// scales, h1, h2, phi: [m + 1] each
+struct GmVecs {
+  double *s, *h1, *h2, *phi, *part;   // part [(m + 1)][GM_MAXB]
+};
+
+__global__ void k_gm_begin(GmCtl* ctl, GmVecs g, double beta, double tol) {
+  ctl->sumphi2 = 1.0;
+  ctl->beta = beta;
+  ctl->tol = tol;
+  ctl->done = 0;
+  for (int i = 0; i < 3 * GM_SLICES; ++i) (&ctl->cnt[0][0])[i] = 0u;
+  g.s[0] = 1.0;
+  g.phi[0] = 1.0;
+}
+
+template <typename T, int MODE>
+__global__ void __launch_bounds__(256)
+k_gm_step(const T* q, T* V, int64_t n, int j, int rows, int tr,
+          const GmVecs g, GmCtl* ctl, double* __restrict__ col) {
+  extern __shared__ double gm_smem[];
+  __shared__ double wt[256], red[256];
+  __shared__ int s_last;
+  pdl_wait_all();
+  if (ctl->done) return;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int nj = j + 1, per = (nj + gridDim.y - 1) / gridDim.y;
+  const int i0 = min(nj, (int)blockIdx.y * per), i1 = min(nj, i0 + per);
+  double* coef = gm_smem;            // [nj]
+  double* dacc = gm_smem + nj;       // [per] dot products of the block's rows
+  if (MODE != kDot1)
+    for (int i = tid; i < nj; i += 256) coef[i] = (MODE == kDot2 ? g.h1[i] : g.h2[i]) * g.s[i];
+  if (MODE != kNorm)
+    for (int i = tid; i < per; i += 256) dacc[i] = 0.0;
+  const double sj = g.s[j];
+  T* u = V + (int64_t)nj * n;
+  const int64_t r_end = min(n, ((int64_t)blockIdx.x + 1) * rows);
+  const int r = tid % tr, js = tid / tr, split = 256 / tr;
+  double nrm = 0.0;
+  for (int64_t base = (int64_t)blockIdx.x * rows; base < r_end; base += tr) {
+    const int nr = (int)min((int64_t)tr, r_end - base);
+    __syncthreads();                 // coef; wt and red are reused
+    if (MODE == kDot1) {
+      if (tid < nr) wt[tid] = (double)q[base + tid];
+    } else {
+      double acc = 0.0;
+      if (r < nr) {
+        const T* vr = V + base + r;
+#pragma unroll 4
+        for (int i = js; i < nj; i += split) acc = fma(-coef[i], (double)vr[(int64_t)i * n], acc);
+      }
+      red[tid] = acc;
+      __syncthreads();
+      if (tid < nr) {
+        double w = MODE == kDot2 ? sj * (double)q[base + tid] : (double)u[base + tid];
+        for (int k = 0; k < split; ++k) w += red[tid + k * tr];
+        const T wr = (T)w;
+        wt[tid] = (double)wr;
+        if (blockIdx.y == 0) u[base + tid] = wr;
+        if (MODE == kNorm) nrm = fma((double)wr, (double)wr, nrm);
+      }
+    }
+    if (MODE == kNorm) continue;
+    __syncthreads();
+    for (int ib = i0 + 4 * wid; ib < i1; ib += 32) {
+      double a[4] = {0.0, 0.0, 0.0, 0.0};
+      for (int rr = lane; rr < nr; rr += 32) {
+        const double w = wt[rr];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          a[k] = fma((double)V[(int64_t)min(ib + k, i1 - 1) * n + base + rr], w, a[k]);
+      }
+      // four sums over the warp in six additions: lanes >= 16 keep a[2..3],
+      // then every other eight lanes one of the two
+      const bool h16 = lane & 16, h8 = lane & 8;
+      const double s0 = __shfl_xor_sync(~0u, h16 ? a[0] : a[2], 16);
+      const double s1 = __shfl_xor_sync(~0u, h16 ? a[1] : a[3], 16);
+      const double b0 = (h16 ? a[2] : a[0]) + s0, b1 = (h16 ? a[3] : a[1]) + s1;
+      double c = (h8 ? b1 : b0) + __shfl_xor_sync(~0u, h8 ? b0 : b1, 8);
+      for (int o = 4; o > 0; o >>= 1) c += __shfl_xor_sync(~0u, c, o);
+      const int i = ib + (h16 ? 2 : 0) + (h8 ? 1 : 0);
+      if ((lane & 7) == 0 && i < i1) dacc[i - i0] += c;
+    }
+  }
+  __syncthreads();
+  const int nb = gridDim.x;
+  if (MODE == kNorm) {
+    for (int o = 16; o > 0; o >>= 1) nrm += __shfl_xor_sync(~0u, nrm, o);
+    if (lane == 0) red[wid] = nrm;
+    __syncthreads();
+    if (tid == 0) {
+      double s = 0.0;
+      for (int w = 0; w < 8; ++w) s += red[w];
+      g.part[blockIdx.x] = s;
+    }
+  } else {
+    for (int i = i0 + tid; i < i1; i += 256) g.part[(int64_t)i * GM_MAXB + blockIdx.x] = dacc[i - i0];
+  }
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) {
+    unsigned* c = &ctl->cnt[MODE][blockIdx.y];
+    s_last = atomicAdd(c, 1u) == (unsigned)nb - 1u;
+    if (s_last) *c = 0u;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  if (MODE != kNorm) {               // eight lanes per dot product
+    for (int ib = i0; ib < i1; ib += 32) {
+      const int i = ib + (tid >> 3);
+      double s = 0.0;
+      if (i < i1)
+        for (int b = tid & 7; b < nb; b += 8) s += __ldcg(g.part + (int64_t)i * GM_MAXB + b);
+      for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(~0u, s, o);
+      if (i < i1 && (tid & 7) == 0) {
+        if (MODE == kDot1) g.h1[i] = s * sj * g.s[i];
+        else g.h2[i] = s * g.s[i];
+      }
+    }
+    return;
+  }
+  // the column, its norm and the residual
+  double ph = 0.0, s = 0.0;
+  for (int i = tid; i < nj; i += 256) {
+    const double c = g.h1[i] + g.h2[i];
+    col[1 + i] = c;
+    ph = fma(g.phi[i], c, ph);
+  }
+  for (int b = tid; b < nb; b += 256) s += __ldcg(g.part + b);
+  for (int o = 16; o > 0; o >>= 1) {
+    s += __shfl_xor_sync(~0u, s, o);
+    ph += __shfl_xor_sync(~0u, ph, o);
+  }
+  __syncthreads();
+  if (lane == 0) {
+    red[wid] = s;
+    red[8 + wid] = ph;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    s = ph = 0.0;
+    for (int w = 0; w < 8; ++w) {
+      s += red[w];
+      ph += red[8 + w];
+    }
+    const double nr = sqrt(s);
+    col[1 + nj] = nr;
+    g.s[nj] = 1.0 / nr;
+    const double f = -ph / nr;
+    g.phi[nj] = f;
+    const double sum = fma(f, f, ctl->sumphi2);
+    ctl->sumphi2 = sum;
+    const double res = ctl->beta / sqrt(sum);
+    const bool done = !(res > ctl->tol) || !(s > 0.0);
+    if (done) ctl->done = 1;
+    col[0] = done ? 1.0 : 0.0;
+  }
+}
+
+// rows per block and tile of the Arnoldi kernels
+static inline int gm_tile(int64_t n) { return n <= 64 * GM_MAXB ? 64 : 256; }
+static inline int gm_rows(int64_t n) {
+  const int tr = gm_tile(n);
+  const int64_t r = (n + GM_MAXB - 1) / GM_MAXB;
+  return (int)((r + tr - 1) / tr * tr);
+}
+
+template <typename T>
+static cudaError_t gm_step(const T* q, T* V, int64_t n, int j, const GmVecs& g, GmCtl* ctl,
+                           double* col, cudaStream_t st) {
+  const int rows = gm_rows(n), tr = gm_tile(n);
+  const int nb = (int)((n + rows - 1) / rows);
+  const int ny = std::max(1, std::min({GM_SLICES, GM_MAXB / nb, (j + 8) / 8}));
+  const size_t sm = (size_t)2 * (j + 1) * 8;
+  cudaError_t e;
+  if ((e = launch_maybe_pdl(k_gm_step<T, kDot1>, dim3(nb, ny), dim3(256), sm, st, true, q, V, n, j,
+                            rows, tr, g, ctl, col)) != cudaSuccess ||
+      (e = launch_maybe_pdl(k_gm_step<T, kDot2>, dim3(nb, ny), dim3(256), sm, st, true, q, V, n, j,
+                            rows, tr, g, ctl, col)) != cudaSuccess)
+    return e;
+  return launch_maybe_pdl(k_gm_step<T, kNorm>, dim3(nb, 1), dim3(256), sm, st, true, q, V, n, j,
+                          rows, tr, g, ctl, col);
+}
+
+// page-locked ring of Hessenberg columns (each: last step of the cycle or
+// not, then the column) and the events of the steps
+struct GmHost {
+  double* ring = nullptr;
+  cudaEvent_t ev[GM_RING] = {};
+  cudaError_t init(int m) {
+    cudaError_t e = cudaMallocHost((void**)&ring, (size_t)GM_RING * (m + 3) * 8);
+    for (int i = 0; i < GM_RING && e == cudaSuccess; ++i)
+      e = cudaEventCreateWithFlags(&ev[i], cudaEventDisableTiming);
+    return e;
+  }
+  ~GmHost() {
+    for (cudaEvent_t v : ev)
+      if (v) cudaEventDestroy(v);
+    if (ring) cudaFreeHost(ring);
+  }
+};
+
 // ---- GMRES(m) --------------------------------------------------------------
 
 // Givens-based least squares of the Arnoldi relation, host side
@@ -442,6 +657,7 @@ template <typename T, typename TX>
 SolveStatus solve_gmres(const ApplyFn<T>& apply, int64_t n, const TX* b, TX* x, double rtol,
                         int maxit, int restart, cudaStream_t st, Workspace& ws, SolveInfo* info,
                         const ApplyFn<TX>* apply_x) {
+  static_assert(std::is_same<T, TX>::value, "rx is also the Arnoldi step's A U_j");
   // apply_x: operator in the precision of x/b for the outer residual (T == TX: same as apply)
   const int m = restart;
   T* V;
@@ -449,9 +665,19 @@ SolveStatus solve_gmres(const ApplyFn<T>& apply, int64_t n, const TX* b, TX* x, 
   double *part, *dsc;
   CK(ws.alloc((void**)&V, (size_t)(m + 1) * n * sizeof(T)));
   CK(ws.alloc((void**)&rx, (size_t)n * sizeof(TX)));
-  CK(ws.alloc((void**)&part, (size_t)(m + 2) * RED_BLOCKS * 8));
+  CK(ws.alloc((void**)&part, (size_t)RED_BLOCKS * 8));
   CK(ws.alloc((void**)&dsc, (m + 4) * 8));
-  std::vector<double> col(m + 2), y(m + 1);
+  GmVecs g;
+  GmCtl* ctl;
+  CK(ws.alloc((void**)&g.s, (size_t)4 * (m + 1) * 8));
+  g.h1 = g.s + (m + 1);
+  g.h2 = g.h1 + (m + 1);
+  g.phi = g.h2 + (m + 1);
+  CK(ws.alloc((void**)&g.part, (size_t)(m + 1) * GM_MAXB * 8));
+  CK(ws.alloc((void**)&ctl, sizeof(GmCtl)));
+  GmHost gh;
+  CK(gh.init(m));
+  std::vector<double> y(m + 1), scale(m + 2);
   int total = 0, cycles = 0;
   double relres = INFINITY, bnorm = 0.0;
   {
@@ -480,43 +706,36 @@ SolveStatus solve_gmres(const ApplyFn<T>& apply, int64_t n, const TX* b, TX* x, 
     if (relres <= rtol) { status = SBM_OK; break; }
     if (!std::isfinite(relres)) break;
     k_convert_scaled<T, TX><<<vec_grid(n), 256, 0, st>>>(V, rx, 1.0 / std::sqrt(rr), n);
+    k_gm_begin<<<1, 1, 0, st>>>(ctl, g, std::sqrt(rr), 0.5 * rtol * bnorm);
+    CK(cudaGetLastError());
     Hess H(m);
     H.g[0] = std::sqrt(rr);
-    int k = 0;
-    bool conv = false;
-    for (int j = 0; j < m && total < maxit; ++j) {
-      T* vj = V + (size_t)j * n;
-      T* w = V + (size_t)(j + 1) * n;
-      CK(apply(vj, w, st));
-      // CGS2: h = V^T w; w -= V h; twice
-      CK(multi_dot<T>(V, n, w, n, j + 1, part, dsc, st));
-      k_multi_axpy<T><<<vec_grid(n), 256, 0, st>>>(w, V, n, dsc, j + 1, n);
-      CK(cudaMemcpyAsync(col.data(), dsc, (j + 1) * 8, cudaMemcpyDeviceToHost, st));
-      CK(multi_dot<T>(V, n, w, n, j + 1, part, dsc, st));
-      k_multi_axpy<T><<<vec_grid(n), 256, 0, st>>>(w, V, n, dsc, j + 1, n);
-      std::vector<double> h2(j + 1);
-      CK(cudaMemcpyAsync(h2.data(), dsc, (j + 1) * 8, cudaMemcpyDeviceToHost, st));
-      CK(multi_dot<T>(w, 0, w, n, 1, part, dsc + m + 2, st));
-      double hn2;
-      CK(cudaMemcpyAsync(&hn2, dsc + m + 2, 8, cudaMemcpyDeviceToHost, st));
-      CK(cudaStreamSynchronize(st));
-      for (int i = 0; i <= j; ++i) col[i] += h2[i];
-      col[j + 1] = std::sqrt(hn2);
-      k_scale_inv_sqrt<T><<<vec_grid(n), 256, 0, st>>>(w, w, dsc + m + 2, n);
-      const double res = H.add_column(j, col.data());
-      ++total;
-      k = j + 1;
-      if (res / bnorm <= rtol * 0.5 || hn2 == 0.0 || !std::isfinite(res)) {
-        conv = true;
-        break;
+    scale[0] = 1.0;
+    const int lim = std::min(m, maxit - total);
+    int k = 0, enq = 0;
+    while (k < lim) {
+      for (; enq < lim && enq < k + GM_AHEAD; ++enq) {
+        CK(apply(V + (size_t)enq * n, rx, st));
+        CK(gm_step<T>(rx, V, n, enq, g, ctl, gh.ring + (size_t)(enq % GM_RING) * (m + 3), st));
+        CK(cudaEventRecord(gh.ev[enq % GM_RING], st));
       }
+      CK(cudaEventSynchronize(gh.ev[k % GM_RING]));
+      const double* slot = gh.ring + (size_t)(k % GM_RING) * (m + 3);
+      const bool last = slot[0] != 0.0;   // the device ended the cycle with this step
+      const double* col = slot + 1;
+      const double hn = col[k + 1];
+      scale[k + 1] = 1.0 / hn;
+      const double res = H.add_column(k, col);
+      ++total;
+      ++k;
+      if (last || res / bnorm <= rtol * 0.5 || !(hn > 0.0) || !std::isfinite(res)) break;
     }
     H.solve(k, y.data());
+    for (int i = 0; i < k; ++i) y[i] *= scale[i];
     CK(cudaMemcpyAsync(dsc, y.data(), k * 8, cudaMemcpyHostToDevice, st));
     k_update_x<TX, T><<<vec_grid(n), 256, 0, st>>>(x, V, n, dsc, k, 1.0, n);
     CK(cudaGetLastError());
     ++cycles;
-    (void)conv;
   }
   if (status != SBM_OK) {
     // final true residual

@@ -68,6 +68,57 @@ def test_gmres_disk_workload():
     assert np.linalg.norm(x.cpu().numpy() - xref) <= 1e-7 * np.linalg.norm(xref)
 
 
+@pytest.mark.parametrize("w,restart,maxit", [
+    (S._wl("one", 3, 1, 1, S.ball(3, (0.0,) * 3, 0.9)), 1000, 12),      # 8 DoFs: the space is exhausted
+    (S.DISK_2D_Q2, 1, 3),                                    # cycles of one step
+    (S.DISK_2D_Q2, 40, 57),                                  # a second, shorter cycle
+    (S.SPHERE_3D_Q4.resized(20, degree=2), 33, 33),          # 64-row tiles (n <= 19 456)
+    (S.SPHERE_3D_Q4.resized(22, degree=2), 33, 33),          # 256-row tiles
+    (S.SPHERE_3D_Q4.resized(36, degree=3), 10, 10),          # several tiles per block
+], ids=["exhausted", "restart1", "two_cycles", "tile64", "tile256", "tiles"])
+def test_gmres_iterates_match_full_orthogonalisation(w, restart, maxit):
+    """x after maxit steps against GMRES written out in numpy (QR of the
+    Hessenberg matrix) on the same applies.  Both minimise the same residual;
+    their difference is rounding times the conditioning of the Krylov basis'
+    least squares problem (below 1e4 after so few steps): 1e-10."""
+    P = G.Problem.from_workload(w)
+    b = torch.from_numpy(S.random_vector(5, P.n_dofs, "uniform")).cuda()
+    x = torch.zeros_like(b)
+    it, rr, ok = G.sbm_gmres(P.handle, b, x, rtol=1e-13, maxit=maxit, restart=restart)
+    ref, done = torch.zeros_like(b), 0
+    bn = float(b.norm())
+    while done < maxit:
+        r = b - P.apply_f64(ref, torch.empty_like(b))
+        if float(r.norm()) <= 1e-13 * bn:
+            break
+        m = min(restart, maxit - done)
+        V, H = [r / r.norm()], np.zeros((m + 1, m))
+        k = 0
+        while k < m:
+            q = P.apply_f64(V[-1], torch.empty_like(b))
+            for _ in range(2):
+                for i, v in enumerate(V):
+                    h = torch.dot(v, q)
+                    H[i, k] += float(h)
+                    q = q - h * v
+            H[k + 1, k] = float(q.norm())
+            V.append(q / q.norm())
+            k += 1
+            e = np.zeros(k + 1)
+            e[0] = float(r.norm())
+            y, res = np.linalg.lstsq(H[:k + 1, :k], e, rcond=None)[:2]
+            if np.linalg.norm(H[:k + 1, :k] @ y - e) <= 0.5e-13 * bn:
+                break
+        ref = ref + sum(float(c) * v for c, v in zip(y, V))
+        done += k
+    assert it <= maxit
+    if ok:                                # both at the tolerance
+        assert float((b - P.apply_f64(x, torch.empty_like(b))).norm()) <= 1e-13 * bn
+    else:
+        assert it == done
+        assert float((x - ref).norm()) <= 1e-10 * float(ref.norm())
+
+
 @pytest.mark.parametrize("w", [S.DISK_2D_Q2, S.SPHERE_3D_Q4.resized(8, degree=2)],
                          ids=lambda w: w.name)
 def test_mixed_precision_ir(w):
