@@ -100,7 +100,8 @@ __global__ void __launch_bounds__(block_threads<T, 3, N>(R), (direct_min_blocks<
 cg_direct_ord_kernel(const ChunkArgs<T> a, const __grid_constant__ KTab<T> t,
                      const __grid_constant__ OrdArgs o) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  chunk_loop_direct<T, N, R, false, true>(a, t, t, smem_raw, 0, 0, 0, 0, &o);
+  // waits before its folds: it may run as a dependent of the face kernel
+  chunk_loop_direct<T, N, R, true, true, true>(a, t, t, smem_raw, 0, 0, 0, 0, &o);
 }
 
 // Resident blocks per SM x SMs of a kernel (the persistent grid of the
