@@ -57,12 +57,11 @@ template <typename T, int D, int N, int R>
 __global__ void __launch_bounds__(block_threads<T, D, N>(R), (chunk_min_blocks<T, D, N, R>()))
 cg_chunk_kernel(const ChunkArgs<T> a, const __grid_constant__ KTab<T> t) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  // FP32: launched as a programmatic dependent of the face kernel (coherent
-  // face loads, a wait before the first fold); FP64 launches plainly
-  constexpr bool kPdl = std::is_same<T, float>::value;
-  if constexpr (kPdl) pdl_trigger();
+  // launched as a programmatic dependent of the face kernel (coherent face
+  // loads, a wait before the first chunk's cells)
+  pdl_trigger();
   chunk_xline_build<T, D, N, R>(smem_raw, t, a.xfix, threadIdx.x);
-  chunk_loop<T, D, N, R, kPdl, block_threads<T, D, N>(R), kPdl>(a, t, smem_raw, blockIdx.y,
+  chunk_loop<T, D, N, R, true, block_threads<T, D, N>(R), true>(a, t, smem_raw, blockIdx.y,
                                                          a.q0 + blockIdx.x, a.q1, gridDim.x);
 }
 
@@ -89,9 +88,8 @@ template <typename T, int N, int R>
 __global__ void __launch_bounds__(block_threads<T, 3, N>(R), (direct_min_blocks<T, N>()))
 cg_direct_kernel(const ChunkArgs<T> a, const __grid_constant__ KTab<T> t) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  constexpr bool kPdl = std::is_same<T, float>::value;     // as cg_chunk_kernel
-  if constexpr (kPdl) pdl_trigger();
-  chunk_loop_direct<T, N, R, kPdl, false, kPdl>(a, t, t, smem_raw, blockIdx.y,
+  pdl_trigger();                                           // as cg_chunk_kernel
+  chunk_loop_direct<T, N, R, true, false, true>(a, t, t, smem_raw, blockIdx.y,
                                                 a.q0 + blockIdx.x, a.q1, gridDim.x);
 }
 
@@ -172,7 +170,7 @@ assemble_set_kernel(const T* __restrict__ ycol, const int32_t* __restrict__ mult
                     const uint8_t* __restrict__ multi_mask, T* __restrict__ y, int64_t n,
                     int64_t nmulti, int ncol) {
   const int64_t tile = (int64_t)(gridDim.x - 1u - blockIdx.x);
-  assemble_pair<T, false, std::is_same<T, float>::value>(ycol, multi, multi_mask, y, n, nmulti,
+  assemble_pair<T, false, true>(ycol, multi, multi_mask, y, n, nmulti,
                                                          ncol, tile * 512 + threadIdx.x, 256);
 }
 
@@ -225,15 +223,15 @@ static cudaError_t apply_r(const HostProblem& hp, const DeviceData& dd, const Ch
   const bool pr = prof && prof->on;
   int nlaunch = 0;
   if (pr && (err = prof->mark(st)) != cudaSuccess) return err;
-  // programmatic dependent launches (FP32 whole applies, no profiling marks
+  // programmatic dependent launches (whole applies, no profiling marks
   // between the kernels): the cell kernels (shapes 0, 2, 3) after the
   // CUDA-core face kernel (which x's producers precede in the stream), the
   // assembly after the cell kernel.  Measured (unprofiled applies, GB300):
   // FP32 p = 6 ellipsoid (shape 3) 62.7 -> 57.4 us, p = 3 / 4 spheres
-  // (shapes 0, 3) 1-5 % faster, shape 2 1-8 % faster (cell_reg.cu); the
-  // FP64 p = 4 sphere 2.3 % slower (1.026 ->
-  // 1.049 ms), so FP64 launches without it.
-  allow_pdl = allow_pdl && std::is_same<T, float>::value;
+  // (shapes 0, 3) 1-5 % faster, shape 2 1-8 % faster (cell_reg.cu); FP64 (with
+  // the fixed-point faces) disk of 1 801 DoFs 18.4 -> 13.4 us, p = 3 box of
+  // 24^3 cells 29.2 -> 22.7, p = 6 ellipsoid 148 -> 137, p = 4 sphere 381 ->
+  // 372 us.
   bool pdl_cell = false;
   if (part.f1 > part.f0) {
     err = face_mode != 0 ? launch_faces<T>(hp, dd, x, fo, face_mode, st)

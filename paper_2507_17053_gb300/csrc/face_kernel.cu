@@ -27,8 +27,7 @@ template <typename T, int D, int N, int EXT>
 __global__ void __launch_bounds__(Shape<D, N>::CPB * Shape<D, N>::L)
 sface_kernel(const FaceArgs<T> a, const __grid_constant__ KTab<T> t) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  // FP32: the cell kernel may start (it waits before its folds)
-  if constexpr (std::is_same<T, float>::value) pdl_trigger();
+  pdl_trigger();                   // the cell kernel may start (it waits before its folds)
   face_group<T, D, N, EXT, Shape<D, N>::CPB>(a, t, t, smem_raw,
                                               a.face0 + blockIdx.x * Shape<D, N>::CPB, a.nface,
                                               blockIdx.y);
@@ -44,6 +43,7 @@ __global__ void __launch_bounds__(fix_faces<N>() * N * N, N <= 5 ? 4 : 3)
 sface_fix_kernel(const FaceArgs<double> a, const __grid_constant__ KTab<double> t) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int FPB = fix_faces<N>();
+  pdl_trigger();                   // as sface_kernel
   face_fix_begin<N, FPB>(a, smem_raw);
   face_group_fix<N, FPB>(a, t, smem_raw, a.face0 + blockIdx.x * FPB, a.nface, blockIdx.y);
 }
