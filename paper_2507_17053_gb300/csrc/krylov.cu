@@ -5,10 +5,9 @@
 // solvers (Section 4.2).  These drivers keep every vector on the device:
 //  * reductions are deterministic (fixed grid, fixed tree order, FP64
 //    accumulation), so a solve is bitwise reproducible;
-//  * CG keeps its scalars on the device and runs CG_CHUNK iterations per
-//    CUDA-graph launch; a converged/failed flag turns the remaining
-//    iterations of a chunk into no-ops, and the host reads the state once
-//    per chunk;
+//  * CG keeps its scalars on the device; the host enqueues iterations
+//    CG_AHEAD ahead of the outcome it reads, and a converged/failed flag turns
+//    those after the last one into no-ops;
 //  * GMRES(m) orthogonalises with classical Gram-Schmidt applied twice
 //    (CGS2), three kernels per Arnoldi step; each writes its column of the
 //    Hessenberg matrix to page-locked memory, and the host (Givens rotations)
@@ -25,7 +24,7 @@ namespace sbm {
 
 constexpr int RED_BLOCKS = 1216;   // 8 x 152 SMs
 constexpr int RED_THREADS = 256;
-constexpr int CG_CHUNK = 16;
+constexpr int CG_AHEAD = 2;
 
 // ---- deterministic reductions ---------------------------------------------
 
@@ -37,26 +36,47 @@ __device__ __forceinline__ void pdl_wait_all() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-// Sum over the block (every thread gets it), fixed order: warp shuffles, then
-// the warps' sums in order -- 5 + 8 additions on the double-precision pipe (2
-// per SM and clock), against 8 half-empty tree levels of every warp.
+// Sums over the block in fixed order, in thread 0 (sh: 16 values).  The
+// double-precision pipe does 2 operations per SM and clock, so additions are
+// what a small reduction costs: warp shuffles, the two sums of block_sum2
+// sharing theirs (half of the lanes carry on with each after the first step),
+// then one warp over the warps' sums.
 __device__ __forceinline__ double block_sum(double v, double* sh) {
   const int tid = threadIdx.x;
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(~0u, v, o);
   if ((tid & 31) == 0) sh[tid >> 5] = v;
   __syncthreads();
   double r = 0.0;
-  for (int w = 0; w < RED_THREADS / 32; ++w) r += sh[w];
+  if (tid < 32) {
+    r = tid < RED_THREADS / 32 ? sh[tid] : 0.0;
+    for (int o = RED_THREADS / 64; o > 0; o >>= 1) r += __shfl_xor_sync(~0u, r, o);
+  }
   __syncthreads();
   return r;
 }
+__device__ __forceinline__ void block_sum2(double& a, double& b, double* sh) {
+  const int tid = threadIdx.x;
+  const bool h = tid & 16;
+  double v = (h ? b : a) + __shfl_xor_sync(~0u, h ? a : b, 16);
+  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(~0u, v, o);
+  if ((tid & 15) == 0) sh[(tid >> 5) + (h ? 8 : 0)] = v;
+  __syncthreads();
+  if (tid < 32) {
+    double r = tid < RED_THREADS / 16 ? sh[tid] : 0.0;
+    for (int o = RED_THREADS / 64; o > 0; o >>= 1) r += __shfl_xor_sync(~0u, r, o);
+    a = r;
+    b = __shfl_sync(~0u, r, 8);
+  }
+  __syncthreads();
+}
 
 // Blocks of a reduction over n values: 512 values per block (two per thread)
-// up to eight blocks per SM.  A reduction's time over a small vector is that
-// of its blocks' sums, not of the loads.
+// up to two blocks per SM, so that a small vector's time is not that of its
+// blocks' sums; 2 048 per block up to eight per SM, which a vector larger than
+// the L2 cache needs to keep enough loads in flight.
 static inline int red_blocks(int64_t n) {
-  const int64_t b = (n + 511) / 512;
-  return (int)(b < 1 ? 1 : b > RED_BLOCKS ? RED_BLOCKS : b);
+  const int64_t b = std::min<int64_t>((n + 511) / 512, RED_BLOCKS / 4);
+  return (int)std::max<int64_t>(1, std::max(b, std::min<int64_t>(n / 2048, RED_BLOCKS)));
 }
 
 // True in every thread of the grid's last block to get here, whose reads
@@ -75,11 +95,20 @@ __device__ __forceinline__ bool last_block(unsigned* cnt) {
   return s_last != 0;
 }
 
-// sum of part[0 .. nb-1] (every thread), nb partials of other blocks
+// sum of part[0 .. nb-1] (in thread 0), nb partials of other blocks
 __device__ __forceinline__ double part_sum(const double* part, int nb, double* sh) {
   double s = 0.0;
   for (int i = threadIdx.x; i < nb; i += blockDim.x) s += __ldcg(part + i);
   return block_sum(s, sh);
+}
+
+__device__ __forceinline__ void part_sum2(const double* part, int nb, double* sh, double (&v)[2]) {
+  v[0] = v[1] = 0.0;
+  for (int i = threadIdx.x; i < nb; i += blockDim.x) {
+    v[0] += __ldcg(part + i);
+    v[1] += __ldcg(part + RED_BLOCKS + i);
+  }
+  block_sum2(v[0], v[1], sh);
 }
 
 // part[j * RED_BLOCKS + block] = partial sum of a_j . b over this block's rows,
@@ -88,7 +117,7 @@ template <typename T>
 __global__ void k_multi_dot(const T* __restrict__ a, int64_t lda, const T* __restrict__ b,
                             int64_t n, double* __restrict__ part) {
   pdl_wait_all();
-  __shared__ double sh[RED_THREADS / 32];
+  __shared__ double sh[RED_THREADS / 16];
   const T* aj = a + (int64_t)blockIdx.y * lda;
   double s = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
@@ -100,7 +129,7 @@ __global__ void k_multi_dot(const T* __restrict__ a, int64_t lda, const T* __res
 
 // out[j] = sum of part[j * RED_BLOCKS + 0 .. nb-1] (blockIdx.x = j)
 __global__ void k_finalize(const double* __restrict__ part, int nb, double* __restrict__ out) {
-  __shared__ double sh[RED_THREADS / 32];
+  __shared__ double sh[RED_THREADS / 16];
   const double s = part_sum(part + blockIdx.x * RED_BLOCKS, nb, sh);
   if (threadIdx.x == 0) out[blockIdx.x] = s;
 }
@@ -119,26 +148,25 @@ struct CgState {
 // reduction also updates the scalars (five kernels before, box of 226 981
 // DoFs, 372 iterations: 20.7 -> 18.1 ms).
 
-// r = b - q; z = dinv * r (or r); p = z; partials of r.z, r.r, b.b
+// r = b - q; z = dinv * r (no preconditioner: z is r, not stored); p = z; partials of r.z, r.r, b.b
 __global__ void k_cg_init(const double* __restrict__ b, const double* __restrict__ q,
-                          double* __restrict__ r, double* __restrict__ z, double* __restrict__ p,
+                          double* __restrict__ r, double* z, double* __restrict__ p,
                           const double* __restrict__ dinv, int64_t n, double* __restrict__ part) {
-  __shared__ double sh[RED_THREADS / 32];
+  __shared__ double sh[RED_THREADS / 16];
   double srz = 0.0, srr = 0.0, sbb = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
     const double ri = b[i] - q[i];
     const double zi = dinv ? ri * dinv[i] : ri;
     r[i] = ri;
-    z[i] = zi;
+    if (dinv) z[i] = zi;
     p[i] = zi;
     srz = fma(ri, zi, srz);
     srr = fma(ri, ri, srr);
     sbb = fma(b[i], b[i], sbb);
   }
   srz = block_sum(srz, sh);
-  srr = block_sum(srr, sh);
-  sbb = block_sum(sbb, sh);
+  block_sum2(srr, sbb, sh);
   if (threadIdx.x == 0) {
     part[blockIdx.x] = srz;
     part[RED_BLOCKS + blockIdx.x] = srr;
@@ -147,7 +175,7 @@ __global__ void k_cg_init(const double* __restrict__ b, const double* __restrict
 }
 
 __global__ void k_cg_init_fin(const double* __restrict__ part, int nb, CgState* st) {
-  __shared__ double sh[RED_THREADS / 32];
+  __shared__ double sh[RED_THREADS / 16];
   double v[3];
   for (int j = 0; j < 3; ++j) {
     v[j] = part_sum(part + j * RED_BLOCKS, nb, sh);
@@ -163,7 +191,7 @@ __global__ void k_cg_init_fin(const double* __restrict__ part, int nb, CgState* 
 
 // alpha = rz / (p, q): partials per block, the last block's sum
 __global__ void k_cg_dot(const double* p, const double* q, int64_t n, double* part, CgState* st) {
-  __shared__ double sh[RED_THREADS / 32];
+  __shared__ double sh[RED_THREADS / 16];
   pdl_wait_all();
   double s = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
@@ -189,8 +217,8 @@ __global__ void k_cg_dot(const double* p, const double* q, int64_t n, double* pa
 // x += alpha p; r -= alpha q; z = dinv r; beta from r.z, r.r (the last block)
 __global__ void k_cg_update(double* x, double* r, double* z, const double* p, const double* q,
                             const double* __restrict__ dinv, int64_t n, CgState* st,
-                            double* part) {
-  __shared__ double sh[RED_THREADS / 32];
+                            double* part, int* host_done) {
+  __shared__ double sh[RED_THREADS / 16];
   pdl_wait_all();
   const double al = st->alpha;
   double srz = 0.0, srr = 0.0;
@@ -199,21 +227,23 @@ __global__ void k_cg_update(double* x, double* r, double* z, const double* p, co
     const double pi = p[i], qi = q[i], xi = x[i], r0 = r[i];   // loads before the stores
     x[i] = fma(al, pi, xi);
     const double ri = fma(-al, qi, r0);
-    const double zi = dinv ? ri * dinv[i] : ri;
     r[i] = ri;
-    z[i] = zi;
-    srz = fma(ri, zi, srz);
     srr = fma(ri, ri, srr);
+    if (dinv) {
+      const double zi = ri * dinv[i];
+      z[i] = zi;
+      srz = fma(ri, zi, srz);
+    }
   }
-  srz = block_sum(srz, sh);
-  srr = block_sum(srr, sh);
+  if (dinv) block_sum2(srz, srr, sh);
+  else srz = srr = block_sum(srr, sh);
   if (threadIdx.x == 0) {
     part[blockIdx.x] = srz;
     part[RED_BLOCKS + blockIdx.x] = srr;
   }
   if (!last_block(&st->cnt[1])) return;
   double v[2];
-  for (int j = 0; j < 2; ++j) v[j] = part_sum(part + j * RED_BLOCKS, gridDim.x, sh);
+  part_sum2(part, gridDim.x, sh, v);
   if (threadIdx.x == 0) {
     if (st->done) {
       st->beta = 0.0;
@@ -227,6 +257,7 @@ __global__ void k_cg_update(double* x, double* r, double* z, const double* p, co
       st->rz = v[0];
       if (st->done) st->beta = 0.0;
     }
+    *host_done = st->done;
   }
 }
 
@@ -302,10 +333,6 @@ static inline int vec_grid(int64_t n) {
 void Workspace::release() {
   for (void* p : bufs) cudaFree(p);
   bufs.clear();
-  if (host_state) cudaFreeHost(host_state);
-  host_state = nullptr;
-  if (cap) cudaStreamDestroy(cap);
-  cap = nullptr;
 }
 
 cudaError_t Workspace::alloc(void** p, size_t bytes) {
@@ -331,51 +358,49 @@ static cudaError_t multi_dot(const T* a, int64_t lda, const T* b, int64_t n, int
 
 // ---- CG --------------------------------------------------------------------
 
+// Page-locked copy of the state, the iterations' outcomes and their events.
+struct CgHost {
+  static constexpr int kRing = CG_AHEAD + 1;
+  char* mem = nullptr;
+  cudaEvent_t ev[kRing] = {};
+  CgState* state() { return (CgState*)mem; }
+  int* done(int i) { return (int*)(mem + 256) + i; }
+  cudaError_t init() {
+    static_assert(sizeof(CgState) <= 256, "CgHost layout");
+    cudaError_t e = cudaMallocHost((void**)&mem, 256 + kRing * sizeof(int));
+    for (int i = 0; i < kRing && e == cudaSuccess; ++i)
+      e = cudaEventCreateWithFlags(&ev[i], cudaEventDisableTiming);
+    return e;
+  }
+  ~CgHost() {
+    for (cudaEvent_t v : ev)
+      if (v) cudaEventDestroy(v);
+    if (mem) cudaFreeHost(mem);
+  }
+};
+
 SolveStatus solve_cg(const ApplyFn<double>& apply, int64_t n, const double* b, double* x,
                      const double* diag, double rtol, int maxit, cudaStream_t st, Workspace& ws,
                      SolveInfo* info) {
-  double *r, *z, *p, *q, *dinv = nullptr, *part;
-  CgState* dst;
-  CK(ws.alloc((void**)&r, n * 8));
-  CK(ws.alloc((void**)&z, n * 8));
-  CK(ws.alloc((void**)&p, n * 8));
-  CK(ws.alloc((void**)&q, n * 8));
-  CK(ws.alloc((void**)&part, 3 * RED_BLOCKS * 8));
-  CK(ws.alloc((void**)&dst, sizeof(CgState)));
+  // one allocation: r, p, q [, z, 1 / diag], the partials and the state
+  const int nb = red_blocks(n);
+  const size_t vec = ((size_t)n * 8 + 255) / 256 * 256;
+  char* base;
+  CK(ws.alloc((void**)&base, vec * (diag ? 5 : 3) + 3 * RED_BLOCKS * 8 + sizeof(CgState)));
+  double* r = (double*)base;
+  double* p = (double*)(base + vec);
+  double* q = (double*)(base + 2 * vec);
+  double* z = diag ? (double*)(base + 3 * vec) : r;
+  double* dinv = diag ? (double*)(base + 4 * vec) : nullptr;
+  double* part = (double*)(base + vec * (diag ? 5 : 3));
+  CgState* dst = (CgState*)(part + 3 * RED_BLOCKS);
   if (diag) {
-    CK(ws.alloc((void**)&dinv, n * 8));
     k_reciprocal<<<vec_grid(n), 256, 0, st>>>(diag, dinv, n);
     CK(cudaGetLastError());
   }
-  if (!ws.host_state) CK(cudaMallocHost(&ws.host_state, 4096));
-  CgState* hs = (CgState*)ws.host_state;
-  if (!ws.cap) CK(cudaStreamCreateWithFlags(&ws.cap, cudaStreamNonBlocking));
-
-  const int nb = red_blocks(n);
-  // one chunk of CG iterations, captured once
-  cudaGraph_t graph;
-  cudaGraphExec_t exec;
-  CK(cudaStreamBeginCapture(ws.cap, cudaStreamCaptureModeThreadLocal));
-  for (int it = 0; it < CG_CHUNK; ++it) {
-    cudaError_t e = apply(p, q, ws.cap);
-    if (e != cudaSuccess) {
-      cudaStreamEndCapture(ws.cap, &graph);
-      return {SBM_ERR_CUDA, e};
-    }
-    const double *cp = p, *cq = q, *cz = z, *cd = dinv;
-    if ((e = launch_maybe_pdl(k_cg_dot, dim3(nb), dim3(RED_THREADS), 0, ws.cap, true, cp, cq, n,
-                              part, dst)) != cudaSuccess ||
-        (e = launch_maybe_pdl(k_cg_update, dim3(nb), dim3(RED_THREADS), 0, ws.cap, true, x, r, z,
-                              cp, cq, cd, n, dst, part)) != cudaSuccess ||
-        (e = launch_maybe_pdl(k_cg_p, dim3(vec_grid(n)), dim3(256), 0, ws.cap, true, p, cz, n,
-                              (const CgState*)dst)) != cudaSuccess) {
-      cudaStreamEndCapture(ws.cap, &graph);
-      return {SBM_ERR_CUDA, e};
-    }
-  }
-  CK(cudaStreamEndCapture(ws.cap, &graph));
-  CK(cudaGraphInstantiate(&exec, graph, 0));
-  cudaGraphDestroy(graph);
+  CgHost ch;
+  CK(ch.init());
+  CgState* hs = ch.state();
 
   int total = 0, restarts = 0, status = SBM_NOT_DONE;
   double relres = INFINITY;
@@ -390,14 +415,30 @@ SolveStatus solve_cg(const ApplyFn<double>& apply, int64_t n, const double* b, d
     k_cg_init<<<nb, RED_THREADS, 0, st>>>(b, q, r, z, p, dinv, n, part);
     k_cg_init_fin<<<1, RED_THREADS, 0, st>>>(part, nb, dst);
     CK(cudaGetLastError());
-    int done = 0;
-    while (true) {
-      CK(cudaMemcpyAsync(hs, dst, sizeof(CgState), cudaMemcpyDeviceToHost, st));
-      CK(cudaStreamSynchronize(st));
-      done = hs->done;
-      if (done || hs->maxit <= 0) break;
-      CK(cudaGraphLaunch(exec, st));
+    // the iterations, CG_AHEAD enqueued beyond the one whose outcome is read
+    // (those after the last one change nothing)
+    CK(cudaMemcpyAsync(hs, dst, sizeof(CgState), cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    const double *cp = p, *cq = q, *cz = z, *cd = dinv;
+    const int lim = hs->done ? 0 : init.maxit;
+    for (int it = 0, enq = 0; it < lim; ++it) {
+      for (; enq < lim && enq <= it + CG_AHEAD; ++enq) {
+        const int slot = enq % CgHost::kRing;
+        CK(apply(p, q, st));
+        CK(launch_maybe_pdl(k_cg_dot, dim3(nb), dim3(RED_THREADS), 0, st, true, cp, cq, n, part,
+                            dst));
+        CK(launch_maybe_pdl(k_cg_update, dim3(nb), dim3(RED_THREADS), 0, st, true, x, r, z, cp,
+                            cq, cd, n, dst, part, ch.done(slot)));
+        CK(cudaEventRecord(ch.ev[slot], st));
+        CK(launch_maybe_pdl(k_cg_p, dim3(vec_grid(n)), dim3(256), 0, st, true, p, cz, n,
+                            (const CgState*)dst));
+      }
+      CK(cudaEventSynchronize(ch.ev[it % CgHost::kRing]));
+      if (*ch.done(it % CgHost::kRing)) break;
     }
+    CK(cudaMemcpyAsync(hs, dst, sizeof(CgState), cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    const int done = hs->done;
     total += hs->iters;
     // true residual
     CK(apply(x, q, st));
@@ -414,7 +455,6 @@ SolveStatus solve_cg(const ApplyFn<double>& apply, int64_t n, const double* b, d
       break;
     }
   }
-  cudaGraphExecDestroy(exec);
   info->iters = total;
   info->relres = relres;
   info->restarts = restarts;
@@ -700,21 +740,24 @@ SolveStatus solve_gmres(const ApplyFn<T>& apply, int64_t n, const TX* b, TX* x, 
   static_assert(std::is_same<T, TX>::value, "rx is also the Arnoldi step's A U_j");
   // apply_x: operator in the precision of x/b for the outer residual (T == TX: same as apply)
   const int m = restart;
-  T* V;
-  TX* rx;
-  double *part, *dsc;
-  CK(ws.alloc((void**)&V, (size_t)(m + 1) * n * sizeof(T)));
-  CK(ws.alloc((void**)&rx, (size_t)n * sizeof(TX)));
-  CK(ws.alloc((void**)&part, (size_t)RED_BLOCKS * 8));
-  CK(ws.alloc((void**)&dsc, (m + 4) * 8));
+  // one allocation: the basis, A U_j / the outer residual, scalars, partials
   GmVecs g;
-  GmCtl* ctl;
-  CK(ws.alloc((void**)&g.s, (size_t)4 * (m + 1) * 8));
-  g.h1 = g.s + (m + 1);
-  g.h2 = g.h1 + (m + 1);
-  g.phi = g.h2 + (m + 1);
-  CK(ws.alloc((void**)&g.part, (size_t)(m + 1) * GM_MAXB * 8));
-  CK(ws.alloc((void**)&ctl, sizeof(GmCtl)));
+  const auto up = [](size_t v) { return (v + 255) / 256 * 256; };
+  const size_t bV = up((size_t)(m + 1) * n * sizeof(T)), br = up((size_t)n * sizeof(TX)),
+               bs = up((size_t)5 * (m + 4) * 8), bp = up((size_t)(m + 1) * GM_MAXB * 8),
+               bq = up((size_t)RED_BLOCKS * 8);
+  char* base;
+  CK(ws.alloc((void**)&base, bV + br + bs + bp + bq + sizeof(GmCtl)));
+  T* V = (T*)base;
+  TX* rx = (TX*)(base + bV);
+  double* dsc = (double*)(base + bV + br);
+  g.s = dsc + (m + 4);
+  g.h1 = g.s + (m + 4);
+  g.h2 = g.h1 + (m + 4);
+  g.phi = g.h2 + (m + 4);
+  g.part = (double*)(base + bV + br + bs);
+  double* part = (double*)(base + bV + br + bs + bp);
+  GmCtl* ctl = (GmCtl*)(base + bV + br + bs + bp + bq);
   GmHost gh;
   CK(gh.init(m));
   std::vector<double> y(m + 1), scale(m + 2);
@@ -826,7 +869,7 @@ template <typename T>
 __global__ void k_bi_init(const T* __restrict__ b, const T* __restrict__ q, T* __restrict__ r,
                           T* __restrict__ rh, T* __restrict__ p, int64_t n,
                           double* __restrict__ part) {
-  __shared__ double sh[RED_THREADS / 32];
+  __shared__ double sh[RED_THREADS / 16];
   double srr = 0.0, sbb = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -837,8 +880,7 @@ __global__ void k_bi_init(const T* __restrict__ b, const T* __restrict__ q, T* _
     srr = fma((double)ri, (double)ri, srr);
     sbb = fma((double)b[i], (double)b[i], sbb);
   }
-  srr = block_sum(srr, sh);
-  sbb = block_sum(sbb, sh);
+  block_sum2(srr, sbb, sh);
   if (threadIdx.x == 0) {
     part[blockIdx.x] = srr;
     part[RED_BLOCKS + blockIdx.x] = sbb;
@@ -846,11 +888,9 @@ __global__ void k_bi_init(const T* __restrict__ b, const T* __restrict__ q, T* _
 }
 
 __global__ void k_bi_init_fin(const double* __restrict__ part, int nb, BiState* st) {
-  __shared__ double sh[RED_THREADS / 32];
+  __shared__ double sh[RED_THREADS / 16];
   double v[2];
-  for (int j = 0; j < 2; ++j) {
-    v[j] = part_sum(part + j * RED_BLOCKS, nb, sh);
-  }
+  part_sum2(part, nb, sh, v);
   if (threadIdx.x == 0) {
     st->rr = v[0];
     st->bb = v[1];
@@ -866,7 +906,7 @@ __global__ void k_bi_init_fin(const double* __restrict__ part, int nb, BiState* 
 // alpha = rho / (r^, v)
 __global__ void k_bi_alpha(const double* __restrict__ part, int nb, BiState* st) {
   pdl_wait_all();
-  __shared__ double sh[RED_THREADS / 32];
+  __shared__ double sh[RED_THREADS / 16];
   if (st->done) return;
   const double s = part_sum(part, nb, sh);
   if (threadIdx.x == 0) {
@@ -892,7 +932,7 @@ template <typename T>
 __global__ void k_bi_dot2(const T* __restrict__ t, const T* __restrict__ s, int64_t n,
                           const BiState* st, double* __restrict__ part) {
   pdl_wait_all();
-  __shared__ double sh[RED_THREADS / 32];
+  __shared__ double sh[RED_THREADS / 16];
   if (st->done) return;
   double sts = 0.0, stt = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
@@ -901,8 +941,7 @@ __global__ void k_bi_dot2(const T* __restrict__ t, const T* __restrict__ s, int6
     sts = fma(ti, (double)s[i], sts);
     stt = fma(ti, ti, stt);
   }
-  sts = block_sum(sts, sh);
-  stt = block_sum(stt, sh);
+  block_sum2(sts, stt, sh);
   if (threadIdx.x == 0) {
     part[blockIdx.x] = sts;
     part[RED_BLOCKS + blockIdx.x] = stt;
@@ -912,12 +951,10 @@ __global__ void k_bi_dot2(const T* __restrict__ t, const T* __restrict__ s, int6
 // omega = (t, s) / (t, t)  (0 when t = 0: the update then keeps r = s)
 __global__ void k_bi_omega(const double* __restrict__ part, int nb, BiState* st) {
   pdl_wait_all();
-  __shared__ double sh[RED_THREADS / 32];
+  __shared__ double sh[RED_THREADS / 16];
   if (st->done) return;
   double v[2];
-  for (int j = 0; j < 2; ++j) {
-    v[j] = part_sum(part + j * RED_BLOCKS, nb, sh);
-  }
+  part_sum2(part, nb, sh, v);
   if (threadIdx.x == 0) {
     st->omega = (v[1] > 0.0) ? v[0] / v[1] : 0.0;
     if (!isfinite(st->omega)) st->done = 2;
@@ -931,7 +968,7 @@ __global__ void k_bi_update(T* __restrict__ x, T* __restrict__ r, const T* __res
                             const T* __restrict__ rh, int64_t n, const BiState* st,
                             double* __restrict__ part) {
   pdl_wait_all();
-  __shared__ double sh[RED_THREADS / 32];
+  __shared__ double sh[RED_THREADS / 16];
   if (st->done) return;
   const double al = st->alpha, om = st->omega;
   double srh = 0.0, srr = 0.0;
@@ -944,8 +981,7 @@ __global__ void k_bi_update(T* __restrict__ x, T* __restrict__ r, const T* __res
     srh = fma((double)rh[i], (double)ri, srh);
     srr = fma((double)ri, (double)ri, srr);
   }
-  srh = block_sum(srh, sh);
-  srr = block_sum(srr, sh);
+  block_sum2(srh, srr, sh);
   if (threadIdx.x == 0) {
     part[blockIdx.x] = srh;
     part[RED_BLOCKS + blockIdx.x] = srr;
@@ -955,12 +991,10 @@ __global__ void k_bi_update(T* __restrict__ x, T* __restrict__ r, const T* __res
 // rho' = (r^, r); convergence / breakdown tests; beta = (rho'/rho)(alpha/omega)
 __global__ void k_bi_beta(const double* __restrict__ part, int nb, BiState* st) {
   pdl_wait_all();
-  __shared__ double sh[RED_THREADS / 32];
+  __shared__ double sh[RED_THREADS / 16];
   if (st->done) return;
   double v[2];
-  for (int j = 0; j < 2; ++j) {
-    v[j] = part_sum(part + j * RED_BLOCKS, nb, sh);
-  }
+  part_sum2(part, nb, sh, v);
   if (threadIdx.x == 0) {
     st->iters += 1;
     st->rr = v[1];
@@ -981,7 +1015,7 @@ template <typename T>
 __global__ void k_bi_replace(const T* __restrict__ b, const T* __restrict__ q,
                              T* __restrict__ r, const T* __restrict__ rh, int64_t n,
                              double* __restrict__ part) {
-  __shared__ double sh[RED_THREADS / 32];
+  __shared__ double sh[RED_THREADS / 16];
   double srh = 0.0, srr = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -990,8 +1024,7 @@ __global__ void k_bi_replace(const T* __restrict__ b, const T* __restrict__ q,
     srh = fma((double)rh[i], (double)ri, srh);
     srr = fma((double)ri, (double)ri, srr);
   }
-  srh = block_sum(srh, sh);
-  srr = block_sum(srr, sh);
+  block_sum2(srh, srr, sh);
   if (threadIdx.x == 0) {
     part[blockIdx.x] = srh;
     part[RED_BLOCKS + blockIdx.x] = srr;
@@ -1000,12 +1033,10 @@ __global__ void k_bi_replace(const T* __restrict__ b, const T* __restrict__ q,
 
 // rho = (r^, r) and rr = (r, r) of the replaced residual; convergence test
 __global__ void k_bi_replace_fin(const double* __restrict__ part, int nb, BiState* st) {
-  __shared__ double sh[RED_THREADS / 32];
+  __shared__ double sh[RED_THREADS / 16];
   if (st->done) return;
   double v[2];
-  for (int j = 0; j < 2; ++j) {
-    v[j] = part_sum(part + j * RED_BLOCKS, nb, sh);
-  }
+  part_sum2(part, nb, sh, v);
   if (threadIdx.x == 0) {
     st->rr = v[1];
     st->rho = v[0];

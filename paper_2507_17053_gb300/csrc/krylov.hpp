@@ -31,8 +31,6 @@ struct SolveStatus {
 // Device scratch of one solve; released by the caller.
 struct Workspace {
   std::vector<void*> bufs;
-  void* host_state = nullptr;
-  cudaStream_t cap = nullptr;
   cudaError_t alloc(void** p, size_t bytes);
   void release();
 };
