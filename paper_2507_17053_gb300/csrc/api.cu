@@ -155,6 +155,7 @@ static void free_device(DeviceData* dd) {
   cudaFree(dd->fix_exp);
   cudaFree(dd->fix_tab);
   cudaFree(dd->nbr);
+  cudaFree(dd->dg_exp);
   cudaFree(dd->stage_x);
   cudaFree(dd->stage_y);
   for (cudaEvent_t ev : dd->ev_in)
@@ -325,6 +326,9 @@ static int build_device(const HostProblem& hp, DeviceData* dd) {
   }
   cudaError_t e;
   if ((e = upload(&dd->nbr, nbr.data(), nbr.size())) != cudaSuccess) goto err;
+  if (hp.desc.dg && d == 3 &&
+      (e = cudaMalloc((void**)&dd->dg_exp, (size_t)Nc * sizeof(int32_t))) != cudaSuccess)
+    goto err;
   if (d == 3 &&
       (e = upload(&dd->xfix, hp.fx.xline.data(), hp.fx.xline.size())) != cudaSuccess)
     goto err;

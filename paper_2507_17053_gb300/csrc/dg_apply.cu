@@ -1,43 +1,28 @@
 // Matrix-free apply (FP64 or FP32) of the SIPG discontinuous Galerkin SBM operator.
 //
-// Cell-centric: every block owns CPB cells and writes their DoFs once (a DG
-// cell's DoFs belong to it alone), so there is a single launch, no colouring
-// and no atomics.  Per cell: the cell term (Algorithm 1; 3D in the eigenbasis
-// of the 1D pencil, 2D by sweeps, as in the CG kernel), then its 2d faces in
-// the order (k, s):
+// Cell-centric: every block owns some cells and writes their DoFs once (a DG
+// cell's DoFs belong to it alone), so there is no colouring and there are no
+// atomics.  Each interior face is evaluated from both sides (twice the face
+// arithmetic, no write conflict), the neighbour's values read straight from
+// global memory; surrogate faces (Algorithm 3) are computed beforehand by the
+// face kernel and folded in here.
+//
+// 2D, per cell: the cell term (Algorithm 1), then its faces in the order (k, s):
 //  * interior face (neighbour active), Algorithm 2 from this cell's side:
 //      [u] = u_K1 - u_K2, {dn u} = (dn u_K1 + dn u_K2)/2 with n = +e_k, K1 the
 //      lower cell; the value test gets +T_v (K1) or -T_v (K2),
 //      T_v = sigma_F [u] - {dn u}, and the normal-derivative test -[u]/2;
-//    the neighbour's trace comes straight from global memory (each face is
-//    evaluated from both sides: twice the face arithmetic, no write conflict);
-//  * surrogate face: Algorithm 3, computed for all faces beforehand by the
-//    face kernel (face_kernel.cu) and folded in here from its scratch.
-// Interior-face arithmetic in nodal form: the face integrands are linear in
-// the nodal traces and the face quadrature is exact, so interpolation to the
-// Gauss points, weights and transposed interpolation collapse into the 1D
-// mass matrices: nodal traces -> pointwise combination -> (M x M) -> added to
-// the cell result.
-#include "sweeps.cuh"
+//  * surrogate face: added from the face kernel's scratch.
+// 3D: all terms of an axis as one operator per line (below).
+#include "chunk_body.cuh"
 
 namespace sbm {
 
-template <int D, int N>
-struct DgShape {
-  static constexpr int L = (D == 3) ? N * N : N;
-  static constexpr int ND = L * N;
-  static constexpr int CPB = (128 / L) > 0 ? (128 / L) : 1;
-};
-
-// The result tile A (3D FP32: the padded layout of TilePad, node (j0, j1, j2)
-// at j0 + PX j1 + PX n j2, cells NDP apart; FP64 (pipe-bound, registers
-// first) and 2D unpadded; 2D: the pair tile's two halves).
-template <typename T, int D, int N>
-struct DgTile {
-  static constexpr bool kPad = D == 3 && std::is_same<T, float>::value;
-  static constexpr int PX = kPad ? TilePad<T, N>::PX : N;
-  static constexpr int NDP = kPad ? TilePad<T, N>::NDP : (D == 3 ? 1 : 2) * DgShape<D, N>::ND;
-  static constexpr int elems = DgShape<D, N>::CPB * NDP;   // A, before the input tiles
+// 2D: lines of n nodes, cells per block
+template <int N>
+struct Dg2 {
+  static constexpr int ND = N * N;
+  static constexpr int CPB = 128 / N;
 };
 
 template <typename T>
@@ -47,27 +32,24 @@ struct DgArgs {
   const int32_t* __restrict__ cell_rank;   // ordered cell -> active-cell rank
   const int32_t* __restrict__ nbr;         // [rank][2k+s] neighbour rank or -1
   const int32_t* __restrict__ face_start;  // ordered cell -> surrogate-face range
+  const int32_t* __restrict__ face_kind;   // 3D
   const T* __restrict__ face_out;          // [F][2L] from the face kernel
+  const int32_t* __restrict__ cexp;        // 3D FP64: exponents of the cells
   int ncell;
   T sigma_f;
 };
 
-template <typename T, int D, int N>
-__global__ void __launch_bounds__(DgShape<D, N>::CPB * DgShape<D, N>::L)
+template <typename T, int N>
+__global__ void __launch_bounds__(Dg2<N>::CPB * N)
 dg_apply_kernel(const DgArgs<T> a, const __grid_constant__ KTab<T> t) {
-  constexpr int L = DgShape<D, N>::L, ND = DgShape<D, N>::ND, CPB = DgShape<D, N>::CPB;
+  constexpr int ND = Dg2<N>::ND, CPB = Dg2<N>::CPB;
   using Pair2 = typename PairOf<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  // 3D: a scalar sweep tile (the eigenbasis phases run in place and leave the
-  // cell results there); 2D: a pair tile for the sweeps, then the results
-  using DT = DgTile<T, D, N>;
-  T* A = reinterpret_cast<T*>(smem_raw);       // sweep tile, then the result tile
+  T* A = reinterpret_cast<T*>(smem_raw);       // pair tile of the sweeps, then the results
   Pair2* AE = reinterpret_cast<Pair2*>(smem_raw);
-  T* X = A + DT::elems;                        // CPB input tiles (unpadded)
-  T* U1 = X + CPB * ND;        // face scratch, CPB * L each
-  T* U2 = U1 + CPB * L;
-  T* P1 = U2 + CPB * L;
-  T* P2 = P1 + CPB * L;
+  T* X = A + 2 * CPB * ND;                     // CPB input tiles
+  T* P1 = X + CPB * ND;                        // face scratch, CPB * N each
+  T* P2 = P1 + CPB * N;
   const int tid = threadIdx.x;
   const int first = blockIdx.x * CPB;
   const int ncells = min(CPB, a.ncell - first);
@@ -76,72 +58,43 @@ dg_apply_kernel(const DgArgs<T> a, const __grid_constant__ KTab<T> t) {
     X[r] = __ldg(a.x + (size_t)__ldg(a.cell_rank + first + c) * ND + (r - c * ND));
   }
   __syncthreads();
-  const int c = tid / L, tl = tid - c * L;
+  const int c = tid / N, tl = tid - c * N;
   const bool act = c < ncells;
   const int pos = first + (act ? c : 0);
   const int rank = __ldg(a.cell_rank + pos);
   T* Xc = X + c * ND;
-  T* R = A + c * (D == 3 ? DT::NDP : ND);
+  T* R = A + c * ND;
   {
-    // cell term (Algorithm 1), then the line result into R (node (j0, j1, j2)
-    // at j0 + n j1 + n^2 j2): 3D the z-line tl, back to the nodes its last
-    // phase read; 2D the x-line tl, once every thread is past the sweeps
+    // cell term (Algorithm 1), then the x-line result into R once every
+    // thread is past the sweeps
     T out[N];
-    if constexpr (D == 3) {
-      const XLineOp<T, N> xop(t, tl % N, tl / N);
-      cell_fd_3d<T, N, DT::kPad>(t, X, c * ND + tl, N * N, A, c, tl, act, xop, out);
-      if (act) {
+    cell_sweeps_2d<T, N>(t, X, c * ND + tl, N, AE, c, tl, act, out);
+    __syncthreads();
+    if (act) {
 #pragma unroll
-        for (int m = 0; m < N; ++m)
-          R[DT::PX == N ? tl + N * N * m : tl % N + DT::PX * (tl / N + N * m)] = out[m];
-      }
-    } else {
-      cell_sweeps_2d<T, N>(t, X, c * ND + tl, N, AE, c, tl, act, out);
-      __syncthreads();
-      if (act) {
-#pragma unroll
-        for (int m = 0; m < N; ++m) R[N * tl + m] = out[m];
-      }
+      for (int m = 0; m < N; ++m) R[N * tl + m] = out[m];
     }
   }
   __syncthreads();
 
   int fptr = act ? __ldg(a.face_start + pos) : 0;   // next surrogate face of this cell
-  T* u1 = U1 + c * L;
-  T* u2 = U2 + c * L;
-  T* p1 = P1 + c * L;
-  T* p2 = P2 + c * L;
-  for (int k = 0; k < D; ++k) {
-    int sk, sa, sb;
-    if (D == 2) {
-      sk = (k == 0) ? 1 : N;
-      sa = (k == 0) ? N : 1;
-      sb = 0;
-    } else {
-      sk = (k == 0) ? 1 : (k == 1 ? N : N * N);
-      sa = (k == 0) ? N : 1;
-      sb = (k == 2) ? N : N * N;
-    }
-    const int bt = (tl % N) * sa + (D == 3 ? (tl / N) * sb : 0);
-    // the same strides in the result tile (3D FP32: padded)
-    int rk = sk, rbt = bt;
-    if constexpr (DT::PX != N) {
-      rk = (k == 0) ? 1 : (k == 1 ? DT::PX : DT::PX * N);
-      rbt = (tl % N) * ((k == 0) ? DT::PX : 1) + (tl / N) * ((k == 2) ? DT::PX : DT::PX * N);
-    }
+  T* p1 = P1 + c * N;
+  T* p2 = P2 + c * N;
+  for (int k = 0; k < 2; ++k) {
+    const int sk = (k == 0) ? 1 : N, bt = tl * ((k == 0) ? N : 1);
     for (int s = 0; s < 2; ++s) {
-      const int nb = act ? __ldg(a.nbr + (size_t)rank * 2 * D + 2 * k + s) : -1;
+      const int nb = act ? __ldg(a.nbr + (size_t)rank * 4 + 2 * k + s) : -1;
       const bool interior = nb >= 0;
       const int kend = s ? N - 1 : 0;
       const T sg = s ? T(1) : T(-1);
       const T* fo = nullptr;
-      if (act && !interior) fo = a.face_out + (size_t)(fptr++) * 2 * L;
+      if (act && !interior) fo = a.face_out + (size_t)(fptr++) * 2 * N;
       // A. nodal traces (own side and, for interior faces, the neighbour's),
       // and the two integrands in nodal form: with Gauss quadrature exact on
       // the face, interpolating to the Gauss points, weighting and
-      // interpolating back is h^(d-1) (M x M) (the exact 1D mass matrices), so
-      //   value test:  h^(d-1) (M x M) sg (sigma_F [u] - h^-1 {d_k u}),
-      //   normal-derivative test:  h^(d-1) (M x M) (-[u] / (2 h))
+      // interpolating back is h M (the exact 1D mass matrix), so
+      //   value test:  h M sg (sigma_F [u] - h^-1 {d_k u}),
+      //   normal-derivative test:  h M (-[u] / (2 h))
       if (act) {
         T um = Xc[kend * sk + bt], dm = T(0);
 #pragma unroll
@@ -163,71 +116,386 @@ dg_apply_kernel(const DgArgs<T> a, const __grid_constant__ KTab<T> t) {
         p2[tl] = a2;
       }
       __syncthreads();
-      // B. (M x M) on both integrands, the first axis, then the second
-      T rv = T(0), rg = T(0);
-      if (D == 3) {
-        if (act) {
-          const int ia = tl % N, jb = tl / N;
-          T v1 = T(0), v2 = T(0);
-#pragma unroll
-          for (int j = 0; j < N; ++j) {
-            v1 = fma(t.M[ia][j], p1[j + N * jb], v1);
-            v2 = fma(t.M[ia][j], p2[j + N * jb], v2);
-          }
-          u1[tl] = v1;
-          u2[tl] = v2;
-        }
-        __syncthreads();
-        if (act) {
-          const int ia = tl % N, ib = tl / N;
-#pragma unroll
-          for (int j = 0; j < N; ++j) {
-            rv = fma(t.M[ib][j], u1[ia + N * j], rv);
-            rg = fma(t.M[ib][j], u2[ia + N * j], rg);
-          }
-        }
-      } else {
-        if (act) {
-#pragma unroll
-          for (int j = 0; j < N; ++j) {
-            rv = fma(t.M[tl][j], p1[j], rv);
-            rg = fma(t.M[tl][j], p2[j], rg);
-          }
-        }
-      }
-      if (act && !interior) {           // surrogate face: results of the face kernel
-        rv = __ldg(fo + tl);
-        rg = __ldg(fo + L + tl);
-      }
+      // B. M on both integrands
       if (act) {
-        R[kend * rk + rbt] += rv;
+        T rv = T(0), rg = T(0);
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+          rv = fma(t.M[tl][j], p1[j], rv);
+          rg = fma(t.M[tl][j], p2[j], rg);
+        }
+        if (!interior) {                // surrogate face: results of the face kernel
+          rv = __ldg(fo + tl);
+          rg = __ldg(fo + N + tl);
+        }
+        R[kend * sk + bt] += rv;
 #pragma unroll
         for (int j = 0; j < N; ++j)
-          R[j * rk + rbt] = fma(s ? t.D1[j] : t.D0[j], rg, R[j * rk + rbt]);
+          R[j * sk + bt] = fma(s ? t.D1[j] : t.D0[j], rg, R[j * sk + bt]);
       }
       __syncthreads();
     }
   }
   for (int r = tid; r < ncells * ND; r += blockDim.x) {
-    const int cc = r / ND, q = r - cc * ND;
-    const int ar = DT::PX != N ? cc * DT::NDP + q % N + DT::PX * (q / N) : r;
-    a.y[(size_t)__ldg(a.cell_rank + first + cc) * ND + q] = A[ar];
+    const int cc = r / ND;
+    a.y[(size_t)__ldg(a.cell_rank + first + cc) * ND + (r - cc * ND)] = A[r];
   }
 }
 
-template <typename T, int D, int N>
-static cudaError_t dg_t(const HostProblem& hp, const DeviceData& dd, const T* x, T* y,
-                        cudaStream_t st, Profiler* prof, int face_mode) {
-  constexpr int L = DgShape<D, N>::L, ND = DgShape<D, N>::ND, CPB = DgShape<D, N>::CPB;
-  const KTab<T> t = make_ktab<T>(hp);
-  const size_t smem = (size_t)(DgTile<T, D, N>::elems + CPB * ND + 4 * CPB * L) * sizeof(T);
-  cudaError_t err;
-  if (smem > 48 * 1024) {
-    err = cudaFuncSetAttribute(dg_apply_kernel<T, D, N>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (err != cudaSuccess) return err;
+// ---- 3D ------------------------------------------------------------------------
+//
+// With exact quadrature the interior-face terms of axis k have the tensor
+// structure of the cell term, a 1D operator along k times the mass matrices
+// of the other two axes.  Per line along k, with g_s = u - (the neighbour's
+// line, mirrored in the face s):
+//   r_k = K u + sum_{s interior} Own_s g_s,
+//   Own_s = pen e_s e_s^T - 1/2 sg (e_s D_s^T + D_s e_s^T)
+// (the mirrored neighbour has the negative of the end derivative D_s, so jump
+// and mean of the normal derivative are both products of g_s), and
+//   y = h (M_z (M_y r_x + M_x r_y) + M_y M_x r_z) + surrogate faces.
+// Each face costs 2n products per line instead of 7n (its traces, two mass
+// products of the two integrands, the test functions); four line phases.
+//
+// FP64 runs on the integer units (fixed_point.cuh): the exponent of a cell is
+// the largest of its own and its neighbours', from dg_exp_kernel; r_k of
+// 57-bit values leaves at 59 bits, so that the sum of the last phase stays
+// below 2^61.
+//
+// Measured on GB300, whole applies, before (cell term, then six faces through
+// traces, mass products and folds) -> now: FP64 torus of 64^3 cells at p = 3
+// (1.57 M DoFs) 254 -> 61.5 us, FP32 35.3 -> 16.8 us.  FP64 is bound by the
+// integer pipes, FP32 by launch and load latency at this size.
+template <typename T>
+struct DgTabs;
+template <>
+struct DgTabs<double> {
+  fix::DgTab x;
+};
+template <>
+struct DgTabs<float> {
+  float w[kMaxN];                  // h w
+};
+
+template <typename T, int N>
+struct Dg3 {
+  static constexpr int L = N * N, ND = L * N;
+  static constexpr int R = 256 / L;                       // cells per block
+  static constexpr int NT = FixMap<N>::threads(R);
+  static constexpr int PX = TilePad<T, N>::PX, NDP = TilePad<T, N>::NDP, PL = PX * N;
+  static constexpr size_t smem = (size_t)4 * R * NDP * 8 / (8 / sizeof(T));
+};
+
+// FP32 lines: plain values
+template <typename T, int N>
+struct DgLine {
+  using V = T;
+  const KTab<T>& t;
+  const DgTabs<T>& d;
+  __device__ __forceinline__ V in(T x, int) const { return x; }
+  __device__ __forceinline__ void stiff(const V (&v)[N], V (&y)[N]) const {
+    line_apply<T, N>(t.Kh, t.fKh, v, y);
   }
-  DgArgs<T> a;
+  __device__ __forceinline__ void mass(const V (&v)[N], V (&y)[N]) const {
+    line_apply<T, N>(t.M, t.fM, v, y);
+  }
+  // y_s += w . g, the end value of g
+  template <int S>
+  __device__ __forceinline__ V side(const V (&v)[N], const V (&nb)[N], V (&y)[N]) const {
+    V r = T(0);
+#pragma unroll
+    for (int j = 0; j < N; ++j) r = fma(d.w[S ? N - 1 - j : j], v[j] - nb[N - 1 - j], r);
+    y[S ? N - 1 : 0] += r;
+    return S ? v[N - 1] - nb[0] : v[0] - nb[N - 1];
+  }
+  __device__ __forceinline__ void ends(V g0, V g1, V (&y)[N]) const {
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      if (j > 0) y[j] = fma(d.w[j], g0, y[j]);
+      if (j < N - 1) y[j] = fma(d.w[N - 1 - j], g1, y[j]);
+    }
+  }
+};
+
+// FP64 lines: fixed point
+template <int N>
+struct DgLine<double, N> {
+  using V = int64_t;
+  const KTab<double>& t;
+  const DgTabs<double>& d;
+  __device__ __forceinline__ V in(double x, int E) const {
+    const uint64_t b = (uint64_t)__double_as_longlong(x);
+    return (fix::plain_exp(E) ? fix::from_double<false>(b, E) : fix::from_double<true>(b, E)) >> 3;
+  }
+  __device__ __forceinline__ void stiff(const V (&v)[N], V (&y)[N]) const {
+    fix::apply_line<N, 3>([&](int i, int j) { return d.x.K.E[i][j]; },
+                          [&](int i, int j) { return d.x.K.O[i][j]; }, v, y);
+  }
+  __device__ __forceinline__ void mass(const V (&v)[N], V (&y)[N]) const {
+    fix::apply_line<N, 0>([&](int i, int j) { return d.x.M.E[i][j]; },
+                          [&](int i, int j) { return d.x.M.O[i][j]; }, v, y);
+  }
+  template <int S>
+  __device__ __forceinline__ V side(const V (&v)[N], const V (&nb)[N], V (&y)[N]) const {
+    fix::Split g[N];
+#pragma unroll
+    for (int j = 0; j < N; ++j) g[j] = fix::split(v[j] - nb[N - 1 - j]);
+    y[S ? N - 1 : 0] += fix::dot<3, N>([&](int j) { return d.x.w[S ? N - 1 - j : j]; }, g);
+    return S ? v[N - 1] - nb[0] : v[0] - nb[N - 1];
+  }
+  __device__ __forceinline__ void ends(V g0, V g1, V (&y)[N]) const {
+    const fix::Split s0 = fix::split(g0), s1 = fix::split(g1);
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      if (j == 0 || j == N - 1) {
+        const fix::Split q[1] = {j ? s0 : s1};
+        y[j] += fix::dot<3, 1>([&](int) { return d.x.w[N - 1]; }, q);
+      } else {
+        const fix::Split q[2] = {s0, s1};
+        y[j] += fix::dot<3, 2>([&](int i) { return d.x.w[i ? N - 1 - j : j]; }, q);
+      }
+    }
+  }
+};
+
+// r of one line: v the cell's values, nb0 / nb1 the neighbours' ranks (-1:
+// none), element j of the same line of a neighbour at its base + off + st j
+template <typename T, int N>
+__device__ __forceinline__ void dg_line(const DgLine<T, N>& A, const T* __restrict__ x, int nb0,
+                                        int nb1, int off, int st, int E,
+                                        const typename DgLine<T, N>::V (&v)[N],
+                                        typename DgLine<T, N>::V (&y)[N]) {
+  using V = typename DgLine<T, N>::V;
+  constexpr int ND = N * N * N;
+  T f[N];
+  V q[N], g0 = 0, g1 = 0;
+  if (nb0 >= 0) {
+#pragma unroll
+    for (int j = 0; j < N; ++j) f[j] = __ldg(x + (size_t)nb0 * ND + off + st * j);
+  }
+  A.stiff(v, y);
+  if (nb0 >= 0) {
+#pragma unroll
+    for (int j = 0; j < N; ++j) q[j] = A.in(f[j], E);
+    g0 = A.template side<0>(v, q, y);
+  }
+  if (nb1 >= 0) {
+#pragma unroll
+    for (int j = 0; j < N; ++j) q[j] = A.in(__ldg(x + (size_t)nb1 * ND + off + st * j), E);
+    g1 = A.template side<1>(v, q, y);
+  }
+  A.ends(g0, g1, y);
+}
+
+// exponent words (fixed_point.cuh) of the cells: groups of G lanes per cell
+template <int N>
+__global__ void __launch_bounds__(256)
+dg_exp_kernel(const double* __restrict__ x, int32_t* __restrict__ e, int ncell) {
+  constexpr int ND = N * N * N, G = ND < 32 ? 8 : 32;
+  pdl_trigger();
+  const int cell = (blockIdx.x * 256 + threadIdx.x) / G, l = threadIdx.x % G;
+  uint32_t m = 0u;
+  if (cell < ncell)
+#pragma unroll
+    for (int i = l; i < ND; i += G)
+      m = max(m, fix::mag_hi((uint64_t)__double_as_longlong(__ldg(x + (size_t)cell * ND + i))));
+#pragma unroll
+  for (int o = G / 2; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(~0u, m, o));
+  if (cell < ncell && l == 0) e[cell] = max(1, (int)(m >> 20));
+  pdl_wait();                      // done only after the face kernel: the next one waits for both
+}
+
+template <typename T, int N>
+__global__ void __launch_bounds__(Dg3<T, N>::NT, std::is_same<T, double>::value && N > 4 ? 3 : 4)
+dg3_kernel(const DgArgs<T> a, const __grid_constant__ KTab<T> t,
+           const __grid_constant__ DgTabs<T> d) {
+  using Sh = Dg3<T, N>;
+  using Line = DgLine<T, N>;
+  using V = typename Line::V;
+  constexpr bool FX = std::is_same<T, double>::value;
+  constexpr int L = Sh::L, ND = Sh::ND, PX = Sh::PX, PL = Sh::PL;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int tid = threadIdx.x;
+  int c, tl;
+  FixMap<N>::of(tid, c, tl);
+  const int first = blockIdx.x * Sh::R;
+  const bool act = c < min(Sh::R, a.ncell - first);
+  V* const U = reinterpret_cast<V*>(smem_raw) + (act ? c : 0) * Sh::NDP;
+  V* const X = U + Sh::R * Sh::NDP;
+  V* const Y = X + Sh::R * Sh::NDP;
+  V* const Z = Y + Sh::R * Sh::NDP;
+  const int la = tl % N, lb = tl / N;
+  const int zl = la + PX * lb, yl = la + PL * lb, xl = PX * tl;   // first nodes of the lines
+  const Line A{t, d};
+  int rank = 0, E = 1;
+  int nb[6] = {-1, -1, -1, -1, -1, -1};
+  V v[N], y[N];
+  if (act) {
+    rank = __ldg(a.cell_rank + first + c);
+    const int2* pn = reinterpret_cast<const int2*>(a.nbr + (size_t)rank * 6);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const int2 p = __ldg(pn + k);
+      nb[2 * k] = p.x;
+      nb[2 * k + 1] = p.y;
+    }
+    T u[N];
+#pragma unroll
+    for (int j = 0; j < N; ++j) u[j] = __ldg(a.x + (size_t)rank * ND + tl + L * j);
+    if constexpr (FX) {
+      pdl_wait();                  // the exponents
+      E = __ldcg(a.cexp + rank);
+#pragma unroll
+      for (int k = 0; k < 6; ++k)
+        if (nb[k] >= 0) E = max(E, __ldcg(a.cexp + nb[k]));
+    }
+#pragma unroll
+    for (int j = 0; j < N; ++j) U[zl + PL * j] = v[j] = A.in(u[j], E);
+    dg_line<T, N>(A, a.x, nb[4], nb[5], tl, L, E, v, y);
+#pragma unroll
+    for (int j = 0; j < N; ++j) Z[zl + PL * j] = y[j];
+  }
+  FixMap<N>::sync(tid);
+  if (act) {
+#pragma unroll
+    for (int j = 0; j < N; ++j) v[j] = U[yl + PX * j];
+    dg_line<T, N>(A, a.x, nb[2], nb[3], la + L * lb, N, E, v, y);
+#pragma unroll
+    for (int j = 0; j < N; ++j) Y[yl + PX * j] = y[j];
+#pragma unroll
+    for (int j = 0; j < N; ++j) v[j] = U[xl + j];
+    dg_line<T, N>(A, a.x, nb[0], nb[1], N * tl, 1, E, v, y);
+#pragma unroll
+    for (int j = 0; j < N; ++j) X[xl + j] = y[j];
+  }
+  FixMap<N>::sync(tid);
+  if (act) {                       // y-lines: M_y r_x, M_y r_z
+#pragma unroll
+    for (int j = 0; j < N; ++j) v[j] = X[yl + PX * j];
+    A.mass(v, y);
+#pragma unroll
+    for (int j = 0; j < N; ++j) X[yl + PX * j] = y[j];
+#pragma unroll
+    for (int j = 0; j < N; ++j) v[j] = Z[yl + PX * j];
+    A.mass(v, y);
+#pragma unroll
+    for (int j = 0; j < N; ++j) Z[yl + PX * j] = y[j];
+  }
+  FixMap<N>::sync(tid);
+  if (act) {                       // x-lines: M_y r_x + M_x r_y, M_x M_y r_z
+#pragma unroll
+    for (int j = 0; j < N; ++j) v[j] = Y[xl + j];
+    A.mass(v, y);
+#pragma unroll
+    for (int j = 0; j < N; ++j) X[xl + j] += y[j];
+#pragma unroll
+    for (int j = 0; j < N; ++j) v[j] = Z[xl + j];
+    A.mass(v, y);
+#pragma unroll
+    for (int j = 0; j < N; ++j) Z[xl + j] = y[j];
+  }
+  FixMap<N>::sync(tid);
+  if (!act) return;
+  T out[N];                        // z-lines, back to the nodes read first
+#pragma unroll
+  for (int j = 0; j < N; ++j) v[j] = X[zl + PL * j];
+  A.mass(v, y);
+#pragma unroll
+  for (int j = 0; j < N; ++j) y[j] += Z[zl + PL * j];
+  if constexpr (FX) {
+    const int eo = d.x.eoff;
+    const bool bad = E == fix::kExpBad || eo == fix::kFaceExpBad;
+    const bool plain = fix::plain_exp(E) && abs(eo) <= 64;
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      const uint64_t b = plain ? fix::to_double<false>(y[j], E + eo)
+                               : (bad ? 0x7ff8000000000000ull : fix::to_double<true>(y[j], E + eo));
+      out[j] = __longlong_as_double((long long)b);
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < N; ++j) out[j] = y[j];
+  }
+  const int fs = __ldg(a.face_start + first + c), fe = __ldg(a.face_start + first + c + 1);
+  if (!FX && fs < fe) pdl_wait();  // the face kernel's results
+  for (int f = fs; f < fe; ++f) {
+    const int kind = __ldg(a.face_kind + f);
+    fold_face_z<T, N, true>(t, a.face_out + (size_t)f * 2 * L, kind & 3, kind >> 2, la, lb, out);
+  }
+#pragma unroll
+  for (int j = 0; j < N; ++j) a.y[(size_t)rank * ND + tl + L * j] = out[j];
+}
+
+static DgTabs<double> dg_tabs(const HostProblem& hp, double) { return DgTabs<double>{hp.fx.dg}; }
+static DgTabs<float> dg_tabs(const HostProblem& hp, float) {
+  DgTabs<float> d = {};
+  for (int j = 0; j < hp.n; ++j)
+    d.w[j] = (float)(hp.h * (j ? 0.5 * hp.tab.D0[j] : hp.sigma_f * hp.h + hp.tab.D0[0]));
+  return d;
+}
+
+template <typename T, int N>
+static cudaError_t dg3_t(const HostProblem& hp, const DeviceData& dd, const T* x, T* y,
+                         cudaStream_t st, Profiler* prof, int face_mode) {
+  using Sh = Dg3<T, N>;
+  constexpr bool FX = std::is_same<T, double>::value;
+  static cudaError_t attr =
+      Sh::smem > 48 * 1024
+          ? cudaFuncSetAttribute(dg3_kernel<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)Sh::smem)
+          : cudaSuccess;
+  if (attr != cudaSuccess) return attr;
+  DgArgs<T> a = {};
+  a.x = x;
+  a.y = y;
+  a.cell_rank = dd.cell_rank;
+  a.nbr = dd.nbr;
+  a.face_start = dd.face_start;
+  a.face_kind = dd.face_kind;
+  a.face_out = face_out_of<T>(dd);
+  a.cexp = dd.dg_exp;
+  a.ncell = dd.col_start[dd.ncolours];
+  if (a.ncell == 0) return cudaSuccess;
+  const bool pr = prof && prof->on;
+  cudaError_t err;
+  if (pr && (err = prof->mark(st)) != cudaSuccess) return err;
+  int nlaunch = 1;
+  bool pdl = false;
+  if (dd.nface > 0) {
+    if ((err = launch_faces<T>(hp, dd, x, face_out_of<T>(dd), face_mode, st)) != cudaSuccess)
+      return err;
+    nlaunch++;
+    pdl = !pr && face_mode == 0;
+  }
+  if (pr && (err = prof->mark(st)) != cudaSuccess) return err;
+  if constexpr (FX) {
+    constexpr int G = Sh::ND < 32 ? 8 : 32;
+    const unsigned gb = (unsigned)(((int64_t)a.ncell * G + 255) / 256);
+    if ((err = launch_maybe_pdl(dg_exp_kernel<N>, dim3(gb), dim3(256), 0, st, pdl, x, dd.dg_exp,
+                                a.ncell)) != cudaSuccess)
+      return err;
+    nlaunch++;
+    pdl = !pr;
+  }
+  const unsigned grid = (unsigned)((a.ncell + Sh::R - 1) / Sh::R);
+  if ((err = launch_maybe_pdl(dg3_kernel<T, N>, dim3(grid), dim3(Sh::NT), Sh::smem, st, pdl, a,
+                              make_ktab<T>(hp), dg_tabs(hp, T(0)))) != cudaSuccess)
+    return err;
+  if (pr) {
+    prof->count(nlaunch);
+    if ((err = prof->mark(st)) != cudaSuccess) return err;   // cell phase ends
+    return prof->mark(st);                                   // no assembly phase
+  }
+  return cudaSuccess;
+}
+
+template <typename T, int N>
+static cudaError_t dg2_t(const HostProblem& hp, const DeviceData& dd, const T* x, T* y,
+                         cudaStream_t st, Profiler* prof, int face_mode) {
+  constexpr int ND = Dg2<N>::ND, CPB = Dg2<N>::CPB;
+  constexpr size_t smem = (size_t)(3 * CPB * ND + 2 * CPB * N) * sizeof(T);
+  static_assert(smem <= 48 * 1024, "2D DG block");
+  cudaError_t err;
+  DgArgs<T> a = {};
   a.x = x;
   a.y = y;
   a.cell_rank = dd.cell_rank;
@@ -245,8 +513,7 @@ static cudaError_t dg_t(const HostProblem& hp, const DeviceData& dd, const T* x,
     nlaunch++;
   }
   if (pr && (err = prof->mark(st)) != cudaSuccess) return err;
-  const int grid = (a.ncell + CPB - 1) / CPB;
-  dg_apply_kernel<T, D, N><<<grid, CPB * L, smem, st>>>(a, t);
+  dg_apply_kernel<T, N><<<(a.ncell + CPB - 1) / CPB, CPB * N, smem, st>>>(a, make_ktab<T>(hp));
   if ((err = cudaGetLastError()) != cudaSuccess) return err;
   if (pr) {
     prof->count(nlaunch);
@@ -259,10 +526,11 @@ static cudaError_t dg_t(const HostProblem& hp, const DeviceData& dd, const T* x,
 template <typename T>
 cudaError_t launch_dg_apply(const HostProblem& hp, const DeviceData& dd, const T* x, T* y,
                             cudaStream_t st, Profiler* prof, int face_mode) {
-#define SBM_CASE(DD, NN) \
-  if (hp.d == DD && hp.n == NN) return dg_t<T, DD, NN>(hp, dd, x, y, st, prof, face_mode);
-  SBM_CASE(2, 2) SBM_CASE(2, 3) SBM_CASE(2, 4) SBM_CASE(2, 5) SBM_CASE(2, 6) SBM_CASE(2, 7)
-  SBM_CASE(3, 2) SBM_CASE(3, 3) SBM_CASE(3, 4) SBM_CASE(3, 5) SBM_CASE(3, 6) SBM_CASE(3, 7)
+#define SBM_CASE(NN)                                                                     \
+  if (hp.n == NN)                                                                        \
+    return hp.d == 2 ? dg2_t<T, NN>(hp, dd, x, y, st, prof, face_mode)                   \
+                     : dg3_t<T, NN>(hp, dd, x, y, st, prof, face_mode);
+  SBM_CASE(2) SBM_CASE(3) SBM_CASE(4) SBM_CASE(5) SBM_CASE(6) SBM_CASE(7)
 #undef SBM_CASE
   return cudaErrorInvalidValue;
 }

@@ -58,6 +58,15 @@ struct Block {
   Entry O[kMaxHalf][kMaxHalf];
 };
 
+// Line operators of the 3D DG apply (dg_apply.cu): K and M folded, and the
+// interior-face vector w (w[0] = pen + D0[0], w[j] = D0[j] / 2); the result's
+// exponent word is E + eoff (kFaceExpBad: a non-finite penalty).
+struct DgTab {
+  Block K, M;
+  Entry w[2 * kMaxHalf];
+  int eoff;
+};
+
 // a value split for the products
 struct alignas(8) Split {
   int32_t h, l;                      // q = h 2^31 + l, 0 <= l < 2^31

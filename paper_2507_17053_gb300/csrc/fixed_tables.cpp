@@ -206,7 +206,7 @@ fix::Entry entry(const DD& A, int t) {
 
 }  // namespace
 
-bool build_fixed_tables(const Tables1D& tb, double scale, FixedTables* out) {
+bool build_fixed_tables(const Tables1D& tb, double scale, FixedTables* out, double pen) {
   const int n = tb.n, H = n / 2, HE = (n + 1) / 2;
   Pencil P;
   P.n = n;
@@ -347,6 +347,38 @@ bool build_fixed_tables(const Tables1D& tb, double scale, FixedTables* out) {
     for (int j = 0; j < n; ++j) out->face.push_back(entry(P.S[q][j], tS));
   out->face_eq = 2 + 2 * (61 - tS);
   out->face_etm = 2 - tD + 2 * (61 - tM);
+  // DG line operators: row i of K u + sum_s Own_s g_s, |g| <= 2 |u|, scaled to
+  // leave 57-bit values at 59 bits (K = 3); hm goes into the entries
+  DD w[kMaxN];
+  for (int j = 0; j < n; ++j) w[j] = j ? P.D0[j] * DD(0.5) : DD(pen) + P.D0[0];
+  double sw = 0.0, B1 = 0.0;
+  for (int j = 0; j < n; ++j) sw += mag(w[j]);
+  for (int i = 0; i < n; ++i) {
+    double r = 0.0;
+    for (int j = 0; j < n; ++j) r += mag(P.K[i][j]);
+    r += 2.0 * (i == 0 ? sw : mag(w[i]));
+    r += 2.0 * (i == n - 1 ? sw : mag(w[n - 1 - i]));
+    B1 = std::max(B1, r);
+  }
+  out->dg = fix::DgTab{};
+  if (!std::isfinite(B1)) {
+    out->dg.eoff = fix::kFaceExpBad;
+    return true;
+  }
+  const int tR = fit(B1) - 1;
+  auto folded = [&](const DD (&A)[kMaxN][kMaxN], int t, double f, fix::Block* o) {
+    for (int i = 0; i < HE; ++i)
+      for (int j = 0; j < HE; ++j) {
+        const bool mid = (n & 1) && j == H;
+        const DD e = mid ? A[i][j] : (A[i][j] + A[i][n - 1 - j]) * DD(0.5);
+        o->E[i][j] = entry(e * DD(f), t);
+        if (i < H && j < H) o->O[i][j] = entry((A[i][j] - A[i][n - 1 - j]) * DD(0.5) * DD(f), t);
+      }
+  };
+  folded(P.K, tR, hm, &out->dg.K);
+  folded(P.M, tM, 1.0, &out->dg.M);
+  for (int j = 0; j < n; ++j) out->dg.w[j] = entry(w[j] * DD(hm), tR);
+  out->dg.eoff = 2 - tR + 2 * (61 - tM) + eh;
   return true;
 }
 

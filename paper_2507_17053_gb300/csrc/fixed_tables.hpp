@@ -18,10 +18,12 @@ struct FixedTables {
   // matrix, phi_j at the Gauss points), the result exponents of q and tm
   std::vector<fix::Entry> face;
   int face_eq = 0, face_etm = 0;
+  fix::DgTab dg;                     // discontinuous Galerkin line operators (dg_apply.cu)
 };
 
 // Tables of the pencil of t for the cell operator scaled by scale = h^(d-2);
-// false if a bound the arithmetic relies on does not hold.
-bool build_fixed_tables(const Tables1D& t, double scale, FixedTables* out);
+// false if a bound the arithmetic relies on does not hold.  pen: h times the
+// interior-face penalty (DG).
+bool build_fixed_tables(const Tables1D& t, double scale, FixedTables* out, double pen = 0.0);
 
 }  // namespace sbm

@@ -168,6 +168,7 @@ struct DeviceData {
   int32_t* fix_exp = nullptr;
   fix::Entry* fix_tab = nullptr;
   int32_t* nbr = nullptr;        // DG [Nc * 2d] neighbour rank per (k, s), -1 = surrogate
+  int32_t* dg_exp = nullptr;     // 3D DG, FP64: [Nc] largest exponent of each cell (scratch)
   double* stage_x = nullptr;     // host-apply staging buffers (allocated on first use)
   double* stage_y = nullptr;
   // CG: the pipelined host-buffer apply cuts the cells into nslab slabs of

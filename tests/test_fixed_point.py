@@ -212,8 +212,76 @@ int faces() {
   return bad;
 }
 
+// The DG line operator K u + sum_s Own_s g_s at its bounds (57-bit values, every row's signs;
+// overflow stops the program): below 2^59, and right against long double.
+template <int N>
+int dg_lines(double pen) {
+  constexpr int H = N / 2;
+  int bad = 0;
+  Tables1D tb;
+  build_tables(N - 1, &tb);
+  FixedTables ft;
+  if (!build_fixed_tables(tb, 1.0, &ft, pen)) return 1;
+  const fix::DgTab& d = ft.dg;
+  auto Kf = [&](int i, int j) {           // the row's sign pattern from the folded blocks
+    const fix::Entry e = d.K.E[std::min(i, N - 1 - i)][std::min(j, N - 1 - j)];
+    if ((N & 1) && (i == H || j == H)) return (double)e.h;
+    const fix::Entry o = d.K.O[std::min(i, N - 1 - i)][std::min(j, N - 1 - j)];
+    return ((i < N - 1 - i) == (j < N - 1 - j)) ? (double)e.h + o.h : (double)e.h - o.h;
+  };
+  const int64_t B = (1ll << 57) - 1;
+  // eoff = 2 - tR + 2 (61 - tM) (h = 1); tM from an entry of the face tables
+  const fix::Entry m = ft.face[N];
+  const int tM = (int)std::lround(std::log2(((double)m.h * 0x1p30 + 0.5 * m.l) / tb.M[0][0]));
+  const int tR = 2 + 2 * (61 - tM) - d.eoff;
+  for (int row = 0; row < N; ++row) {
+    int64_t v[N], y[N], g[2][N], nb[2][N];
+    for (int j = 0; j < N; ++j) v[j] = Kf(row, j) < 0 ? -B : B;
+    for (int s = 0; s < 2; ++s)
+      for (int j = 0; j < N; ++j) nb[s][N - 1 - j] = (row + j + s) % 3 == 2 ? v[j] : -v[j];
+    fix::apply_line<N, 3>([&](int i, int j) { return d.K.E[i][j]; },
+                          [&](int i, int j) { return d.K.O[i][j]; }, v, y);
+    for (int s = 0; s < 2; ++s) {
+      fix::Split q[N];
+      for (int j = 0; j < N; ++j) {
+        g[s][j] = v[j] - nb[s][N - 1 - j];
+        q[j] = fix::split(g[s][j]);
+      }
+      y[s ? N - 1 : 0] += fix::dot<3, N>([&](int j) { return d.w[s ? N - 1 - j : j]; }, q);
+    }
+    const fix::Split e0 = fix::split(g[0][0]), e1 = fix::split(g[1][N - 1]);
+    for (int j = 0; j < N; ++j) {
+      const fix::Split q1[1] = {j ? e0 : e1}, q2[2] = {e0, e1};
+      if (j == 0 || j == N - 1) y[j] += fix::dot<3, 1>([&](int) { return d.w[N - 1]; }, q1);
+      else y[j] += fix::dot<3, 2>([&](int i) { return d.w[i ? N - 1 - j : j]; }, q2);
+    }
+    for (int i = 0; i < N; ++i) {
+      long double r = 0;
+      for (int j = 0; j < N; ++j) r += (long double)tb.K[i][j] * v[j];
+      for (int s = 0; s < 2; ++s) {
+        const int e = s ? N - 1 : 0;
+        const long double sg = s ? 1 : -1;
+        auto D = [&](int j) { return (long double)(s ? tb.D1[j] : tb.D0[j]); };
+        long double dg = 0;
+        for (int j = 0; j < N; ++j) dg += D(j) * g[s][j];
+        if (i == e) r += pen * g[s][e] - 0.5L * sg * dg;
+        r -= 0.5L * sg * D(i) * g[s][e];
+      }
+      // the double tables' rounding (16 N ulps of the terms, whose sum is below 2^59)
+      bad |= std::llabs(y[i]) > (1ll << 59);
+      if (std::fabs((long double)y[i] - std::ldexp(r, tR - 58)) > 16.0L * N * 0x1p6L) bad = 1;
+    }
+  }
+  if (bad) std::printf("dg n=%d pen %g\n", N, pen);
+  return bad;
+}
+
 int main() {
   int bad = conversions();
+  for (double pen : {1.0, 49.0, 1e6}) {
+    bad |= dg_lines<2>(pen) | dg_lines<3>(pen) | dg_lines<4>(pen) | dg_lines<5>(pen) |
+           dg_lines<6>(pen) | dg_lines<7>(pen);
+  }
   bad |= faces<2>() | faces<3>() | faces<4>() | faces<5>() | faces<6>() | faces<7>();
   for (double h : {2.0, 2.0 / 3, 2.0 / 96, 2.0 / 1000}) {
     bad |= cell<2>(h) | cell<3>(h) | cell<4>(h) | cell<5>(h) | cell<6>(h) | cell<7>(h);
