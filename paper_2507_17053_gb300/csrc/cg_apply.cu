@@ -238,7 +238,7 @@ static cudaError_t apply_r(const HostProblem& hp, const DeviceData& dd, const Ch
                          : launch_face_kernel<T>(hp, dd, x, fo, st, part.f0, part.f1);
     if (err != cudaSuccess) return err;
     nlaunch++;
-    pdl_cell = allow_pdl && !pr && face_mode == 0;
+    pdl_cell = allow_pdl && !pr;
   }
   if (pr && (err = prof->mark(st)) != cudaSuccess) return err;
   int cap = 0;

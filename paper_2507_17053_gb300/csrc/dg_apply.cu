@@ -464,7 +464,7 @@ static cudaError_t dg3_t(const HostProblem& hp, const DeviceData& dd, const T* x
     if ((err = launch_faces<T>(hp, dd, x, face_out_of<T>(dd), face_mode, st)) != cudaSuccess)
       return err;
     nlaunch++;
-    pdl = !pr && face_mode == 0;
+    pdl = !pr;
   }
   if (pr && (err = prof->mark(st)) != cudaSuccess) return err;
   if constexpr (FX) {
