@@ -238,9 +238,10 @@ bool build_fixed_tables(const Tables1D& tb, double scale, FixedTables* out, doub
         for (int j = 0; j < n; ++j) s += mag(X(a, b, i, j));
         B3 = std::max(B3, s * r[a] * r[b]);
       }
+  // (mirrored rows have equal sums)
   for (int b = 0; b < n; ++b)
-    for (int i = 0; i < n; ++i)
-      for (int y = 0; y < n; ++y) {
+    for (int i = 0; i < HE; ++i)
+      for (int y = 0; y < HE; ++y) {
         double s = 0.0;
         for (int j = 0; j < n; ++j)
           for (int yy = 0; yy < n; ++yy) {
@@ -250,9 +251,9 @@ bool build_fixed_tables(const Tables1D& tb, double scale, FixedTables* out, doub
           }
         B4 = std::max(B4, s * r[b]);
       }
-  for (int i = 0; i < n; ++i)
-    for (int y = 0; y < n; ++y)
-      for (int z = 0; z < n; ++z) {
+  for (int i = 0; i < HE; ++i)
+    for (int y = i; y < HE; ++y)
+      for (int z = y; z < HE; ++z) {   // and the axes can be exchanged
         double s = 0.0;
         for (int j = 0; j < n; ++j)
           for (int yy = 0; yy < n; ++yy)
