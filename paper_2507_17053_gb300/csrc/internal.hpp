@@ -63,11 +63,21 @@ struct KTab : KTabFix<T> {
 template <typename T>
 KTab<T> make_ktab(const HostProblem& hp);
 
-constexpr int kMaxSlabs = 16;   // slabs of the pipelined host-buffer apply, at most
-// Their cumulative shares of the cells: small first and last slabs (the copy
-// of x before the first kernel, the copy of y after the last one), large
-// ones between (full launches).
-constexpr double kSlabCuts[] = {0.04, 0.16, 0.40, 0.64, 0.84, 0.96};
+// Slabs of the pipelined host-buffer apply: about 1.2 sqrt(MB of a vector), 8
+// at most, the first and the last one half as large (the copy of x before the
+// first kernel, the copy of y after the last one).  More slabs start the copies
+// of y earlier, each costs three launches and a partly filled last wave.
+// Measured (us): 86 MB 6 slabs 725, 8 703, 11 714, 15 744; 26 MB 6 277, 8 295;
+// 6.4 MB 1 slab 137, 3 115, 6 137.
+constexpr int kMaxSlabs = 8;
+inline int slab_count(int64_t n_dofs) {
+  const double mb = n_dofs * 8e-6;
+  int k = 1;
+  while (k < kMaxSlabs && (k + 1) * (k + 1) <= 1.44 * mb) ++k;
+  return k;
+}
+// share of the cells below cut k = 1 .. count - 1
+inline double slab_cut(int k, int count) { return (k - 0.5) / (count - 1); }
 
 // CG chunking: runs of up to R consecutive active cells of one x-row.
 struct ChunkTable {
