@@ -154,6 +154,7 @@ static void free_device(DeviceData* dd) {
   cudaFree(dd->fix_p0);
   cudaFree(dd->fix_exp);
   cudaFree(dd->fix_tab);
+  cudaFree(dd->face_tab32);
   cudaFree(dd->nbr);
   cudaFree(dd->dg_exp);
   cudaFree(dd->stage_x);
@@ -387,6 +388,14 @@ static int build_device(const HostProblem& hp, DeviceData* dd) {
       goto err;
   }
   if ((e = device_face_phi(hp, fsrc, &dd->face_phi, &dd->face_phi32)) != cudaSuccess) goto err;
+  if (d == 3 && hp.desc.extension == SBM_EXT_EXACT) {
+    const KTab<float> t = make_ktab<float>(hp);
+    std::vector<float> tab;
+    for (int i = 0; i < n; ++i) tab.insert(tab.end(), t.M[i], t.M[i] + n);
+    for (int i = 0; i < n; ++i) tab.insert(tab.end(), t.S[i], t.S[i] + n);
+    tab.insert(tab.end(), t.W, t.W + L);
+    if ((e = upload(&dd->face_tab32, tab.data(), tab.size())) != cudaSuccess) goto err;
+  }
   if (d == 3 && hp.desc.extension == SBM_EXT_EXACT &&
       ((e = device_face_fix((int64_t)fsrc.size(), L, n, dd->face_phi, make_ktab<double>(hp).W,
                             &dd->fix_pp, &dd->fix_p0, &dd->fix_exp)) != cudaSuccess ||

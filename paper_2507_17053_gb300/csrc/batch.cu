@@ -317,6 +317,7 @@ void make_table(const sbm_batch* B, const LaunchPlan& L, const T* const* x, T* c
     q.fa.face_kind = dd.face_kind;
     q.fa.face_phi = face_phi_of<T>(dd);
     q.fa.fix = face_fix_of(p->hp, dd);
+    q.fa.tab32 = dd.face_tab32;
     q.fa.out = fo;
     q.fa.face0 = 0;
     q.fa.nface = dd.nface;

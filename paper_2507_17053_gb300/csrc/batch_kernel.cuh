@@ -139,6 +139,7 @@ __device__ SBM_BK_ITEM void face_item(const Prob<T>& P, const KTab<T>& tu, const
     for (int f0 = it.b; f0 < it.e; f0 += FPB)
       face_group_fix<N, FPB>(P.fa, *P.kt, bk_smem, f0, it.e, rhs);
   } else {
+    face_begin<T, D, N, EXT, FPB>(P.fa, bk_smem);
     for (int f0 = it.b; f0 < it.e; f0 += FPB)
       face_group<T, D, N, EXT, FPB>(P.fa, tu, *P.kt, bk_smem, f0, it.e, rhs);
   }

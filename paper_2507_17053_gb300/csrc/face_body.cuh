@@ -36,6 +36,7 @@ struct FaceArgs {
   const int32_t* __restrict__ face_kind;   // k | (s << 2)
   const T* __restrict__ face_phi;          // [F][L][D][N], or the shifts [F][L][D] (Taylor)
   FaceFix fix;                             // 3D exact, FP64
+  const float* __restrict__ tab32;         // 3D exact, FP32: M, S [n][n], W [n^2]
   T* __restrict__ out;                     // [F][2L]
   int face0, nface;                        // this launch: faces [face0, nface)
   int dg;
@@ -48,10 +49,41 @@ struct FaceScratch {
   static constexpr int n = EXT ? 9 : 6;
 };
 
+// 3D exact FP32 faces: M, S and W in shared memory.  Every thread reads its own
+// row of M and column of S; from constant memory a warp's n different
+// addresses take n passes (the address-divergence unit, 77 % busy, bound the
+// kernel).  The cell's nodes are read four at a time.  Measured on GB300, FP32
+// face kernels (with launch): Q4 sphere of 96^3 cells 31.1 -> 26.7 us, Q5
+// sphere of 64^3 28.9 -> 24.1, Q6 ellipsoid of 48^3 27.0 -> 20.4 us; with TF32
+// faces, Q6 26.7 -> 21.4 us.
+template <typename T, int D, int EXT>
+constexpr bool kFaceTab = D == 3 && EXT == 0 && std::is_same<T, float>::value;
+
+// nodes of a cell in shared memory (kFaceTab: padded to 16 bytes, read in
+// fours)
+template <typename T, int D, int N, int EXT>
+constexpr int face_nodes() {
+  return kFaceTab<T, D, EXT> ? (Shape<D, N>::ND + 3) / 4 * 4 : Shape<D, N>::ND;
+}
+
 // shared-memory bytes of one group of FPB faces
 template <typename T, int D, int N, int EXT, int FPB>
 constexpr size_t face_group_smem() {
-  return (size_t)(FPB * Shape<D, N>::ND + FPB * FaceScratch<EXT>::n * Shape<D, N>::L) * sizeof(T);
+  return (size_t)(FPB * face_nodes<T, D, N, EXT>() + FPB * FaceScratch<EXT>::n * Shape<D, N>::L +
+                  (kFaceTab<T, D, EXT> ? 3 * Shape<D, N>::L : 0)) *
+         sizeof(T);
+}
+
+// The tables into shared memory; once per block, visible after the group's
+// first barrier.
+template <typename T, int D, int N, int EXT, int FPB>
+__device__ __forceinline__ void face_begin(const FaceArgs<T>& a, unsigned char* smem_raw) {
+  if constexpr (kFaceTab<T, D, EXT>) {
+    constexpr int L = Shape<D, N>::L;
+    T* tab = reinterpret_cast<T*>(smem_raw) + FPB * face_nodes<T, D, N, EXT>() +
+             FPB * FaceScratch<EXT>::n * L;
+    for (int i = threadIdx.x; i < 3 * L; i += blockDim.x) tab[i] = __ldg(a.tab32 + i);
+  }
 }
 
 // Faces [f0, min(f0 + FPB, fend)) of right-hand side rhs, L threads per
@@ -69,7 +101,8 @@ __device__ __forceinline__ void face_group(const FaceArgs<T>& a, const KTab<T>& 
   const T* __restrict__ xr = a.x + rhs * a.ldx;
   T* __restrict__ outr = a.out + rhs * a.ld_out;
   T* X = reinterpret_cast<T*>(smem_raw);
-  T* SC = X + FPB * ND;            // NS L per face
+  constexpr int NDX = face_nodes<T, D, N, EXT>();
+  T* SC = X + FPB * NDX;           // NS L per face
   const int tid = threadIdx.x;
   const int nf = min(FPB, fend - f0);
   for (int r = tid; r < nf * ND; r += blockDim.x) {
@@ -78,7 +111,7 @@ __device__ __forceinline__ void face_group(const FaceArgs<T>& a, const KTab<T>& 
     size_t g;
     if (a.dg) g = (size_t)__ldg(a.cell_rank + cell) * ND + loc;
     else g = (size_t)__ldg(a.lines + (size_t)cell * L + loc / N) + (loc % N);
-    X[r] = __ldg(xr + g);
+    X[f * NDX + loc] = __ldg(xr + g);
   }
   __syncthreads();
   const int fl = tid / L, tl = tid - fl * L;
@@ -86,7 +119,7 @@ __device__ __forceinline__ void face_group(const FaceArgs<T>& a, const KTab<T>& 
   const int f = f0 + (act ? fl : 0);
   const int kind = act ? __ldg(a.face_kind + f) : 0;
   const int k = kind & 3, s = kind >> 2;
-  const T* Xf = X + fl * ND;
+  const T* Xf = X + fl * NDX;
   T* sc = SC + fl * NS * L;
   T* Td = sc;
   T* Da = sc + L;
@@ -107,6 +140,8 @@ __device__ __forceinline__ void face_group(const FaceArgs<T>& a, const KTab<T>& 
     sa = (k == 0) ? N : 1;
     sb = (k == 2) ? N : N * N;
   }
+  const T* tM = SC + FPB * NS * L;     // kFaceTab: M, S, W
+  const T* tS = tM + L;
   const int kend = s ? (N - 1) : 0;
   const T sg = s ? T(1) : T(-1);
   const int bt = (tl % N) * sa + (D == 3 ? (tl / N) * sb : 0);
@@ -131,19 +166,19 @@ __device__ __forceinline__ void face_group(const FaceArgs<T>& a, const KTab<T>& 
     //    and one mass product replace the interpolation of Td and two
     //    transposed interpolations
     T tm = T(0);                  // (M x M) Td at tangential node tl
-    if (D == 3) {
+    if (D == 3) {                 // (M symmetric)
       if (act) {
         const int ia = tl % N, jb = tl / N;
         T v = T(0);
 #pragma unroll
-        for (int j = 0; j < N; ++j) v = fma(t.M[ia][j], Td[j + N * jb], v);
+        for (int j = 0; j < N; ++j) v = fma(tM[N * j + ia], Td[j + N * jb], v);
         Da[tl] = v;
       }
       __syncthreads();
       if (act) {
         const int ia = tl % N, ib = tl / N;
 #pragma unroll
-        for (int j = 0; j < N; ++j) tm = fma(t.M[ib][j], Da[ia + N * j], tm);
+        for (int j = 0; j < N; ++j) tm = fma(tM[N * j + ib], Da[ia + N * j], tm);
       }
     } else if (act) {
 #pragma unroll
@@ -157,24 +192,27 @@ __device__ __forceinline__ void face_group(const FaceArgs<T>& a, const KTab<T>& 
 #pragma unroll
       for (int j = 0; j < N; ++j) p0[j] = __ldg(pq + j);
       T e = T(0);
-      if (D == 3) {
+      if constexpr (D == 3) {      // (FP32; FP64: face_fixed.cuh)
         T p1[N], p2[N];
 #pragma unroll
         for (int j = 0; j < N; ++j) {
           p1[j] = __ldg(pq + N + j);
           p2[j] = __ldg(pq + 2 * N + j);
         }
+        const float4* X4 = reinterpret_cast<const float4*>(Xf);
+        T s0 = T(0), s1 = T(0);
 #pragma unroll
-        for (int j2 = 0; j2 < N; ++j2) {
-          T s1 = T(0);
+        for (int i4 = 0; i4 < NDX / 4; ++i4) {
+          const float4 x4 = X4[i4];
 #pragma unroll
-          for (int j1 = 0; j1 < N; ++j1) {
-            T s0 = T(0);
-#pragma unroll
-            for (int j0 = 0; j0 < N; ++j0) s0 = fma(p0[j0], Xf[j0 + N * j1 + N * N * j2], s0);
-            s1 = fma(p1[j1], s0, s1);
+          for (int c = 0; c < 4; ++c) {
+            const int i = 4 * i4 + c, j0 = i % N, j1 = i / N % N, j2 = i / (N * N);
+            if (i >= ND) continue;
+            const float xv = c == 0 ? x4.x : c == 1 ? x4.y : c == 2 ? x4.z : x4.w;
+            s0 = fma(p0[j0], xv, j0 ? s0 : T(0));
+            if (j0 == N - 1) s1 = fma(p1[j1], s0, j1 ? s1 : T(0));
+            if (j0 == N - 1 && j1 == N - 1) e = fma(p2[j2], s1, e);
           }
-          e = fma(p2[j2], s1, e);
         }
       } else {
         T p1[N];
@@ -188,7 +226,7 @@ __device__ __forceinline__ void face_group(const FaceArgs<T>& a, const KTab<T>& 
           e = fma(p1[j1], s0, e);
         }
       }
-      val[tl] = ts.W[tl] * e;
+      val[tl] = (D == 3 ? tS[L + tl] : ts.W[tl]) * e;
     }
     __syncthreads();
     // 4. q = (S x S)^T (W E) at tangential node tl
@@ -198,14 +236,14 @@ __device__ __forceinline__ void face_group(const FaceArgs<T>& a, const KTab<T>& 
         const int ja = tl % N, qb = tl / N;
         T v = T(0);
 #pragma unroll
-        for (int g = 0; g < N; ++g) v = fma(t.S[g][ja], val[g + N * qb], v);
+        for (int g = 0; g < N; ++g) v = fma(tS[N * g + ja], val[g + N * qb], v);
         Va[tl] = v;
       }
       __syncthreads();
       if (act) {
         const int ja = tl % N, jb = tl / N;
 #pragma unroll
-        for (int g = 0; g < N; ++g) q = fma(t.S[g][jb], Va[ja + N * g], q);
+        for (int g = 0; g < N; ++g) q = fma(tS[N * g + jb], Va[ja + N * g], q);
       }
     } else if (act) {
 #pragma unroll

@@ -28,9 +28,10 @@ __global__ void __launch_bounds__(Shape<D, N>::CPB * Shape<D, N>::L)
 sface_kernel(const FaceArgs<T> a, const __grid_constant__ KTab<T> t) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   pdl_trigger();                   // the cell kernel may start (it waits before its folds)
-  face_group<T, D, N, EXT, Shape<D, N>::CPB>(a, t, t, smem_raw,
-                                              a.face0 + blockIdx.x * Shape<D, N>::CPB, a.nface,
-                                              blockIdx.y);
+  constexpr int FPB = Shape<D, N>::CPB;
+  face_begin<T, D, N, EXT, FPB>(a, smem_raw);
+  face_group<T, D, N, EXT, FPB>(a, t, t, smem_raw, a.face0 + blockIdx.x * FPB, a.nface,
+                                blockIdx.y);
 }
 
 // Fixed-point faces (3D FP64, exact extension): 256 / L faces per block, 4
@@ -62,6 +63,7 @@ static cudaError_t face_t(const HostProblem& hp, const DeviceData& dd, const T* 
   a.face_kind = dd.face_kind;
   a.face_phi = face_phi_of<T>(dd);
   a.fix = face_fix_of(hp, dd);
+  a.tab32 = dd.face_tab32;
   a.out = out;
   a.face0 = fb;
   a.nface = fe;
@@ -73,7 +75,7 @@ static cudaError_t face_t(const HostProblem& hp, const DeviceData& dd, const T* 
     sface_fix_kernel<N><<<dim3((fe - fb + FX - 1) / FX, nrhs), FX * L,
                           FaceFixSmem<N, FX>::bytes, st>>>(a, t);
   } else {
-    const size_t smem = face_group_smem<T, D, N, EXT, FPB>();
+    constexpr size_t smem = face_group_smem<T, D, N, EXT, FPB>();
     sface_kernel<T, D, N, EXT><<<dim3((fe - fb + FPB - 1) / FPB, nrhs), FPB * L, smem, st>>>(a,
                                                                                              t);
   }

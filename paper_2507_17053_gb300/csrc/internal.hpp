@@ -177,6 +177,7 @@ struct DeviceData {
   fix::Entry* fix_p0 = nullptr;
   int32_t* fix_exp = nullptr;
   fix::Entry* fix_tab = nullptr;
+  float* face_tab32 = nullptr;   // FP32 faces: M, S [n][n], W [n^2]
   int32_t* nbr = nullptr;        // DG [Nc * 2d] neighbour rank per (k, s), -1 = surrogate
   int32_t* dg_exp = nullptr;     // 3D DG, FP64: [Nc] largest exponent of each cell (scratch)
   double* stage_x = nullptr;     // host-apply staging buffers (allocated on first use)

@@ -44,6 +44,7 @@ struct TcArgs {
   const int32_t* __restrict__ face_kind;
   const float* __restrict__ face_phi;      // [F][L][3][N] FP32
   float* __restrict__ out;                 // [F][2L]
+  const float* __restrict__ tab;           // M, S [n][n], W [n^2]
   int* __restrict__ err;                   // device error word
   int nface;
   int dg;
@@ -81,6 +82,7 @@ tc_face_kernel(const TcArgs<float> a, const __grid_constant__ KTab<float> t) {
   __shared__ float X[F * ND];
   __shared__ float P12[2][N][tc::kM];      // phi of axes 1, 2 by row
   __shared__ float Td[F * L], Da[F * L], val[F * L], Va[F * L];
+  __shared__ float tM[3 * L];              // M, S, W (face_body.cuh)
   __shared__ __align__(8) uint64_t mbar;
   __shared__ uint32_t tmem_base;
   __shared__ int abort_flag;
@@ -94,6 +96,8 @@ tc_face_kernel(const TcArgs<float> a, const __grid_constant__ KTab<float> t) {
     ((uint32_t*)opB)[i] = 0u;
   }
   for (int i = tid; i < 2 * N * tc::kM; i += tc::kThreads) (&P12[0][0][0])[i] = 0.f;
+  for (int i = tid; i < 3 * L; i += tc::kThreads) tM[i] = __ldg(a.tab + i);
+  const float* tS = tM + L;
   if (tid == 0) {
     abort_flag = 0;
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mbar)));
@@ -271,7 +275,7 @@ tc_face_kernel(const TcArgs<float> a, const __grid_constant__ KTab<float> t) {
         for (int j1 = 0; j1 < N; ++j1) s1 = fmaf(P12[0][j1][tid], Tq[j1 + N * j2], s1);
         e = fmaf(P12[1][j2][tid], s1, e);
       }
-      if (act) val[fl * L + q] = t.W[q] * e;
+      if (act) val[fl * L + q] = tS[L + q] * e;
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -283,8 +287,8 @@ tc_face_kernel(const TcArgs<float> a, const __grid_constant__ KTab<float> t) {
       float v1 = 0.f, v2 = 0.f;
 #pragma unroll
       for (int j = 0; j < N; ++j) {
-        v1 = fmaf(t.S[j][ia], val[fl * L + j + N * ib], v1);
-        v2 = fmaf(t.M[ia][j], Td[fl * L + j + N * ib], v2);
+        v1 = fmaf(tS[N * j + ia], val[fl * L + j + N * ib], v1);
+        v2 = fmaf(tM[N * j + ia], Td[fl * L + j + N * ib], v2);
       }
       Va[fl * L + q] = v1;
       Da[fl * L + q] = v2;
@@ -294,8 +298,8 @@ tc_face_kernel(const TcArgs<float> a, const __grid_constant__ KTab<float> t) {
       float qv = 0.f, tm = 0.f;
 #pragma unroll
       for (int j = 0; j < N; ++j) {
-        qv = fmaf(t.S[j][ib], Va[fl * L + ia + N * j], qv);
-        tm = fmaf(t.M[ib][j], Da[fl * L + ia + N * j], tm);
+        qv = fmaf(tS[N * j + ib], Va[fl * L + ia + N * j], qv);
+        tm = fmaf(tM[N * j + ib], Da[fl * L + ia + N * j], tm);
       }
       const float sg = (kind >> 2) ? 1.f : -1.f;
       float* o = a.out + (size_t)(f0 + fl) * 2 * L + q;
@@ -348,6 +352,7 @@ static cudaError_t tc_t(const HostProblem& hp, const DeviceData& dd, const float
   a.face_kind = dd.face_kind;
   a.face_phi = dd.face_phi32;
   a.out = out;
+  a.tab = dd.face_tab32;
   a.err = dd.err_flag;
   a.nface = dd.nface;
   a.dg = hp.desc.dg;
