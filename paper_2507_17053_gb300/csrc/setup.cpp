@@ -485,7 +485,8 @@ int setup_prepare(const sbm_desc& desc, HostProblem* hp, std::string* err) {
     *err = "1D eigenbasis of the cell operator is inaccurate";
     return SBM_ERR_UNSUPPORTED;
   }
-  if (d == 3 && !build_fixed_tables(P.tab, P.h, &P.fx, P.sigma_f * P.h)) {
+  // (2D too: problems of one degree share one unit table in a batch)
+  if (!build_fixed_tables(P.tab, P.h, &P.fx, P.sigma_f * P.h)) {
     *err = "fixed-point tables of the cell operator are out of bounds";
     return SBM_ERR_UNSUPPORTED;
   }
