@@ -125,6 +125,10 @@ static void free_device(DeviceData* dd) {
   cudaFree(dd->reg_cell_chunk);
   cudaFree(dd->reg_block_first);
   cudaFree(dd->reg_mask);
+  cudaFree(dd->plane_cell_chunk);
+  cudaFree(dd->plane_block_first);
+  cudaFree(dd->plane_mask);
+  cudaFree(dd->plane_xops);
   cudaFree(dd->cell_rank);
   cudaFree(dd->face_start);
   cudaFree(dd->face_kind);
@@ -358,7 +362,9 @@ static int build_device(const HostProblem& hp, DeviceData* dd) {
           cudaSuccess)
         goto err;
     }
-    if ((e = build_cell_reg_tables(hp, ch_first[0], dd)) != cudaSuccess) goto err;
+    if ((e = build_cell_reg_tables(hp, ch_first[0], dd)) != cudaSuccess ||
+        (e = build_cell_plane_tables(hp, ch_first[0], dd)) != cudaSuccess)
+      goto err;
     // ordered positions grouped by the parity colour of the cell (diagonal kernel)
     {
       std::vector<int32_t> pos;

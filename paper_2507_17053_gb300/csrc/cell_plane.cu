@@ -1,6 +1,6 @@
-// Cell term of the continuous Galerkin apply with n threads per cell, each
-// holding one x-plane of the cell (n^2 nodes) in registers (3D): tile shape 2
-// of the single applies.
+// Cell term of the continuous Galerkin FP32 apply with n threads per cell, each
+// holding one x-plane of the cell (n^2 nodes) in registers (3D, p >= 3; at p = 1
+// and 2 one thread holds the whole cell, cell_reg.cu).
 //
 // The chunk kernel (cg_apply.cu) holds one line per thread: every one of the
 // five line phases of the eigenbasis cell term (Algorithm 1 in the exact form
@@ -22,8 +22,17 @@
 //     chunk colouring of tile shape 0.
 // The results are bitwise those of tile shape 0; the assembly kernel of that
 // shape completes the DoFs several colours share.
-// @PLANE@
+// Measured on GB300, FP32 applies with the best other tile shape -> this:
+// Q4 sphere of 96^3 cells 132 (one thread per cell, cell_reg.cu, 168 registers
+// and 12 warps per SM) -> 115 us, Q3 57.7 -> 55.7, Q5 of 64^3 88.6 (chunks
+// without staged runs) -> 77, Q6 ellipsoid of 48^3 48.9 -> 46.1 us.  The cell
+// term of the Q4 sphere takes 71 us for 133 MB: load latency (6 of 13 stall
+// cycles per instruction) and 1 180 instructions per warp of six cells.  In
+// FP64 the fixed-point plane (50 registers and more of 64-bit values) is
+// slower than the chunks (p = 4 535 against 372 us).
 #include <algorithm>
+#include <cmath>
+#include <vector>
 
 #include "chunk_body.cuh"
 
@@ -37,7 +46,7 @@ template <int N>
 struct PlaneShape {
   static constexpr int L = N * N;
   static constexpr int CW = 32 / N;                                  // cells per warp
-  static constexpr int W = N == 3 ? 3 : N == 6 ? 7 : N <= 4 ? 4 : 5; // warps
+  static constexpr int W = N == 4 ? 4 : N == 6 ? 7 : 5;              // warps
   static constexpr int CPB = CW * W, NT = 32 * W;
   static constexpr int PX = N % 2 ? N : N + 1;                       // line stride
   static constexpr int CS = PX * L | 1;                              // cell stride
@@ -45,108 +54,60 @@ struct PlaneShape {
   static_assert(CPB >= 256 / L, "a block holds a chunk");
 };
 constexpr int plane_cells(int n) {
-  return n == 2 ? PlaneShape<2>::CPB : n == 3 ? PlaneShape<3>::CPB : n == 4 ? PlaneShape<4>::CPB
-       : n == 5 ? PlaneShape<5>::CPB : n == 6 ? PlaneShape<6>::CPB : PlaneShape<7>::CPB;
+  return n == 4 ? PlaneShape<4>::CPB : n == 5 ? PlaneShape<5>::CPB
+       : n == 6 ? PlaneShape<6>::CPB : PlaneShape<7>::CPB;
 }
 
-// resident warps asked of the compiler
-#ifndef SBM_PW32
-#define SBM_PW32 (N <= 4 ? 40 : N == 5 ? 30 : 20)
-#endif
-#ifndef SBM_PW64
-#define SBM_PW64 (N <= 3 ? 32 : N == 4 ? 24 : N == 5 ? 20 : N == 6 ? 14 : 10)
-#endif
-template <typename T, int N>
-constexpr int plane_min_blocks() {
-  return (std::is_same<T, float>::value ? SBM_PW32 : SBM_PW64) / PlaneShape<N>::W;
-}
+// Resident warps asked of the compiler (FP32 applies, spheres of 96^3 cells at
+// p = 3, 4, 64^3 at p = 5, ellipsoid of 48^3 at p = 6; 28 / 36 / 44 warps):
+// p = 3 59.7 / 55.7 / 60.1 us, p = 4 119.1 / 115.3 / 121.4, p = 5 77.0 / 87.9 /
+// 123.0 (spills), p = 6 46.1 with 20, 47.4 / 67.2 / 76.6.
+constexpr int plane_warps(int n) { return n == 4 ? 36 : n == 5 ? 36 : n == 6 ? 28 : 20; }
+template <int N>
+constexpr int plane_min_blocks() { return plane_warps(N) / PlaneShape<N>::W; }
 
-template <typename T>
 struct PlaneArgs {
-  const T* __restrict__ x;
-  T* __restrict__ y;
-  T* __restrict__ ycol;                     // [ncolours][n_dofs]
+  const float* __restrict__ x;
+  float* __restrict__ y;
+  float* __restrict__ ycol;                 // [ncolours][n_dofs]
   const int32_t* __restrict__ lines;        // ordered cells x L
   const int32_t* __restrict__ face_start;
   const int32_t* __restrict__ face_kind;
-  const T* face_out;                        // [F][2L]
+  const float* face_out;                    // [F][2L]
   const int32_t* __restrict__ chunk_first;  // tile shape 0
   const uint8_t* __restrict__ chunk_col;
   const int32_t* __restrict__ cell_chunk;   // ordered cell -> its chunk
   const uint32_t* __restrict__ mask;        // [Nc][n][MW]: node of the plane shared by several
                                             //   colours
   const int32_t* __restrict__ block_first;  // [nblocks + 1] first chunk of each block
-  const fix::Entry* __restrict__ xfix;      // FP64: x-line operators
+  const float* __restrict__ xops;           // x-line operators, slot by slot (XLineOp)
   int64_t n_dofs;
-  int eoff;
-};
-
-// one line's phases; FP64 in fixed point
-template <typename T, int N>
-struct PlaneOps {
-  using V = T;
-  static __device__ __forceinline__ void to_modes(const KTab<T>& t, const V (&v)[N], V (&w)[N]) {
-    line_to_modes<T, N>(t.fVt, v, w);
-  }
-  static __device__ __forceinline__ void xline(const T* m, const V (&v)[N], V (&y)[N]) {
-    XLineShared<T, N>{m}.apply(v, y);
-  }
-  static __device__ __forceinline__ void back_y(const KTab<T>& t, const V (&w)[N], V (&y)[N]) {
-    modes_to_line<T, N>(t.fV, w, y);
-  }
-  static __device__ __forceinline__ void back_z(const KTab<T>& t, const V (&w)[N], V (&y)[N]) {
-    modes_to_line<T, N>(t.fV, w, y);
-  }
-};
-template <int N>
-struct PlaneOps<double, N> {
-  using V = int64_t;
-  static __device__ __forceinline__ void to_modes(const KTab<double>& t, const V (&v)[N],
-                                                  V (&w)[N]) {
-    fix::to_modes<N, 0>(t.xVt, v, w);
-  }
-  static __device__ __forceinline__ void xline(const double* md, const V (&v)[N], V (&y)[N]) {
-    using Op = XLineOp<double, N>;
-    constexpr int HE = (N + 1) / 2;
-    const fix::Entry* m = reinterpret_cast<const fix::Entry*>(md);
-    fix::apply_line<N, fix::shift_x(N)>(
-        [&](int i, int j) { return m[Op::sym(i, j, HE)]; },
-        [&](int i, int j) { return m[HE * (HE + 1) / 2 + Op::sym(i, j, N / 2)]; }, v, y);
-  }
-  static __device__ __forceinline__ void back_y(const KTab<double>& t, const V (&w)[N],
-                                                V (&y)[N]) {
-    fix::from_modes<N, fix::shift_y(N)>(t.xV, w, y);
-  }
-  static __device__ __forceinline__ void back_z(const KTab<double>& t, const V (&w)[N],
-                                                V (&y)[N]) {
-    fix::from_modes<N, fix::shift_z(N)>(t.xV, w, y);
-  }
 };
 
 // surrogate face (k, s): fold_face_z's operations on the nodes (j0, y, z) of
 // the thread's plane x = j0
-template <typename T, int N>
-__device__ __forceinline__ void fold_plane(const KTab<T>& t, const T* fo, int k, int s, int j0,
-                                           T (&u)[N * N]) {
+template <int N>
+__device__ __forceinline__ void fold_plane(const KTab<float>& t, const float* fo, int k, int s, int j0,
+                                           float (&u)[N * N]) {
   constexpr int L = N * N;
-  const T* rv = fo;
-  const T* rg = fo + L;
+  const float* rv = fo;
+  const float* rg = fo + L;
   const int kend = s ? N - 1 : 0;
   if (k == 0) {
-    const T dk = s ? t.D1[j0] : t.D0[j0];
+    const float dk = s ? t.D1[j0] : t.D0[j0];
 #pragma unroll
     for (int l = 0; l < L; ++l) {
-      T add = mul_rn(dk, ld_face<true>(rg + l));
+      float add = mul_rn(dk, ld_face<true>(rg + l));
       if (j0 == kend) add = add_rn(add, ld_face<true>(rv + l));
       u[l] = add_rn(u[l], add);
     }
   } else if (k == 1) {
 #pragma unroll
     for (int m = 0; m < N; ++m) {
-      const T g = ld_face<true>(rg + j0 + N * m), v = ld_face<true>(rv + j0 + N * m);
+      const float g = ld_face<true>(rg + j0 + N * m), v = ld_face<true>(rv + j0 + N * m);
 #pragma unroll
       for (int b = 0; b < N; ++b) {
-        T add = mul_rn(s ? t.D1[b] : t.D0[b], g);
+        float add = mul_rn(s ? t.D1[b] : t.D0[b], g);
         if (b == kend) add = add_rn(add, v);
         u[b + N * m] = add_rn(u[b + N * m], add);
       }
@@ -154,10 +115,10 @@ __device__ __forceinline__ void fold_plane(const KTab<T>& t, const T* fo, int k,
   } else {
 #pragma unroll
     for (int b = 0; b < N; ++b) {
-      const T g = ld_face<true>(rg + j0 + N * b), v = ld_face<true>(rv + j0 + N * b);
+      const float g = ld_face<true>(rg + j0 + N * b), v = ld_face<true>(rv + j0 + N * b);
 #pragma unroll
       for (int m = 0; m < N; ++m) {
-        T& o = u[b + N * m];
+        float& o = u[b + N * m];
         o = fma(s ? t.D1[m] : t.D0[m], g, o);
         if (m == kend) o = add_rn(o, v);
       }
@@ -165,27 +126,65 @@ __device__ __forceinline__ void fold_plane(const KTab<T>& t, const T* fo, int k,
   }
 }
 
-template <typename T, int N>
-__global__ void __launch_bounds__(PlaneShape<N>::NT, (plane_min_blocks<T, N>()))
-cg_plane_kernel(const PlaneArgs<T> a, const __grid_constant__ KTab<T> t) {
+// h K + mu_ab M of modes (a, b) in XLineOp's packed form, as XLineShared
+template <int N>
+__device__ __forceinline__ void plane_xline(const float* m, const float (&v)[N],
+                                            float (&y)[N]) {
+  using Op = XLineOp<float, N>;
+  constexpr int H = N / 2, HE = (N + 1) / 2;
+  const LineFold<float, N> f(v);
+  LineAcc<float, N> acc;
+  const float* e = m;
+  const float* o = m + HE * (HE + 1) / 2;
+#pragma unroll
+  for (int i = 0; i < HE; ++i)
+#pragma unroll
+    for (int j = 0; j < HE; ++j) acc.s[i] = fma(e[Op::sym(i, j, HE)], f.e[j], acc.s[i]);
+#pragma unroll
+  for (int i = 0; i < H; ++i)
+#pragma unroll
+    for (int j = 0; j < H; ++j) acc.d[i] = fma(o[Op::sym(i, j, H)], f.o[j], acc.d[i]);
+  acc.unfold(y);
+}
+
+// barrier id of two warps; immediate ids, as a register one reserves all 16
+template <int ID, int W>
+__device__ __forceinline__ void pair_arrive(int id) {
+  if constexpr (ID < W) {
+    if (id == ID) asm volatile("bar.arrive %0, 64;" ::"n"(ID) : "memory");
+    else pair_arrive<ID + 1, W>(id);
+  }
+}
+template <int ID, int W>
+__device__ __forceinline__ void pair_wait(int id) {
+  if constexpr (ID < W) {
+    if (id == ID) asm volatile("bar.sync %0, 64;" ::"n"(ID) : "memory");
+    else pair_wait<ID + 1, W>(id);
+  }
+}
+
+// Warps run independently but for the x-face of two cells of a chunk in
+// neighbouring warps: the first one arrives at a barrier of the two when its
+// plane is stored, the second one waits there.
+template <int N>
+__global__ void __launch_bounds__(PlaneShape<N>::NT, (plane_min_blocks<N>()))
+cg_plane_kernel(const PlaneArgs a, const __grid_constant__ KTab<float> t) {
   using Sh = PlaneShape<N>;
-  using Op = PlaneOps<T, N>;
-  using V = typename Op::V;
-  using XO = XLineOp<T, N>;
-  constexpr bool FX = std::is_same<T, double>::value;
-  constexpr int L = Sh::L, P = N - 1, PX = Sh::PX, MW = Sh::MW;
-  __shared__ V S[Sh::CPB * Sh::CS];
-  __shared__ T xface[Sh::CPB][L | 1];           // j0 = P plane of each cell
-  __shared__ T xops[XO::kSlots * XO::kPacked];
-  const int tid = threadIdx.x, lane = tid & 31;
-  const int cell = (tid >> 5) * Sh::CW + lane / N, j0 = lane % N;
+  using XO = XLineOp<float, N>;
+  constexpr int L = Sh::L, P = N - 1, PX = Sh::PX, MW = Sh::MW, LAST = Sh::CW * N - 1;
+  __shared__ float S[Sh::CPB * Sh::CS];
+  __shared__ float xops[XO::kSlots * XO::kPacked];
+  for (int i = threadIdx.x; i < XO::kSlots * XO::kPacked; i += Sh::NT) xops[i] = __ldg(a.xops + i);
+  __shared__ float xface[Sh::W][L];             // j0 = P plane of a warp's last cell
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int cell = w * Sh::CW + lane / N, j0 = lane % N;
   const int b0 = __ldg(a.block_first + blockIdx.x), b1 = __ldg(a.block_first + blockIdx.x + 1);
   const int c0 = __ldg(a.chunk_first + b0), c1 = __ldg(a.chunk_first + b1);
   const int pos = c0 + cell;
-  const bool act = lane < Sh::CW * N && pos < c1;
+  const bool act = lane <= LAST && pos < c1;
   int c = 0, nc = 0, ch = 0, off = 0;
   const int32_t* ln = a.lines;
-  T u[L];
+  float u[L], p[N], q[N];
   if (act) {
     ch = __ldg(a.cell_chunk + pos);
     const int f = __ldg(a.chunk_first + ch);
@@ -195,138 +194,87 @@ cg_plane_kernel(const PlaneArgs<T> a, const __grid_constant__ KTab<T> t) {
     off = P * c + j0;
 #pragma unroll
     for (int l = 0; l < L; ++l) u[l] = __ldg(a.x + (__ldg(ln + l) + off));
-  } else {
 #pragma unroll
-    for (int l = 0; l < L; ++l) u[l] = T(0);
-  }
-  if constexpr (FX) {
-    xline_copy<N>(reinterpret_cast<fix::Entry*>(xops), a.xfix, tid);
-  } else {
-    if (tid < L && tid % N <= tid / N)
-      XO(t, tid % N, tid / N).store(xops + XO::slot(tid % N, tid / N) * XO::kPacked);
-  }
-  V v[L], p[N], q[N];
-  int E = 1;
-  if constexpr (FX) {                           // the cell's exponent
-    uint32_t mx = 0u;
+    for (int a1 = 0; a1 < N; ++a1) {            // z-lines -> z-modes
 #pragma unroll
-    for (int l = 0; l < L; ++l) mx = max(mx, fix::mag_hi((uint64_t)__double_as_longlong(u[l])));
-    uint32_t m = mx;
+      for (int k = 0; k < N; ++k) p[k] = u[a1 + N * k];
+      line_to_modes<float, N>(t.fVt, p, q);
 #pragma unroll
-    for (int k = 1; k < N; ++k) {
-      const int from = lane - j0 + (j0 + k < N ? j0 + k : j0 + k - N);
-      m = max(m, __shfl_sync(0xffffffffu, mx, from & 31));
+      for (int k = 0; k < N; ++k) u[a1 + N * k] = q[k];
     }
-    E = max(1, (int)(m >> 20));
-    if (fix::plain_exp(E)) {
+    float* Sc = S + cell * Sh::CS;
 #pragma unroll
-      for (int l = 0; l < L; ++l)
-        v[l] = fix::from_double<false>((uint64_t)__double_as_longlong(u[l]), E);
-    } else {
+    for (int b = 0; b < N; ++b) {               // y-lines -> y-modes
 #pragma unroll
-      for (int l = 0; l < L; ++l)
-        v[l] = fix::from_double<true>((uint64_t)__double_as_longlong(u[l]), E);
+      for (int k = 0; k < N; ++k) p[k] = u[k + N * b];
+      line_to_modes<float, N>(t.fVt, p, q);
+#pragma unroll
+      for (int k = 0; k < N; ++k) Sc[PX * (k + N * b) + j0] = q[k];
     }
-  } else {
-#pragma unroll
-    for (int l = 0; l < L; ++l) v[l] = u[l];
-  }
-#pragma unroll
-  for (int a1 = 0; a1 < N; ++a1) {              // z-lines -> z-modes
-#pragma unroll
-    for (int k = 0; k < N; ++k) p[k] = v[a1 + N * k];
-    Op::to_modes(t, p, q);
-#pragma unroll
-    for (int k = 0; k < N; ++k) v[a1 + N * k] = q[k];
-  }
-#pragma unroll
-  for (int b = 0; b < N; ++b) {                 // y-lines -> y-modes
-#pragma unroll
-    for (int k = 0; k < N; ++k) p[k] = v[k + N * b];
-    Op::to_modes(t, p, q);
-#pragma unroll
-    for (int k = 0; k < N; ++k) v[k + N * b] = q[k];
-  }
-  V* const Sc = S + (lane < Sh::CW * N ? cell : 0) * Sh::CS;
-  if (act) {
-#pragma unroll
-    for (int l = 0; l < L; ++l) Sc[PX * l + j0] = v[l];
   }
   __syncthreads();                              // xops; the planes
   if (act) {                                    // x-lines of z-mode j0
 #pragma unroll
     for (int a1 = 0; a1 < N; ++a1) {
-      V* line = Sc + PX * (a1 + N * j0);
+      float* line = S + cell * Sh::CS + PX * (a1 + N * j0);
 #pragma unroll
       for (int k = 0; k < N; ++k) p[k] = line[k];
-      Op::xline(xops + XO::slot(a1, j0) * XO::kPacked, p, q);
+      plane_xline<N>(xops + XO::slot(a1, j0) * XO::kPacked, p, q);
 #pragma unroll
       for (int k = 0; k < N; ++k) line[k] = q[k];
     }
   }
   __syncwarp();
   if (act) {
+    const float* Sc = S + cell * Sh::CS;
 #pragma unroll
-    for (int l = 0; l < L; ++l) v[l] = Sc[PX * l + j0];
-  }
+    for (int b = 0; b < N; ++b) {               // y-modes back
 #pragma unroll
-  for (int b = 0; b < N; ++b) {                 // y-modes back
+      for (int k = 0; k < N; ++k) p[k] = Sc[PX * (k + N * b) + j0];
+      modes_to_line<float, N>(t.fV, p, q);
 #pragma unroll
-    for (int k = 0; k < N; ++k) p[k] = v[k + N * b];
-    Op::back_y(t, p, q);
-#pragma unroll
-    for (int k = 0; k < N; ++k) v[k + N * b] = q[k];
-  }
-#pragma unroll
-  for (int a1 = 0; a1 < N; ++a1) {              // z-modes back
-#pragma unroll
-    for (int k = 0; k < N; ++k) p[k] = v[a1 + N * k];
-    Op::back_z(t, p, q);
-#pragma unroll
-    for (int k = 0; k < N; ++k) v[a1 + N * k] = q[k];
-  }
-  if constexpr (FX) {
-    if (fix::plain_exp(E)) {
-#pragma unroll
-      for (int l = 0; l < L; ++l)
-        u[l] = __longlong_as_double((long long)fix::to_double<false>(v[l], E + a.eoff));
-    } else {
-#pragma unroll
-      for (int l = 0; l < L; ++l)
-        u[l] = E == fix::kExpBad
-                   ? __longlong_as_double(0x7ff8000000000000ll)
-                   : __longlong_as_double((long long)fix::to_double<true>(v[l], E + a.eoff));
+      for (int k = 0; k < N; ++k) u[k + N * b] = q[k];
     }
-  } else {
 #pragma unroll
-    for (int l = 0; l < L; ++l) u[l] = v[l];
-  }
-  if (act) {
+    for (int a1 = 0; a1 < N; ++a1) {            // z-modes back
+#pragma unroll
+      for (int k = 0; k < N; ++k) p[k] = u[a1 + N * k];
+      modes_to_line<float, N>(t.fV, p, q);
+#pragma unroll
+      for (int k = 0; k < N; ++k) u[a1 + N * k] = q[k];
+    }
     const int fs = __ldg(a.face_start + pos), fe = __ldg(a.face_start + pos + 1);
     if (fs < fe) pdl_wait();
     for (int f2 = fs; f2 < fe; ++f2) {
       const int kind = __ldg(a.face_kind + f2);
-      fold_plane<T, N>(t, a.face_out + (size_t)f2 * 2 * L, kind & 3, kind >> 2, j0, u);
-    }
-    if (j0 == P && c < nc - 1) {
-#pragma unroll
-      for (int l = 0; l < L; ++l) xface[cell][l] = u[l];
+      fold_plane<N>(t, a.face_out + (size_t)f2 * 2 * L, kind & 3, kind >> 2, j0, u);
     }
   }
-  __syncthreads();
-  if (!act || (j0 == P && c < nc - 1)) return;
+  __syncwarp();
   // the x-face plane shared with the previous cell of the chunk: prev + own
-  if (j0 == 0 && c > 0) {
+  if (w + 1 < Sh::W) {
+    if (lane == LAST) {
 #pragma unroll
-    for (int l = 0; l < L; ++l) u[l] = add_rn(xface[cell - 1][l], u[l]);
+      for (int l = 0; l < L; ++l) xface[w][l] = u[l];
+    }
+    pair_arrive<1, Sh::W>(w + 1);
   }
+  if (w > 0) pair_wait<1, Sh::W>(w);
+  const bool add = act && j0 == 0 && c > 0;
+#pragma unroll
+  for (int l = 0; l < L; ++l) {
+    float prev = __shfl_up_sync(0xffffffffu, u[l], 1);
+    if (lane == 0 && add) prev = xface[w - 1][l];
+    if (add) u[l] = add_rn(prev, u[l]);
+  }
+  if (!act || (j0 == P && c < nc - 1)) return;
   uint32_t mk[MW];
 #pragma unroll
   for (int i = 0; i < MW; ++i) mk[i] = __ldg(a.mask + ((size_t)pos * N + j0) * MW + i);
-  T* yc = a.ycol + (size_t)__ldg(a.chunk_col + ch) * a.n_dofs;
+  float* yc = a.ycol + (size_t)__ldg(a.chunk_col + ch) * a.n_dofs;
 #pragma unroll
   for (int l = 0; l < L; ++l) {
-    T* dst = ((mk[l >> 5] >> (l & 31)) & 1u) ? yc : a.y;
+    float* dst = ((mk[l >> 5] >> (l & 31)) & 1u) ? yc : a.y;
     dst[__ldg(ln + l) + off] = u[l];
   }
 }
@@ -356,10 +304,29 @@ __global__ void k_plane_mask(const int32_t* __restrict__ cell_chunk,
   }
 }
 
-template <typename T, int N>
-cudaError_t launch_plane(const HostProblem& hp, const DeviceData& dd, const T* x, T* y,
-                         const T* fo, T* ycol, cudaStream_t st, bool pdl) {
-  PlaneArgs<T> a;
+// the x-line operators, with the device's arithmetic (fused multiply-adds)
+template <int N>
+std::vector<float> make_xops(const KTab<float>& t) {
+  using XO = XLineOp<float, N>;
+  constexpr int H = N / 2, HE = (N + 1) / 2;
+  std::vector<float> o((size_t)XO::kSlots * XO::kPacked, 0.f);
+  for (int b = 0; b < N; ++b)
+    for (int a = 0; a <= b; ++a) {
+      float* m = o.data() + XO::sym(a, b, N) * XO::kPacked;
+      const float mu = t.hlam[a] + t.hlam[b];
+      for (int i = 0; i < HE; ++i)
+        for (int j = i; j < HE; ++j) m[XO::tri(i, j, HE)] = std::fma(mu, t.fM.E[i][j], t.fKh.E[i][j]);
+      for (int i = 0; i < H; ++i)
+        for (int j = i; j < H; ++j)
+          m[HE * (HE + 1) / 2 + XO::tri(i, j, H)] = std::fma(mu, t.fM.O[i][j], t.fKh.O[i][j]);
+    }
+  return o;
+}
+
+template <int N>
+cudaError_t launch_plane(const HostProblem& hp, const DeviceData& dd, const float* x, float* y,
+                         const float* fo, float* ycol, cudaStream_t st, bool pdl) {
+  PlaneArgs a;
   a.x = x;
   a.y = y;
   a.ycol = ycol;
@@ -372,29 +339,36 @@ cudaError_t launch_plane(const HostProblem& hp, const DeviceData& dd, const T* x
   a.cell_chunk = dd.plane_cell_chunk;
   a.mask = dd.plane_mask;
   a.block_first = dd.plane_block_first;
-  a.xfix = dd.xfix;
+  a.xops = dd.plane_xops;
   a.n_dofs = hp.n_dofs;
-  a.eoff = hp.fx.eoff;
   // pdl: a programmatic dependent of the face kernel; a thread waits for it
   // only when its cell has surrogate faces and reads the results with
   // coherent loads.  The kernel does not trigger its own dependents early
   // (the assembly starts as its blocks finish).
-  return launch_maybe_pdl(cg_plane_kernel<T, N>, dim3(dd.plane_nblocks), dim3(PlaneShape<N>::NT),
-                          0, st, pdl, a, make_ktab<T>(hp));
+  return launch_maybe_pdl(cg_plane_kernel<N>, dim3(dd.plane_nblocks), dim3(PlaneShape<N>::NT), 0,
+                          st, pdl, a, make_ktab<float>(hp));
+}
+
+std::vector<float> xops_of(const HostProblem& hp) {
+  const KTab<float> t = make_ktab<float>(hp);
+  switch (hp.n) {
+    case 4: return make_xops<4>(t);
+    case 5: return make_xops<5>(t);
+    case 6: return make_xops<6>(t);
+    default: return make_xops<7>(t);
+  }
 }
 
 }  // namespace
 
-bool cell_plane_available(const HostProblem& hp, bool fp32) {
-  return hp.d == 3 && !hp.desc.dg && hp.n >= 2 && hp.n <= (fp32 ? 7 : 7);
-}
+bool cell_plane_used(const HostProblem& hp) { return hp.d == 3 && !hp.desc.dg && hp.n >= 4; }
 
-// The tables of tile shape 2 (3D continuous Galerkin): the chunk of every
+// The tables of the plane kernel: the chunk of every
 // ordered cell, blocks of whole chunks (at most plane_cells(n) cells), and the
 // per-plane multi-colour bits (from the device run bits of tile shape 0).
 cudaError_t build_cell_plane_tables(const HostProblem& hp, const std::vector<int32_t>& ch_first,
                                     DeviceData* dd) {
-  if (hp.d != 3 || hp.desc.dg) return cudaSuccess;
+  if (!cell_plane_used(hp)) return cudaSuccess;
   const int nch = (int)ch_first.size() - 1;
   const int nc_all = ch_first.back();
   const int cells = plane_cells(hp.n);
@@ -429,28 +403,24 @@ cudaError_t build_cell_plane_tables(const HostProblem& hp, const std::vector<int
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
   }
+  const std::vector<float> xo = xops_of(hp);
+  if (e == cudaSuccess) e = cudaMalloc((void**)&dd->plane_xops, xo.size() * sizeof(float));
+  if (e == cudaSuccess)
+    e = cudaMemcpy(dd->plane_xops, xo.data(), xo.size() * sizeof(float), cudaMemcpyHostToDevice);
   dd->plane_nblocks = (int)block_first.size() - 1;
   return e;
 }
 
-template <typename T>
-cudaError_t launch_cell_plane(const HostProblem& hp, const DeviceData& dd, const T* x, T* y,
-                              const T* fo, T* ycol, cudaStream_t st, bool pdl) {
+cudaError_t launch_cell_plane(const HostProblem& hp, const DeviceData& dd, const float* x,
+                              float* y, const float* fo, float* ycol, cudaStream_t st, bool pdl) {
   if (!dd.plane_mask) return cudaErrorInvalidValue;
   switch (hp.n) {
-    case 2: return launch_plane<T, 2>(hp, dd, x, y, fo, ycol, st, pdl);
-    case 3: return launch_plane<T, 3>(hp, dd, x, y, fo, ycol, st, pdl);
-    case 4: return launch_plane<T, 4>(hp, dd, x, y, fo, ycol, st, pdl);
-    case 5: return launch_plane<T, 5>(hp, dd, x, y, fo, ycol, st, pdl);
-    case 6: return launch_plane<T, 6>(hp, dd, x, y, fo, ycol, st, pdl);
-    case 7: return launch_plane<T, 7>(hp, dd, x, y, fo, ycol, st, pdl);
+    case 4: return launch_plane<4>(hp, dd, x, y, fo, ycol, st, pdl);
+    case 5: return launch_plane<5>(hp, dd, x, y, fo, ycol, st, pdl);
+    case 6: return launch_plane<6>(hp, dd, x, y, fo, ycol, st, pdl);
+    case 7: return launch_plane<7>(hp, dd, x, y, fo, ycol, st, pdl);
     default: return cudaErrorInvalidValue;
   }
 }
-template cudaError_t launch_cell_plane<float>(const HostProblem&, const DeviceData&, const float*,
-                                              float*, const float*, float*, cudaStream_t, bool);
-template cudaError_t launch_cell_plane<double>(const HostProblem&, const DeviceData&,
-                                               const double*, double*, const double*, double*,
-                                               cudaStream_t, bool);
 
 }  // namespace sbm

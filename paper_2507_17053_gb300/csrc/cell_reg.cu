@@ -1,9 +1,8 @@
 // Cell term of the continuous Galerkin apply with one thread per cell and
-// the cell's whole (p+1)^3 tile in registers (3D, FP32, p <= 4): tile shape 2
-// of the single applies.  (FP64 applies accept shape 2 for p <= 3 and run it
-// as shape 0, which gives the same bits: the register form's cell term took
-// 0.56 ms against 0.38 ms at p = 3 in double precision, and the fixed-point
-// cell term needs two registers per node and more.)
+// the cell's whole (p+1)^3 tile in registers (3D, FP32, p <= 2; above, n
+// threads per cell, cell_plane.cu; at p = 2, sphere of 96^3 cells, 24.4 us
+// against 27.1 with planes).  (FP64 applies accept shape 2 for p <= 3 and run
+// it as shape 0, which gives the same bits.)
 //
 // The chunk kernel (cg_apply.cu) spends most of its issue slots outside the
 // arithmetic: staging runs in shared memory, splitting run indices, five
@@ -35,23 +34,14 @@ namespace sbm {
 namespace {
 
 // Threads (cells) per block, a block holding whole chunks of R = 256 / n^2
-// cells: 96 at p = 4, 32 at p = 2, 3, 64 at p = 1 (a chunk of 64 cells).
-// A thread lives one cell, about 25 us at p = 4, so the grid's last,
-// partly filled wave costs up to that much; the sizes were measured
-// (unprofiled FP32 applies, spheres of 96^3 cells, 128^3 at p = 2; 64
-// threads before): p = 4 0.1352 -> 0.1331 ms (96; 32: 0.1429, 128:
-// 0.1351), p = 3 0.0577 -> 0.0562 ms (32; 96: 0.0597), p = 2 0.0469 ->
-// 0.0458 ms (32).  (Earlier, without the programmatic launch, 64-cell
-// blocks beat 128-cell ones at p = 4: 0.096 -> 0.083 ms.)
-constexpr int reg_threads(int n) { return n == 5 ? 96 : (n == 2 ? 64 : 32); }
+// cells: 32 at p = 2 (64: 0.0469 against 0.0458 ms, sphere of 128^3 cells), 64
+// at p = 1 (a chunk of 64 cells).
+constexpr int reg_threads(int n) { return n == 2 ? 64 : 32; }
 
-// Resident blocks asked of the compiler, as warps per SM: FP32 p <= 3, 16
-// (128 registers, no spills; p = 3 cell term 41.2 -> 37.9 us against 12 at
-// 148 registers); p = 4, 12 (168 registers; 14 or 16 warps spill the tile:
-// 83 -> 102 us).
+// resident blocks asked of the compiler: 16 warps per SM (128 registers)
 template <typename T, int N>
 constexpr int reg_min_blocks() {
-  return (N <= 4 ? 16 : 12) * 32 / reg_threads(N);
+  return 16 * 32 / reg_threads(N);
 }
 
 template <int N>
@@ -327,10 +317,8 @@ cudaError_t launch_reg(const HostProblem& hp, const DeviceData& dd, const T* x, 
   // has surrogate faces (the other cells need nothing from it) and then reads
   // the face results with coherent loads.  The kernel does not trigger its
   // own dependents early (the assembly starts as its blocks finish): an early
-  // trigger cost 0.5-1 %.  Measured, unprofiled FP32 applies on GB300,
-  // spheres with 96^3 cells (128^3 at p = 2): p = 4 0.1427 -> 0.1409 ms,
-  // p = 3 0.0623 -> 0.0577 ms, p = 2 0.0520 -> 0.0480 ms; results bitwise
-  // unchanged.
+  // trigger cost 0.5-1 %.  Measured, unprofiled FP32 apply on GB300, p = 2
+  // sphere of 128^3 cells: 0.0520 -> 0.0480 ms; results bitwise unchanged.
   cudaError_t e = pdl ? launch_maybe_pdl(cg_cell_reg_kernel<T, N, true>, dim3(dd.reg_nblocks),
                                          dim3(reg_threads(N)), 0, st, true, a, t, xo)
                       : launch_maybe_pdl(cg_cell_reg_kernel<T, N, false>, dim3(dd.reg_nblocks),
@@ -340,18 +328,21 @@ cudaError_t launch_reg(const HostProblem& hp, const DeviceData& dd, const T* x, 
 
 }  // namespace
 
+bool cell_reg_used(const HostProblem& hp) { return hp.d == 3 && !hp.desc.dg && hp.n <= 3; }
+
+// what tile shape 2 accepts: FP32 p <= 4, FP64 p <= 3
 bool cell_reg_available(const HostProblem& hp, bool fp32) {
   return hp.d == 3 && !hp.desc.dg && hp.n >= 2 && hp.n <= (fp32 ? 5 : 4);
 }
 
-// The per-cell tables of tile shape 2 (3D continuous Galerkin, n <= 5): the
+// The per-cell tables of the register kernel (3D continuous Galerkin, n <= 3): the
 // chunk of every ordered cell, blocks of whole chunks (at most
 // reg_threads(n) cells; a chunk has at most 256 / n^2 <= reg_threads(n)),
 // and the per-cell multi-colour bits (from the device run bits of tile
 // shape 0).
 cudaError_t build_cell_reg_tables(const HostProblem& hp, const std::vector<int32_t>& ch_first,
                                   DeviceData* dd) {
-  if (!cell_reg_available(hp, true)) return cudaSuccess;
+  if (!cell_reg_used(hp)) return cudaSuccess;
   const int nch = (int)ch_first.size() - 1;
   const int nc_all = ch_first.back();
   const int threads = reg_threads(hp.n);
@@ -392,12 +383,10 @@ cudaError_t build_cell_reg_tables(const HostProblem& hp, const std::vector<int32
 
 cudaError_t launch_cell_reg(const HostProblem& hp, const DeviceData& dd, const float* x, float* y,
                             const float* fo, float* ycol, cudaStream_t st, bool pdl) {
-  if (!cell_reg_available(hp, true) || !dd.reg_mask) return cudaErrorInvalidValue;
+  if (!dd.reg_mask) return cudaErrorInvalidValue;
   switch (hp.n) {
     case 2: return launch_reg<float, 2>(hp, dd, x, y, fo, ycol, st, pdl);
     case 3: return launch_reg<float, 3>(hp, dd, x, y, fo, ycol, st, pdl);
-    case 4: return launch_reg<float, 4>(hp, dd, x, y, fo, ycol, st, pdl);
-    case 5: return launch_reg<float, 5>(hp, dd, x, y, fo, ycol, st, pdl);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -228,7 +228,7 @@ static cudaError_t apply_r(const HostProblem& hp, const DeviceData& dd, const Ch
   // CUDA-core face kernel (which x's producers precede in the stream), the
   // assembly after the cell kernel.  Measured (unprofiled applies, GB300):
   // FP32 p = 6 ellipsoid (shape 3) 62.7 -> 57.4 us, p = 3 / 4 spheres
-  // (shapes 0, 3) 1-5 % faster, shape 2 1-8 % faster (cell_reg.cu); FP64 (with
+  // (shapes 0, 3) 1-5 % faster, shape 2 1-8 % faster (cell_plane.cu); FP64 (with
   // the fixed-point faces) disk of 1 801 DoFs 18.4 -> 13.4 us, p = 3 box of
   // 24^3 cells 29.2 -> 22.7, p = 6 ellipsoid 148 -> 137, p = 4 sphere 381 ->
   // 372 us.
@@ -266,10 +266,11 @@ static cudaError_t apply_r(const HostProblem& hp, const DeviceData& dd, const Ch
   OrdArgs oa{ct.ord, ct.add_bits, ct.deps, ct.ndeps, ct.done, ct.tickets, dd.err_flag, ct.n,
              ct.dep_cap};
   const int nl0 = nlaunch;
-  if (reg) {                 // tile shape 2: one thread per cell (cell_reg.cu)
+  if (reg) {                 // one or n threads per cell (cell_reg.cu, cell_plane.cu)
     if constexpr (std::is_same<T, float>::value) {
-      if ((err = launch_cell_reg(hp, dd, x, y, fo, ycol, st, pdl_cell)) != cudaSuccess)
-        return err;
+      err = cell_reg_used(hp) ? launch_cell_reg(hp, dd, x, y, fo, ycol, st, pdl_cell)
+                              : launch_cell_plane(hp, dd, x, y, fo, ycol, st, pdl_cell);
+      if (err != cudaSuccess) return err;
       nlaunch++;
     }
   } else if (ord && part.q1 > part.q0) {      // colour-ordered stores, no assembly
@@ -341,9 +342,9 @@ static cudaError_t apply_r(const HostProblem& hp, const DeviceData& dd, const Ch
 }
 
 // variant 0: R cells per chunk; variant 1: R/2 (a second tile shape for the
-// autotuner); variant 2: the cells of variant 0's chunks one thread each
-// (cell_reg.cu; whole applies only -- a slab of the host pipeline runs
-// variant 0, which gives the same bits); variant 3 (3D): variant 0's chunks
+// autotuner); variant 2: the cells of variant 0's chunks one thread or n
+// threads each (FP32, whole applies; FP64 runs variant 0, which gives the same
+// bits); variant 3 (3D): variant 0's chunks
 // without staged runs (chunk_loop_direct; slabs too).  Both chunkings are built at set-up
 // with the same colouring rule, so the variants give bitwise-equal results.
 template <typename T, int D, int N>
@@ -353,9 +354,14 @@ static cudaError_t apply_t(const HostProblem& hp, const DeviceData& dd, const T*
   constexpr int R = ChunkShape<D, N>::R;
   constexpr int RH = (R / 2) > 0 ? R / 2 : 1;
   const int v = (variant == 1 && RH < R) ? 1 : 0;
-  // (FP64 runs variant 2 as variant 0, which gives the same bits)
-  const bool reg = std::is_same<T, float>::value && variant == 2 && slab < 0 && nrhs == 1 &&
-                   cell_reg_available(hp, true);
+  // FP32 whole applies of shapes 0 and 2 run the register kernels, which give
+  // the same bits and were faster than the chunk kernel at every degree and size
+  // measured (us, chunk kernel / shape 3 / register kernels: p = 1 128^3 47.5 /
+  // 35.1 / 24.8, p = 2 96^3 55.6 / 42.3 / 24.4, p = 3 105 / 78.9 / 55.4, p = 4
+  // 195 / 153 / 114, p = 5 64^3 109 / 88.6 / 77, p = 6 48^3 60 / 48.9 / 46.1,
+  // p = 4 32^3 20.6 / 15.8 / 16.7: the autotuner still has shape 3)
+  const bool reg = std::is_same<T, float>::value && D == 3 && slab < 0 && nrhs == 1 &&
+                   (variant == 2 || (variant == 0 && !ordered));
   const bool direct = variant == 3 && D == 3;
   const ChunkTable& ct = dd.chunks[v];
   // colour-ordered stores: whole single applies of chunking 0 by the chunk

@@ -154,13 +154,19 @@ struct DeviceData {
   ChunkTable chunks[2];          // CG: R and R/2 cells per chunk (two tile shapes)
   int variant[2] = {0, 0};       // tile shape of the single applies: [FP64, FP32]
   bool ordered[2] = {false, false};  // colour-ordered stores instead of the assembly
-  // tile shape 2 (3D CG, n <= 5; cell_reg.cu): one thread per cell on the
-  // chunks of shape 0 -- chunk of every ordered cell, blocks of whole
-  // chunks, per-cell bits of the nodes several colours share
+  // FP32 whole applies (3D CG) on the chunks of shape 0: chunk of every
+  // ordered cell, blocks of whole chunks, bits of the nodes several colours
+  // share; n <= 3 one thread per cell (cell_reg.cu; bits per cell), above n
+  // threads per cell (cell_plane.cu; bits per x-plane, x-line operators)
   int32_t* reg_cell_chunk = nullptr;
   int32_t* reg_block_first = nullptr;
   uint32_t* reg_mask = nullptr;
   int reg_nblocks = 0;
+  int32_t* plane_cell_chunk = nullptr;
+  int32_t* plane_block_first = nullptr;
+  uint32_t* plane_mask = nullptr;
+  float* plane_xops = nullptr;
+  int plane_nblocks = 0;
   int32_t* diag_pos = nullptr;   // CG: ordered positions grouped by cell parity (diagonal)
   std::vector<int> diag_col_start;
   double* ycol = nullptr;        // CG [ncolours * n_dofs] colour accumulation buffers (scratch)
@@ -260,14 +266,21 @@ cudaError_t launch_maybe_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size
   return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
-// Tile shape 2: the cell term with one thread per cell and the tile in
-// registers (cell_reg.cu); accepted for 3D CG problems with n <= 5 (FP32) or
-// n <= 4 (FP64, which runs shape 0 instead); bitwise equal to tile shape 0.
+// FP32 whole applies of 3D CG problems on the chunks of shape 0, bitwise equal
+// to the chunk kernel: one thread per cell (n <= 3), n threads per cell (n >= 4).
+// cell_reg_available: what tile shape 2 is accepted for.
 bool cell_reg_available(const HostProblem& hp, bool fp32);
+bool cell_reg_used(const HostProblem& hp);
 cudaError_t build_cell_reg_tables(const HostProblem& hp, const std::vector<int32_t>& ch_first,
                                   DeviceData* dd);
 cudaError_t launch_cell_reg(const HostProblem& hp, const DeviceData& dd, const float* x, float* y,
                             const float* fo, float* ycol, cudaStream_t st, bool pdl = false);
+bool cell_plane_used(const HostProblem& hp);
+cudaError_t build_cell_plane_tables(const HostProblem& hp, const std::vector<int32_t>& ch_first,
+                                    DeviceData* dd);
+cudaError_t launch_cell_plane(const HostProblem& hp, const DeviceData& dd, const float* x,
+                              float* y, const float* fo, float* ycol, cudaStream_t st,
+                              bool pdl = false);
 
 // The surrogate faces [fb, fe) of the kernel face order (all: 0, -1) into
 // the per-face scratch (face_kernel.cu).

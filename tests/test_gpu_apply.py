@@ -115,6 +115,14 @@ def test_host_entry_point_equals_device_apply(w):
         np.testing.assert_array_equal(yp, yd)
 
 
+@pytest.mark.parametrize("w", [S.SPHERE_3D_Q4.resized(32), S.SPHERE_3D_Q4.resized(60),
+                               S.DISK_2D_Q2.resized(400, degree=4)], ids=lambda w: w.name)
+def test_host_entry_point_with_several_slabs(w):
+    """The same on vectors of 3 MB and more, which the pipeline cuts into 2 to 5 slabs."""
+    test_host_entry_point_equals_device_apply(w)
+
+
+
 def _sample_rows(O, rng, nrand=10000, nface_cells=200):
     rows = rng.choice(O.n_dofs, size=min(nrand, O.n_dofs), replace=False)
     fc = np.unique(O.mesh.sfaces[:, 0])

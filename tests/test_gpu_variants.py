@@ -85,3 +85,36 @@ def test_f32_apply_error_vs_oracle(w):
     err = _rel(y, ref)
     print(f"{w.name}: fp32 rel err {err:.3e}")
     assert err <= 5e-7
+
+
+@pytest.mark.parametrize("w", [w for w in DG_CASES if w.dim == 3], ids=lambda w: w.name)
+def test_f32_dg_apply_error_vs_oracle(w):
+    """The FP32 line operators of the 3D DG apply, to test_f32_apply_error_vs_oracle's bound."""
+    O = OracleProblem.from_workload(w)
+    P = G.Problem.from_workload(w)
+    x = S.random_vector(w.seed, O.n_dofs, w.dist)
+    y = P.apply_f32(torch.from_numpy(x).float().cuda()).double().cpu().numpy()
+    ref = O.apply(x.astype(np.float32).astype(np.float64))
+    assert _rel(y, ref) <= 5e-7
+
+
+@pytest.mark.parametrize("cells", [5, 23, 40])
+@pytest.mark.parametrize("p", range(1, 7))
+def test_register_kernels_equal_chunk_kernels_bitwise(p, cells):
+    """FP32 applies by one or n threads per cell (shape 0) against the chunks
+    without staged runs (shape 3) and, where built, with colour-ordered stores:
+    mesh rows of 1 to 33 active cells, so chunks of every length and blocks
+    that end anywhere."""
+    w = S._wl("ball", 3, p, cells, S.ball(3, (0.02, 0.01, -0.03), 0.81), seed=7)
+    P = G.Problem.from_workload(w)
+    x = torch.from_numpy(S.random_vector(7, P.n_dofs, "uniform")).float().cuda()
+    G.sbm_set_tile_shape(P.handle, 0, 0)
+    y = P.apply_f32(x)
+    G.sbm_set_tile_shape(P.handle, 0, 3)
+    assert torch.equal(P.apply_f32(x), y)
+    G.sbm_set_tile_shape(P.handle, 0, 0)
+    try:
+        G.sbm_set_ordered_stores(P.handle, -1, 1)
+    except G.SbmError:
+        return
+    assert torch.equal(P.apply_f32(x), y)
