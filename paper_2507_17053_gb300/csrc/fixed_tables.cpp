@@ -350,6 +350,10 @@ bool build_fixed_tables(const Tables1D& tb, double scale, FixedTables* out, doub
   out->face_etm = 2 - tD + 2 * (61 - tM);
   // DG line operators: row i of K u + sum_s Own_s g_s, |g| <= 2 |u|, scaled to
   // leave 57-bit values at 59 bits (K = 3); hm goes into the entries
+  // a penalty that is not finite: the results are NaN
+  out->dg = fix::DgTab{};
+  out->dg.eoff = fix::kFaceExpBad;
+  if (!std::isfinite(pen)) return true;
   DD w[kMaxN];
   for (int j = 0; j < n; ++j) w[j] = j ? P.D0[j] * DD(0.5) : DD(pen) + P.D0[0];
   double sw = 0.0, B1 = 0.0;
@@ -361,11 +365,7 @@ bool build_fixed_tables(const Tables1D& tb, double scale, FixedTables* out, doub
     r += 2.0 * (i == n - 1 ? sw : mag(w[n - 1 - i]));
     B1 = std::max(B1, r);
   }
-  out->dg = fix::DgTab{};
-  if (!std::isfinite(B1)) {
-    out->dg.eoff = fix::kFaceExpBad;
-    return true;
-  }
+  if (!std::isfinite(B1)) return true;
   const int tR = fit(B1) - 1;
   auto folded = [&](const DD (&A)[kMaxN][kMaxN], int t, double f, fix::Block* o) {
     for (int i = 0; i < HE; ++i)

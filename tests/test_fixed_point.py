@@ -276,8 +276,28 @@ int dg_lines(double pen) {
   return bad;
 }
 
+// Penalties that are not finite, or whose row sums overflow, never become finite tables.
+template <int N>
+int dg_non_finite() {
+  int bad = 0;
+  Tables1D tb;
+  build_tables(N - 1, &tb);
+  for (double pen : {std::numeric_limits<double>::infinity(),
+                     std::numeric_limits<double>::quiet_NaN(),
+                     std::numeric_limits<double>::max()}) {
+    FixedTables ft;
+    if (!build_fixed_tables(tb, 1.0, &ft, pen) || ft.dg.eoff != fix::kFaceExpBad) {
+      std::printf("n=%d pen %g: eoff %d\n", N, pen, ft.dg.eoff);
+      bad = 1;
+    }
+  }
+  return bad;
+}
+
 int main() {
   int bad = conversions();
+  bad |= dg_non_finite<2>() | dg_non_finite<3>() | dg_non_finite<4>() | dg_non_finite<5>() |
+         dg_non_finite<6>() | dg_non_finite<7>();
   for (double pen : {1.0, 49.0, 1e6}) {
     bad |= dg_lines<2>(pen) | dg_lines<3>(pen) | dg_lines<4>(pen) | dg_lines<5>(pen) |
            dg_lines<6>(pen) | dg_lines<7>(pen);
