@@ -159,7 +159,15 @@ dg_apply_kernel(const DgArgs<T> a, const __grid_constant__ KTab<T> t) {
 // FP64 runs on the integer units (fixed_point.cuh): the exponent of a cell is
 // the largest of its own and its neighbours', from dg_exp_kernel; r_k of
 // 57-bit values leaves at 59 bits, so that the sum of the last phase stays
-// below 2^61.
+// below 2^61.  The penalty is a part of w, and so of that scale, only while it
+// no more than doubles the largest row sum (pen_interior = 1 gives 1.1 to 1.7
+// times the sum without it).  A larger one would take the low bits of K u and
+// of the jump with it, which a conforming u shows: error of a line whose traces
+// match, against 128-bit tables, at up to twice the sum without penalty 4.2e-17
+// (p = 1) .. 4.9e-14 (p = 6), in double precision 1.3e-15 .. 8.0e-14; at 8 to 14
+// times 6.4e-16 .. 2.9e-13 against the same.  There dg_penalty adds it in double
+// precision from the exact jumps (whole applies, inside / added: p = 1 of 656 832
+// DoFs 29 / 50 us, p = 3 of 1.57 M 60 / 97, p = 6 of 2.05 M 113 / 164).
 //
 // Measured on GB300, whole applies, before (cell term, then six faces through
 // traces, mass products and folds) -> now: FP64 torus of 64^3 cells at p = 3
@@ -304,8 +312,69 @@ dg_exp_kernel(const double* __restrict__ x, int32_t* __restrict__ e, int ncell) 
   pdl_wait();                      // done only after the face kernel: the next one waits for both
 }
 
-template <typename T, int N>
-__global__ void __launch_bounds__(Dg3<T, N>::NT, std::is_same<T, double>::value && N > 4 ? 3 : 4)
+// The penalty terms of a cell's interior faces, added to the z-line (la, lb) of
+// the result: h^2 M x M (sigma_F (own - neighbour)) on the face's nodes.  By the
+// whole block, the shared memory free: 6 n^2 doubles per cell, in place.
+template <int N>
+__device__ __forceinline__ void dg_penalty(const DgArgs<double>& a, const KTab<double>& t,
+                                           unsigned char* smem_raw, int rank, const int (&nb)[6],
+                                           int c, int tl, bool act, double (&out)[N]) {
+  constexpr int L = N * N, ND = L * N;
+  const int la = tl % N, lb = tl / N;
+  double* P = reinterpret_cast<double*>(smem_raw) + (act ? c : 0) * 6 * L;
+  double w[6];
+  if (act) {
+#pragma unroll
+    for (int f = 0; f < 6; ++f) {
+      const int k = f / 2, sk = k == 0 ? 1 : k == 1 ? N : L;
+      const int bt = la * (k == 0 ? N : 1) + lb * (k == 2 ? N : L);
+      const int own = bt + (f % 2 ? (N - 1) * sk : 0), other = bt + (f % 2 ? 0 : (N - 1) * sk);
+      w[f] = 0.0;
+      if (nb[f] >= 0)
+        w[f] = t.hface * (a.sigma_f * (__ldg(a.x + (size_t)rank * ND + own) -
+                                       __ldg(a.x + (size_t)nb[f] * ND + other)));
+    }
+  }
+#pragma unroll
+  for (int ax = 0; ax < 2; ++ax) {            // M along the two axes of the faces
+    __syncthreads();
+    if (act) {
+#pragma unroll
+      for (int f = 0; f < 6; ++f) P[f * L + tl] = w[f];
+    }
+    __syncthreads();
+    if (act) {
+#pragma unroll
+      for (int f = 0; f < 6; ++f) {
+        w[f] = 0.0;
+#pragma unroll
+        for (int j = 0; j < N; ++j)
+          w[f] = fma(t.M[ax ? lb : la][j], P[f * L + (ax ? la + N * j : j + N * lb)], w[f]);
+      }
+    }
+  }
+  __syncthreads();
+  if (act) {
+#pragma unroll
+    for (int f = 0; f < 4; ++f) P[f * L + tl] = w[f];
+  }
+  __syncthreads();
+  if (!act) return;
+#pragma unroll
+  for (int m = 0; m < N; ++m) {               // node (la, lb, m): x-faces (lb, m), y-faces (la, m)
+    if (la == 0) out[m] += P[lb + N * m];
+    if (la == N - 1) out[m] += P[L + lb + N * m];
+    if (lb == 0) out[m] += P[2 * L + la + N * m];
+    if (lb == N - 1) out[m] += P[3 * L + la + N * m];
+  }
+  out[0] += w[4];
+  out[N - 1] += w[5];
+}
+
+// PEN: the penalty is not part of the line operators (FP64)
+template <typename T, int N, bool PEN>
+__global__ void __launch_bounds__(Dg3<T, N>::NT,
+                                  std::is_same<T, double>::value && N > 4 ? (PEN ? 2 : 3) : 4)
 dg3_kernel(const DgArgs<T> a, const __grid_constant__ KTab<T> t,
            const __grid_constant__ DgTabs<T> d) {
   using Sh = Dg3<T, N>;
@@ -394,7 +463,7 @@ dg3_kernel(const DgArgs<T> a, const __grid_constant__ KTab<T> t,
     for (int j = 0; j < N; ++j) Z[xl + j] = y[j];
   }
   FixMap<N>::sync(tid);
-  if (!act) return;
+  if (!PEN && !act) return;
   T out[N];                        // z-lines, back to the nodes read first
 #pragma unroll
   for (int j = 0; j < N; ++j) v[j] = X[zl + PL * j];
@@ -403,7 +472,7 @@ dg3_kernel(const DgArgs<T> a, const __grid_constant__ KTab<T> t,
   for (int j = 0; j < N; ++j) y[j] += Z[zl + PL * j];
   if constexpr (FX) {
     const int eo = d.x.eoff;
-    const bool bad = E == fix::kExpBad || eo == fix::kFaceExpBad;
+    const bool bad = E == fix::kExpBad;
     const bool plain = fix::plain_exp(E) && abs(eo) <= 64;
 #pragma unroll
     for (int j = 0; j < N; ++j) {
@@ -414,6 +483,10 @@ dg3_kernel(const DgArgs<T> a, const __grid_constant__ KTab<T> t,
   } else {
 #pragma unroll
     for (int j = 0; j < N; ++j) out[j] = y[j];
+  }
+  if constexpr (PEN) {
+    dg_penalty<N>(a, t, smem_raw, rank, nb, c, tl, act, out);
+    if (!act) return;
   }
   const int fs = __ldg(a.face_start + first + c), fe = __ldg(a.face_start + first + c + 1);
   if (!FX && fs < fe) pdl_wait();  // the face kernel's results
@@ -433,14 +506,14 @@ static DgTabs<float> dg_tabs(const HostProblem& hp, float) {
   return d;
 }
 
-template <typename T, int N>
+template <typename T, int N, bool PEN>
 static cudaError_t dg3_t(const HostProblem& hp, const DeviceData& dd, const T* x, T* y,
                          cudaStream_t st, Profiler* prof, int face_mode) {
   using Sh = Dg3<T, N>;
   constexpr bool FX = std::is_same<T, double>::value;
   static cudaError_t attr =
       Sh::smem > 48 * 1024
-          ? cudaFuncSetAttribute(dg3_kernel<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+          ? cudaFuncSetAttribute(dg3_kernel<T, N, PEN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)Sh::smem)
           : cudaSuccess;
   if (attr != cudaSuccess) return attr;
@@ -453,6 +526,7 @@ static cudaError_t dg3_t(const HostProblem& hp, const DeviceData& dd, const T* x
   a.face_kind = dd.face_kind;
   a.face_out = face_out_of<T>(dd);
   a.cexp = dd.dg_exp;
+  a.sigma_f = (T)hp.sigma_f;
   a.ncell = dd.col_start[dd.ncolours];
   if (a.ncell == 0) return cudaSuccess;
   const bool pr = prof && prof->on;
@@ -477,7 +551,7 @@ static cudaError_t dg3_t(const HostProblem& hp, const DeviceData& dd, const T* x
     pdl = !pr;
   }
   const unsigned grid = (unsigned)((a.ncell + Sh::R - 1) / Sh::R);
-  if ((err = launch_maybe_pdl(dg3_kernel<T, N>, dim3(grid), dim3(Sh::NT), Sh::smem, st, pdl, a,
+  if ((err = launch_maybe_pdl(dg3_kernel<T, N, PEN>, dim3(grid), dim3(Sh::NT), Sh::smem, st, pdl, a,
                               make_ktab<T>(hp), dg_tabs(hp, T(0)))) != cudaSuccess)
     return err;
   if (pr) {
@@ -526,10 +600,13 @@ static cudaError_t dg2_t(const HostProblem& hp, const DeviceData& dd, const T* x
 template <typename T>
 cudaError_t launch_dg_apply(const HostProblem& hp, const DeviceData& dd, const T* x, T* y,
                             cudaStream_t st, Profiler* prof, int face_mode) {
+  constexpr bool FX = std::is_same<T, double>::value;
 #define SBM_CASE(NN)                                                                     \
   if (hp.n == NN)                                                                        \
-    return hp.d == 2 ? dg2_t<T, NN>(hp, dd, x, y, st, prof, face_mode)                   \
-                     : dg3_t<T, NN>(hp, dd, x, y, st, prof, face_mode);
+    return hp.d == 2          ? dg2_t<T, NN>(hp, dd, x, y, st, prof, face_mode)          \
+           : hp.fx.dg_pen_in || !FX                                                      \
+               ? dg3_t<T, NN, false>(hp, dd, x, y, st, prof, face_mode)                  \
+               : dg3_t<T, NN, FX>(hp, dd, x, y, st, prof, face_mode);
   SBM_CASE(2) SBM_CASE(3) SBM_CASE(4) SBM_CASE(5) SBM_CASE(6) SBM_CASE(7)
 #undef SBM_CASE
   return cudaErrorInvalidValue;

@@ -59,8 +59,9 @@ struct Block {
 };
 
 // Line operators of the 3D DG apply (dg_apply.cu): K and M folded, and the
-// interior-face vector w (w[0] = pen + D0[0], w[j] = D0[j] / 2); the result's
-// exponent word is E + eoff (kFaceExpBad: a non-finite penalty).
+// interior-face vector w (w[0] = pen + D0[0], without pen where the apply adds
+// the penalty in double; w[j] = D0[j] / 2); the result's exponent word is
+// E + eoff.
 struct DgTab {
   Block K, M;
   Entry w[2 * kMaxHalf];

@@ -349,23 +349,31 @@ bool build_fixed_tables(const Tables1D& tb, double scale, FixedTables* out, doub
   out->face_eq = 2 + 2 * (61 - tS);
   out->face_etm = 2 - tD + 2 * (61 - tM);
   // DG line operators: row i of K u + sum_s Own_s g_s, |g| <= 2 |u|, scaled to
-  // leave 57-bit values at 59 bits (K = 3); hm goes into the entries
-  // a penalty that is not finite: the results are NaN
-  out->dg = fix::DgTab{};
-  out->dg.eoff = fix::kFaceExpBad;
-  if (!std::isfinite(pen)) return true;
+  // leave 57-bit values at 59 bits (K = 3); hm goes into the entries.  The
+  // penalty is part of them while it no more than doubles the largest row sum
+  // (dg_apply.cu; a sum that overflows or is NaN does not pass).
   DD w[kMaxN];
-  for (int j = 0; j < n; ++j) w[j] = j ? P.D0[j] * DD(0.5) : DD(pen) + P.D0[0];
-  double sw = 0.0, B1 = 0.0;
-  for (int j = 0; j < n; ++j) sw += mag(w[j]);
-  for (int i = 0; i < n; ++i) {
-    double r = 0.0;
-    for (int j = 0; j < n; ++j) r += mag(P.K[i][j]);
-    r += 2.0 * (i == 0 ? sw : mag(w[i]));
-    r += 2.0 * (i == n - 1 ? sw : mag(w[n - 1 - i]));
-    B1 = std::max(B1, r);
+  for (int j = 0; j < n; ++j) w[j] = j ? P.D0[j] * DD(0.5) : P.D0[0];
+  auto row_sums = [&](double w0) {
+    double sw = w0, B = 0.0;
+    for (int j = 1; j < n; ++j) sw += mag(w[j]);
+    for (int i = 0; i < n; ++i) {
+      double r = 0.0;
+      for (int j = 0; j < n; ++j) r += mag(P.K[i][j]);
+      r += 2.0 * (i == 0 ? sw : mag(w[i]));
+      r += 2.0 * (i == n - 1 ? sw : mag(w[n - 1 - i]));
+      if (!(r <= B)) B = r;
+    }
+    return B;
+  };
+  double B1 = row_sums(mag(w[0]));
+  const double B1p = row_sums(std::fabs(pen + w[0].h));
+  out->dg_pen_in = B1p <= 2.0 * B1;
+  if (out->dg_pen_in) {
+    w[0] = DD(pen) + w[0];
+    B1 = B1p;
   }
-  if (!std::isfinite(B1)) return true;
+  out->dg = fix::DgTab{};
   const int tR = fit(B1) - 1;
   auto folded = [&](const DD (&A)[kMaxN][kMaxN], int t, double f, fix::Block* o) {
     for (int i = 0; i < HE; ++i)

@@ -19,6 +19,7 @@ struct FixedTables {
   std::vector<fix::Entry> face;
   int face_eq = 0, face_etm = 0;
   fix::DgTab dg;                     // discontinuous Galerkin line operators (dg_apply.cu)
+  bool dg_pen_in = true;             // the penalty is in dg.w[0] (else added in double)
 };
 
 // Tables of the pencil of t for the cell operator scaled by scale = h^(d-2);

@@ -223,6 +223,7 @@ int dg_lines(double pen) {
   FixedTables ft;
   if (!build_fixed_tables(tb, 1.0, &ft, pen)) return 1;
   const fix::DgTab& d = ft.dg;
+  if (!ft.dg_pen_in) pen = 0.0;           // added elsewhere, in double
   auto Kf = [&](int i, int j) {           // the row's sign pattern from the folded blocks
     const fix::Entry e = d.K.E[std::min(i, N - 1 - i)][std::min(j, N - 1 - j)];
     if ((N & 1) && (i == H || j == H)) return (double)e.h;
@@ -276,28 +277,160 @@ int dg_lines(double pen) {
   return bad;
 }
 
-// Penalties that are not finite, or whose row sums overflow, never become finite tables.
+// The 1D tables in long double: stiffness, end derivatives.
 template <int N>
-int dg_non_finite() {
+struct Exact {
+  long double x[N], K[N][N] = {}, D[2][N];
+  static void legendre(int m, long double t, long double* P, long double* dP) {
+    long double p0 = 1, p1 = t;
+    for (int k = 1; k < m; ++k) {
+      const long double p2 = ((2 * k + 1) * t * p1 - k * p0) / (k + 1);
+      p0 = p1;
+      p1 = p2;
+    }
+    *P = p1;
+    *dP = m * (p0 - t * p1) / (1 - t * t);
+  }
+  void lagrange(long double s, long double* dv) const {
+    for (int j = 0; j < N; ++j) {
+      long double a = 1, b = 0;
+      for (int m = 0; m < N; ++m) {
+        if (m == j) continue;
+        b = (b * (s - x[m]) + a) / (x[j] - x[m]);
+        a = a * (s - x[m]) / (x[j] - x[m]);
+      }
+      dv[j] = b;
+    }
+  }
+  explicit Exact(const Tables1D& tb) {
+    const int p = N - 1;
+    for (int j = 0; j < N; ++j) {
+      long double s = 2 * (long double)tb.nodes[j] - 1, L, d;
+      for (int it = 0; it < 4 && j > 0 && j < p; ++it) {
+        legendre(p, s, &L, &d);
+        s -= d * (1 - s * s) / (2 * s * d - p * (p + 1) * L);
+      }
+      x[j] = (s + 1) / 2;
+    }
+    for (int q = 0; q < N; ++q) {
+      long double s = 2 * (long double)tb.gpts[q] - 1, L, d, dv[N];
+      for (int it = 0; it < 4; ++it) {
+        legendre(N, s, &L, &d);
+        s -= L / d;
+      }
+      legendre(N, s, &L, &d);
+      lagrange((s + 1) / 2, dv);
+      for (int i = 0; i < N; ++i)
+        for (int j = 0; j < N; ++j) K[i][j] += dv[i] * dv[j] / ((1 - s * s) * d * d);
+    }
+    lagrange(0, D[0]);
+    lagrange(1, D[1]);
+  }
+};
+
+// The DG line operator on smooth lines whose traces match the neighbours': no penalty of
+// any size may cost accuracy.  |error| <= 2^-52 B max |u|, B the largest row sum without
+// penalty: the operator's is at most 2 B, inputs are cut at 2^-56 of max |u|, at most 8
+// roundings at 2^-57 of the row sum follow.
+template <int N>
+int dg_matching(double pen) {
   int bad = 0;
   Tables1D tb;
   build_tables(N - 1, &tb);
+  const Exact<N> T(tb);
+  FixedTables ft;
+  if (!build_fixed_tables(tb, 1.0, &ft, pen)) return 1;
+  const fix::DgTab& d = ft.dg;
+  const fix::Entry m = ft.face[N];        // tM as in dg_lines
+  const int tM = (int)std::lround(std::log2(((double)m.h * 0x1p30 + 0.5 * m.l) / tb.M[0][0]));
+  const int unit = d.eoff - 2 * (61 - tM) - 1023;
+  double B = 0;
+  for (int i = 0; i < N; ++i) {
+    double r = 0, sw = 0;
+    for (int j = 0; j < N; ++j) {
+      r += std::fabs(tb.K[i][j]);
+      sw += std::fabs(tb.D0[j]) * (j ? 0.5 : 1.0);
+    }
+    r += i == 0 || i == N - 1 ? 2 * sw + std::fabs(tb.D0[N - 1])
+                              : std::fabs(tb.D0[i]) + std::fabs(tb.D0[N - 1 - i]);
+    B = std::max(B, r);
+  }
+  for (int trial = 0; trial < 200; ++trial) {
+    const double k = 1.0 + 2.0 * std::fabs(rnd()), ph = 3.0 * rnd();
+    double v[N], nb[2][N], big = 0;
+    for (int j = 0; j < N; ++j) {
+      v[j] = std::sin(k * tb.nodes[j] + ph);
+      nb[0][j] = std::sin(k * (tb.nodes[j] - 1) + ph);
+      nb[1][j] = std::sin(k * (tb.nodes[j] + 1) + ph);
+    }
+    nb[0][N - 1] = v[0];
+    nb[1][0] = v[N - 1];
+    for (int j = 0; j < N; ++j)
+      big = std::max({big, std::fabs(v[j]), std::fabs(nb[0][j]), std::fabs(nb[1][j])});
+    const int E = (int)(fix::mag_hi(bits(big)) >> 20);
+    int64_t q[N], y[N], g[2][N];
+    for (int j = 0; j < N; ++j) q[j] = fix::from_double<false>(bits(v[j]), E) >> 3;
+    fix::apply_line<N, 3>([&](int i, int j) { return d.K.E[i][j]; },
+                          [&](int i, int j) { return d.K.O[i][j]; }, q, y);
+    for (int s = 0; s < 2; ++s) {
+      fix::Split w[N];
+      for (int j = 0; j < N; ++j) {
+        g[s][j] = q[j] - (fix::from_double<false>(bits(nb[s][N - 1 - j]), E) >> 3);
+        w[j] = fix::split(g[s][j]);
+      }
+      y[s ? N - 1 : 0] += fix::dot<3, N>([&](int j) { return d.w[s ? N - 1 - j : j]; }, w);
+    }
+    const fix::Split e0 = fix::split(g[0][0]), e1 = fix::split(g[1][N - 1]);
+    for (int j = 0; j < N; ++j) {
+      const fix::Split q1[1] = {j ? e0 : e1}, q2[2] = {e0, e1};
+      if (j == 0 || j == N - 1) y[j] += fix::dot<3, 1>([&](int) { return d.w[N - 1]; }, q1);
+      else y[j] += fix::dot<3, 2>([&](int i) { return d.w[i ? N - 1 - j : j]; }, q2);
+    }
+    for (int i = 0; i < N; ++i) {
+      long double r = 0;
+      for (int j = 0; j < N; ++j) r += T.K[i][j] * v[j];
+      for (int s = 0; s < 2; ++s)
+        for (int j = 0; j < N; ++j)
+          if (i == (s ? N - 1 : 0))
+            r -= (s ? 0.5L : -0.5L) * (T.D[s][j] * v[j] + T.D[!s][j] * nb[s][j]);
+      const double err = (double)std::fabs(std::ldexp((long double)y[i], unit + E) - r);
+      if (!(err <= 0x1p-52 * B * big)) {
+        std::printf("dg traces n=%d pen %g row %d: %g\n", N, pen, i, err);
+        return 1;
+      }
+    }
+  }
+  return bad;
+}
+
+// A penalty that is not finite, or whose row sums overflow, is not in the tables.
+template <int N>
+int dg_non_finite() {
+  Tables1D tb;
+  build_tables(N - 1, &tb);
+  FixedTables f0;
+  if (!build_fixed_tables(tb, 1.0, &f0, 0.0) || !f0.dg_pen_in) return 1;
   for (double pen : {std::numeric_limits<double>::infinity(),
                      std::numeric_limits<double>::quiet_NaN(),
                      std::numeric_limits<double>::max()}) {
     FixedTables ft;
-    if (!build_fixed_tables(tb, 1.0, &ft, pen) || ft.dg.eoff != fix::kFaceExpBad) {
+    if (!build_fixed_tables(tb, 1.0, &ft, pen) || ft.dg_pen_in ||
+        std::memcmp(&ft.dg, &f0.dg, sizeof(ft.dg))) {
       std::printf("n=%d pen %g: eoff %d\n", N, pen, ft.dg.eoff);
-      bad = 1;
+      return 1;
     }
   }
-  return bad;
+  return 0;
 }
 
 int main() {
   int bad = conversions();
   bad |= dg_non_finite<2>() | dg_non_finite<3>() | dg_non_finite<4>() | dg_non_finite<5>() |
          dg_non_finite<6>() | dg_non_finite<7>();
+  for (double pen : {4.0, 49.0, 490.0, 4.9e3, 4.9e7, 1e10}) {
+    bad |= dg_matching<2>(pen) | dg_matching<3>(pen) | dg_matching<4>(pen) |
+           dg_matching<5>(pen) | dg_matching<6>(pen) | dg_matching<7>(pen);
+  }
   for (double pen : {1.0, 49.0, 1e6}) {
     bad |= dg_lines<2>(pen) | dg_lines<3>(pen) | dg_lines<4>(pen) | dg_lines<5>(pen) |
            dg_lines<6>(pen) | dg_lines<7>(pen);

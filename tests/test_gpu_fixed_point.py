@@ -1,11 +1,15 @@
 """The fixed-point FP64 cell term on the GPU: exponent range and non-finite
 values (the arithmetic itself: test_fixed_point.py, and every FP64 apply test)."""
+import dataclasses
+
 import numpy as np
 import pytest
 import torch
 
 import paper_2507_17053_gb300 as G
 import synthetic as S
+from oracle import local
+from oracle.operator import Problem as OracleProblem
 
 pytestmark = pytest.mark.gpu
 
@@ -63,3 +67,78 @@ def test_non_finite_input_stays_in_its_cells(w, value):
         fin = torch.isfinite(yb)
         assert torch.equal(yb[fin], y[fin])
         assert int((~fin).sum()) <= 8 * (w.degree + 1) ** 3
+
+
+# ---- discontinuous Galerkin: interior-face penalties of every size -----------------
+
+DG_BOX = S._wl("box", 3, 2, 5, S.box((0.0,) * 3, (1.5,) * 3), dg=True, seed=5)
+PENALTIES = [1.0, 2.0, 30.0, 1e3, 1e6, 1e9]    # inside the line operators up to about 3
+
+
+def _dg(p, pen=1.0):
+    w = dataclasses.replace(DG_BOX.resized(5, degree=p), pen_interior=pen)
+    return w, G.Problem.from_workload(w)
+
+
+def _inner_cells(O):
+    """Rows of the cells without surrogate faces."""
+    rows = np.ones(len(O.mesh.cells), bool)
+    rows[O.mesh.sfaces[:, 0]] = False
+    return O.dofmap[rows].ravel()
+
+
+@pytest.mark.parametrize("p", range(1, 7))
+def test_dg_penalty_costs_conforming_data_nothing(p):
+    """Data with equal traces: the penalty multiplies zeros, so the apply at
+    any penalty is the one at pen_interior = 1, to test_gpu_apply's bound and
+    on the cells without surrogate faces relative to their own values."""
+    O = OracleProblem.from_workload(_dg(p)[0])
+    X = np.sin(np.arange(5 * p + 1) * 0.37 + 0.2)      # by lattice index: traces equal bitwise
+    lat = p * O.mesh.cells[:, None, :] + local.tensor_index(p + 1, 3)
+    x = np.empty(O.n_dofs)
+    x[O.dofmap] = X[lat[..., 0]] + 0.5 * X[lat[..., 1]] * X[lat[..., 2]]
+    ref, rows = O.apply(x), _inner_cells(O)
+    xd = torch.from_numpy(x).cuda()
+    for pen in PENALTIES:
+        y = _dg(p, pen)[1].apply_f64(xd).cpu().numpy()
+        assert np.abs(y - ref).max() <= 1e-12 * np.abs(ref).max(), pen
+        assert np.abs(y - ref)[rows].max() <= 1e-12 * np.abs(ref[rows]).max(), pen
+
+
+@pytest.mark.parametrize("p", range(1, 7))
+def test_dg_penalty_on_jumps(p):
+    """Random data against the oracle; a node inside a cell does not see the
+    penalty (its test function vanishes on the faces): to the same bound
+    relative to such nodes' own values."""
+    O1 = OracleProblem.from_workload(_dg(p)[0])
+    x = S.random_vector(5, O1.n_dofs, "uniform")
+    xd = torch.from_numpy(x).cuda()
+    ref1 = O1.apply(x)
+    mi = local.tensor_index(p + 1, 3)
+    inside = O1.dofmap[:, np.all((mi > 0) & (mi < p), axis=1)].ravel()
+    for pen in PENALTIES:
+        w, P = _dg(p, pen)
+        y = P.apply_f64(xd).cpu().numpy()
+        ref = OracleProblem.from_workload(w).apply(x)
+        assert np.abs(y - ref).max() <= 1e-12 * np.abs(ref).max(), pen
+        if inside.size:
+            assert np.abs(y - ref1)[inside].max() <= 1e-12 * np.abs(ref1[inside]).max(), pen
+
+
+@pytest.mark.parametrize("p", range(1, 7))
+def test_dg_penalty_not_finite(p):
+    """An infinite penalty (or one that overflows in (p+1)^2 / h) shows on the
+    nodes of interior faces; the others are those of pen_interior = 1."""
+    w, P = _dg(p)
+    O = OracleProblem.from_workload(w)
+    xd = torch.from_numpy(S.random_vector(5, O.n_dofs, "uniform")).cuda()
+    y1 = P.apply_f64(xd).cpu().numpy()
+    mi = local.tensor_index(p + 1, 3)
+    seen = np.zeros(O.n_dofs, bool)
+    for c1, k, c2 in O.mesh.ifaces:
+        seen[O.dofmap[c1][mi[:, k] == p]] = True
+        seen[O.dofmap[c2][mi[:, k] == 0]] = True
+    for pen in (float("inf"), 1.7e308):
+        y = _dg(p, pen)[1].apply_f64(xd).cpu().numpy()
+        assert not np.isfinite(y[seen]).any()
+        assert np.abs(y - y1)[~seen].max(initial=0.0) <= 1e-12 * np.abs(y1[~seen]).max(initial=1.0)
