@@ -300,7 +300,8 @@ __global__ void __launch_bounds__(256)
 dg_exp_kernel(const double* __restrict__ x, int32_t* __restrict__ e, int ncell) {
   constexpr int ND = N * N * N, G = ND < 32 ? 8 : 32;
   pdl_trigger();
-  const int cell = (blockIdx.x * 256 + threadIdx.x) / G, l = threadIdx.x % G;
+  const int64_t cell = fix::group_of(blockIdx.x, 256, threadIdx.x, G);
+  const int l = threadIdx.x % G;
   uint32_t m = 0u;
   if (cell < ncell)
 #pragma unroll

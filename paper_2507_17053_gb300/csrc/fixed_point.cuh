@@ -223,6 +223,11 @@ constexpr int kExpMin = 128, kExpMax = 1900, kExpBad = 0x7ff;
 
 SBM_FIX bool plain_exp(int E) { return E >= kExpMin && E <= kExpMax; }
 
+// index of a thread's group of lanes (2^27 cells of 32 lanes are 2^32 threads)
+SBM_FIX int64_t group_of(unsigned block, int threads, unsigned thread, int lanes) {
+  return ((int64_t)block * threads + thread) / lanes;
+}
+
 // a value's magnitude by its high word; the cell's largest >> 20 is E
 SBM_FIX uint32_t mag_hi(uint64_t bits) { return (uint32_t)(bits >> 32) & 0x7fffffffu; }
 

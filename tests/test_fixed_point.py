@@ -146,6 +146,10 @@ static int conversions() {
   bad |= val(fix::to_double<true>((1ll << 60), 1986)) != 0x1p+1023;
   bad |= val(fix::to_double<true>((1ll << 61) - 1, 1986)) != inf;
   bad |= val(fix::to_double<false>((1ll << 61) - 1, 963)) != 2.0;
+  // the exponents' groups of lanes up to the last of 2^31 - 1 cells
+  bad |= fix::group_of(1u << 24, 256, 0, 32) != 1ll << 27;
+  bad |= fix::group_of((1u << 28) - 1, 256, 255, 32) != (1ll << 31) - 1;
+  bad |= fix::group_of(7, 256, 9, 8) != 225;
   return bad;
 }
 
