@@ -359,23 +359,14 @@ static cudaError_t multi_dot(const T* a, int64_t lda, const T* b, int64_t n, int
 // ---- CG --------------------------------------------------------------------
 
 // Page-locked copy of the state, the iterations' outcomes and their events.
-struct CgHost {
+struct CgHost : HostRing {
   static constexpr int kRing = CG_AHEAD + 1;
-  char* mem = nullptr;
-  cudaEvent_t ev[kRing] = {};
+  using HostRing::HostRing;
   CgState* state() { return (CgState*)mem; }
-  int* done(int i) { return (int*)(mem + 256) + i; }
+  int* done(int i) { return (int*)((char*)mem + 256) + i; }
   cudaError_t init() {
     static_assert(sizeof(CgState) <= 256, "CgHost layout");
-    cudaError_t e = cudaMallocHost((void**)&mem, 256 + kRing * sizeof(int));
-    for (int i = 0; i < kRing && e == cudaSuccess; ++i)
-      e = cudaEventCreateWithFlags(&ev[i], cudaEventDisableTiming);
-    return e;
-  }
-  ~CgHost() {
-    for (cudaEvent_t v : ev)
-      if (v) cudaEventDestroy(v);
-    if (mem) cudaFreeHost(mem);
+    return HostRing::init(256 + kRing * sizeof(int), kRing);
   }
 };
 
@@ -398,7 +389,7 @@ SolveStatus solve_cg(const ApplyFn<double>& apply, int64_t n, const double* b, d
     k_reciprocal<<<vec_grid(n), 256, 0, st>>>(diag, dinv, n);
     CK(cudaGetLastError());
   }
-  CgHost ch;
+  CgHost ch(st);
   CK(ch.init());
   CgState* hs = ch.state();
 
@@ -681,19 +672,13 @@ static cudaError_t gm_step(const T* q, T* V, int64_t n, int j, const GmVecs& g, 
 
 // page-locked ring of Hessenberg columns (each: last step of the cycle or
 // not, then the column) and the events of the steps
-struct GmHost {
-  double* ring = nullptr;
-  cudaEvent_t ev[GM_RING] = {};
-  cudaError_t init(int m) {
-    cudaError_t e = cudaMallocHost((void**)&ring, (size_t)GM_RING * (m + 3) * 8);
-    for (int i = 0; i < GM_RING && e == cudaSuccess; ++i)
-      e = cudaEventCreateWithFlags(&ev[i], cudaEventDisableTiming);
-    return e;
-  }
-  ~GmHost() {
-    for (cudaEvent_t v : ev)
-      if (v) cudaEventDestroy(v);
-    if (ring) cudaFreeHost(ring);
+struct GmHost : HostRing {
+  using HostRing::HostRing;
+  int m = 0;
+  double* slot(int step) { return (double*)mem + (size_t)(step % GM_RING) * (m + 3); }
+  cudaError_t init(int restart) {
+    m = restart;
+    return HostRing::init((size_t)GM_RING * (m + 3) * 8, GM_RING);
   }
 };
 
@@ -758,7 +743,7 @@ SolveStatus solve_gmres(const ApplyFn<T>& apply, int64_t n, const TX* b, TX* x, 
   g.part = (double*)(base + bV + br + bs);
   double* part = (double*)(base + bV + br + bs + bp);
   GmCtl* ctl = (GmCtl*)(base + bV + br + bs + bp + bq);
-  GmHost gh;
+  GmHost gh(st);
   CK(gh.init(m));
   std::vector<double> y(m + 1), scale(m + 2);
   int total = 0, cycles = 0;
@@ -799,11 +784,11 @@ SolveStatus solve_gmres(const ApplyFn<T>& apply, int64_t n, const TX* b, TX* x, 
     while (k < lim) {
       for (; enq < lim && enq < k + GM_AHEAD; ++enq) {
         CK(apply(V + (size_t)enq * n, rx, st));
-        CK(gm_step<T>(rx, V, n, enq, g, ctl, gh.ring + (size_t)(enq % GM_RING) * (m + 3), st));
+        CK(gm_step<T>(rx, V, n, enq, g, ctl, gh.slot(enq), st));
         CK(cudaEventRecord(gh.ev[enq % GM_RING], st));
       }
       CK(cudaEventSynchronize(gh.ev[k % GM_RING]));
-      const double* slot = gh.ring + (size_t)(k % GM_RING) * (m + 3);
+      const double* slot = gh.slot(k);
       const bool last = slot[0] != 0.0;   // the device ended the cycle with this step
       const double* col = slot + 1;
       const double hn = col[k + 1];

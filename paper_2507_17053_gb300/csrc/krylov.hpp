@@ -35,6 +35,32 @@ struct Workspace {
   void release();
 };
 
+// Page-locked memory that kernels enqueued on st write, with the events of its
+// slots; waits for st before it is freed (an error leaves kernels in flight).
+struct HostRing {
+  void* mem = nullptr;
+  std::vector<cudaEvent_t> ev;
+  cudaStream_t st;
+  explicit HostRing(cudaStream_t st) : st(st) {}
+  HostRing(const HostRing&) = delete;
+  HostRing& operator=(const HostRing&) = delete;
+  cudaError_t init(size_t bytes, int slots) {
+    cudaError_t e = cudaMallocHost(&mem, bytes);
+    for (int i = 0; i < slots && e == cudaSuccess; ++i) {
+      cudaEvent_t v;
+      e = cudaEventCreateWithFlags(&v, cudaEventDisableTiming);
+      if (e == cudaSuccess) ev.push_back(v);
+    }
+    return e;
+  }
+  ~HostRing() {
+    if (!mem) return;
+    cudaStreamSynchronize(st);
+    for (cudaEvent_t v : ev) cudaEventDestroy(v);
+    cudaFreeHost(mem);
+  }
+};
+
 // Conjugate gradients (Jacobi-preconditioned when diag != nullptr), FP64.
 SolveStatus solve_cg(const ApplyFn<double>& apply, int64_t n, const double* b, double* x,
                      const double* diag, double rtol, int maxit, cudaStream_t st, Workspace& ws,
