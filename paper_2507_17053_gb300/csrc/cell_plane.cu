@@ -257,8 +257,10 @@ cg_plane_kernel(const PlaneArgs a, const __grid_constant__ KTab<float> t) {
 #pragma unroll
       for (int l = 0; l < L; ++l) xface[w][l] = u[l];
     }
+    __syncwarp();                 // the whole warp arrives, the plane stored
     pair_arrive<1, Sh::W>(w + 1);
   }
+  __syncwarp();
   if (w > 0) pair_wait<1, Sh::W>(w);
   const bool add = act && j0 == 0 && c > 0;
 #pragma unroll
