@@ -472,13 +472,12 @@ dg3_kernel(const DgArgs<T> a, const __grid_constant__ KTab<T> t,
 #pragma unroll
   for (int j = 0; j < N; ++j) y[j] += Z[zl + PL * j];
   if constexpr (FX) {
-    const int eo = d.x.eoff;
-    const bool bad = E == fix::kExpBad;
-    const bool plain = fix::plain_exp(E) && abs(eo) <= 64;
+    const int eb = E + d.x.eoff;
+    const bool bad = E == fix::kExpBad, plain = !bad && fix::plain_result(eb);
 #pragma unroll
     for (int j = 0; j < N; ++j) {
-      const uint64_t b = plain ? fix::to_double<false>(y[j], E + eo)
-                               : (bad ? 0x7ff8000000000000ull : fix::to_double<true>(y[j], E + eo));
+      const uint64_t b = plain ? fix::to_double<false>(y[j], eb)
+                               : (bad ? 0x7ff8000000000000ull : fix::to_double<true>(y[j], eb));
       out[j] = __longlong_as_double((long long)b);
     }
   } else {

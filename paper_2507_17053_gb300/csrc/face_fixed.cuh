@@ -67,8 +67,9 @@ __device__ __forceinline__ int64_t face_dot(const FA& A, const FQ& Q) {
   return fix::dot<K, N>([&](int j) { return e[j]; }, q);
 }
 
-__device__ __forceinline__ double face_to_double(int64_t q, int E, int eoff, bool plain) {
-  const uint64_t b = plain ? fix::to_double<false>(q, E + eoff) : fix::to_double<true>(q, E + eoff);
+__device__ __forceinline__ double face_to_double(int64_t q, int eb) {
+  const uint64_t b = fix::plain_result(eb) ? fix::to_double<false>(q, eb)
+                                           : fix::to_double<true>(q, eb);
   return __longlong_as_double((long long)b);
 }
 
@@ -207,9 +208,8 @@ __device__ __forceinline__ void face_group_fix(const FaceArgs<double>& a, const 
     if (E == fix::kExpBad || fe == fix::kFaceExpBad) {
       q = tm = __longlong_as_double(0x7ff8000000000000ll);
     } else {
-      const bool plain = fix::plain_exp(E) && abs(fe) <= 64;
-      q = face_to_double(qi, E, fe + a.fix.eq, plain);
-      tm = face_to_double(ti, E, a.fix.etm, plain);
+      q = face_to_double(qi, E + fe + a.fix.eq);
+      tm = face_to_double(ti, E + a.fix.etm);
     }
     outr[(size_t)f * 2 * L + tl] = fma(ts.sigma, q, (ts.h_inv * ts.hface) * tm);
     outr[(size_t)f * 2 * L + L + tl] = (s ? -ts.h_inv : ts.h_inv) * q;

@@ -247,6 +247,10 @@ SBM_FIX int64_t from_double(uint64_t bits, int E) {
   return (((int64_t)m ^ s) - s) >> (sh < 63 ? sh : 63);
 }
 
+// to_double<false> serves results that can be neither subnormal nor infinite:
+// biased exponents eb + 63 - lz, 2 <= lz <= 63
+SBM_FIX bool plain_result(int eb) { return eb >= 1 && eb <= 1984; }
+
 // q 2^(eb - 1023) -> double, rounded to nearest; |q| < 2^62
 template <bool Careful>
 SBM_FIX uint64_t to_double(int64_t q, int eb) {

@@ -146,6 +146,16 @@ static int conversions() {
   bad |= val(fix::to_double<true>((1ll << 60), 1986)) != 0x1p+1023;
   bad |= val(fix::to_double<true>((1ll << 61) - 1, 1986)) != inf;
   bad |= val(fix::to_double<false>((1ll << 61) - 1, 963)) != 2.0;
+  // both conversions of a result agree wherever the plain one is taken
+  for (int eb = -2; eb <= 2050; ++eb) {
+    if (fix::plain_result(eb) != (eb >= 1 && eb <= 1984)) bad = 1;
+    if (!fix::plain_result(eb)) continue;
+    for (long long q : {1ll, 3ll, (1ll << 52) - 1, (1ll << 53) + 1, 1ll << 60, (1ll << 61) + 512,
+                        (1ll << 62) - 1})
+      for (long long v : {q, -q})
+        bad |= fix::to_double<false>(v, eb) != fix::to_double<true>(v, eb) ||
+               !std::isnormal(val(fix::to_double<false>(v, eb)));
+  }
   // the exponents' groups of lanes up to the last of 2^31 - 1 cells
   bad |= fix::group_of(1u << 24, 256, 0, 32) != 1ll << 27;
   bad |= fix::group_of((1u << 28) - 1, 256, 255, 32) != (1ll << 31) - 1;
