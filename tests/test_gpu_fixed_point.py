@@ -69,6 +69,63 @@ def test_non_finite_input_stays_in_its_cells(w, value):
         assert int((~fin).sum()) <= 8 * (w.degree + 1) ** 3
 
 
+# ---- discontinuous Galerkin: exponents of a cell and its neighbours ----------------
+
+DG_CASES = [dataclasses.replace(w, dg=True) for w in CASES]
+
+
+@pytest.mark.parametrize("w", DG_CASES, ids=lambda w: f"q{w.degree}")
+def test_dg_power_of_two_scaling_is_exact(w):
+    test_power_of_two_scaling_is_exact(w, 0)
+
+
+@pytest.mark.parametrize("w", DG_CASES, ids=lambda w: f"q{w.degree}")
+def test_dg_subnormal_input(w):
+    test_subnormal_input(w)
+
+
+@pytest.mark.parametrize("value", [float("nan"), float("inf"), -float("inf")])
+@pytest.mark.parametrize("w", DG_CASES, ids=lambda w: f"q{w.degree}")
+def test_dg_non_finite_input_stays_near(w, value):
+    """One non-finite entry: its cell and that cell's neighbours are not finite,
+    every other one is bitwise unchanged."""
+    P = G.Problem.from_workload(w)
+    nd = (w.degree + 1) ** 3
+    O = OracleProblem.from_workload(w)
+    x = torch.from_numpy(S.random_vector(w.seed, P.n_dofs, w.dist)).cuda()
+    y = P.apply_f64(x).view(-1, nd)
+    c = len(O.mesh.cells) // 2
+    xb = x.clone()
+    xb[c * nd + nd // 3] = value
+    yb = P.apply_f64(xb).view(-1, nd)
+    near = {c} | {int(b) for a, _, b in O.mesh.ifaces if a == c} \
+        | {int(a) for a, _, b in O.mesh.ifaces if b == c}
+    far = torch.ones(len(O.mesh.cells), dtype=torch.bool)
+    far[sorted(near)] = False
+    assert not torch.isfinite(yb[~far]).any()
+    assert torch.equal(yb[far], y[far])
+
+
+@pytest.mark.parametrize("w", DG_CASES, ids=lambda w: f"q{w.degree}")
+def test_dg_neighbours_of_other_magnitudes(w):
+    """Cells scaled by 2^-60 .. 2^60, neighbours at random: every cell against
+    the oracle, relative to the largest values the double form sums for it --
+    test_gpu_apply's bound times |A| |x| over the cell and its neighbours."""
+    O = OracleProblem.from_workload(w)
+    P = G.Problem.from_workload(w)
+    nd, nc = (w.degree + 1) ** 3, len(O.mesh.cells)
+    k = np.random.default_rng(5).integers(-60, 61, nc)
+    x = (S.random_vector(w.seed, O.n_dofs, w.dist).reshape(nc, nd) * 2.0 ** k[:, None])
+    y = P.apply_f64(torch.from_numpy(x.ravel()).cuda()).cpu().numpy().reshape(nc, nd)
+    ref = O.apply(x.ravel()).reshape(nc, nd)
+    big = np.abs(x).max(axis=1)
+    for a, _, b in O.mesh.ifaces:
+        m = max(np.abs(x[a]).max(), np.abs(x[b]).max())
+        big[a], big[b] = max(big[a], m), max(big[b], m)
+    one = np.abs(O.apply(np.ones(O.n_dofs) * S.random_vector(9, O.n_dofs, "uniform"))).max()
+    assert (np.abs(y - ref).max(axis=1) <= 1e-12 * one * big).all()
+
+
 # ---- discontinuous Galerkin: interior-face penalties of every size -----------------
 
 DG_BOX = S._wl("box", 3, 2, 5, S.box((0.0,) * 3, (1.5,) * 3), dg=True, seed=5)
