@@ -881,8 +881,8 @@ int sbm_device_status(sbm_problem* prob) {
   return SBM_OK;
 }
 
-// time every tile shape of the single apply (2 where available), in FP64
-// and FP32, on the problem itself, and keep the faster of each
+// time every tile shape of the single apply (but 2: the kernel of shape 0), in
+// FP64 and FP32, on the problem itself, and keep the faster of each
 int sbm_autotune(sbm_problem* prob, int* shape64, int* shape32) {
   if (!prob) return fail(SBM_ERR_ARG, "prob is NULL");
   if (!prob->on_device) return fail(SBM_ERR_STATE, "sbm_setup_face_data not called");
@@ -908,8 +908,8 @@ int sbm_autotune(sbm_problem* prob, int* shape64, int* shape32) {
     for (int vo = 0; vo < 8 && e == cudaSuccess; ++vo) {
       const int v = vo / 2;
       const bool o = vo % 2;
-      if ((v == 2 && (prec == 0 || !cell_reg_available(prob->hp, true))) || (v == 3 && prob->hp.d != 3) ||
-          (o && (v == 1 || v == 2 || !prob->dd.chunks[0].ordered)))
+      if (v == 2 || (v == 3 && prob->hp.d != 3) ||
+          (o && (v == 1 || !prob->dd.chunks[0].ordered)))
         continue;
       prob->dd.variant[prec] = v;
       prob->dd.ordered[prec] = o;

@@ -241,8 +241,6 @@ static cudaError_t apply_r(const HostProblem& hp, const DeviceData& dd, const Ch
     pdl_cell = allow_pdl && !pr;
   }
   if (pr && (err = prof->mark(st)) != cudaSuccess) return err;
-  int cap = 0;
-  if ((err = chunk_prepare<T, D, N, R>(&cap)) != cudaSuccess) return err;
   ChunkArgs<T> a;
   a.x = x;
   a.y = y;
@@ -310,11 +308,18 @@ static cudaError_t apply_r(const HostProblem& hp, const DeviceData& dd, const Ch
       nlaunch++;
     }
   } else if (part.q1 > part.q0) {
-    const int grid = std::min(part.q1 - part.q0, cap);
-    if ((err = launch_maybe_pdl(cg_chunk_kernel<T, D, N, R>, dim3(grid, nrhs), dim3(NT), smem,
-                                st, pdl_cell, a, t)) != cudaSuccess)
-      return err;
-    nlaunch++;
+    // (FP32 in 3D: whole applies on chunks of R cells are the register kernels')
+    if constexpr (std::is_same<T, float>::value && D == 3 && R == ChunkShape<D, N>::R) {
+      return cudaErrorInvalidValue;
+    } else {
+      int cap = 0;
+      if ((err = chunk_prepare<T, D, N, R>(&cap)) != cudaSuccess) return err;
+      const int grid = std::min(part.q1 - part.q0, cap);
+      if ((err = launch_maybe_pdl(cg_chunk_kernel<T, D, N, R>, dim3(grid, nrhs), dim3(NT), smem,
+                                  st, pdl_cell, a, t)) != cudaSuccess)
+        return err;
+      nlaunch++;
+    }
   }
   const bool pdl_asm = allow_pdl && !pr && nlaunch > nl0;
   if (pr && (err = prof->mark(st)) != cudaSuccess) return err;

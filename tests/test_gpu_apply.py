@@ -187,8 +187,9 @@ def test_autotuned_tile_shapes_keep_parity(w):
         G.sbm_set_tile_shape(P.handle, 4, 0)
 
 
-# tile shape 2: one thread per cell, the tile in registers (3D, FP32 p <= 4,
-# FP64 p <= 3); the same chunks and summation order as shape 0
+# tile shape 2 (3D, FP32 p <= 4, FP64 p <= 3): the kernels of shape 0, on FP32
+# those that keep the cell in registers; compared with shape 3, another kernel on
+# the same chunks with the same summation order
 REG_CASES = [S.SPHERE_3D_Q4.resized(n, degree=p) for p, n in ((1, 9), (2, 8), (3, 7), (4, 12))] \
     + [S.ELLIPSOID_3D_Q6.resized(10, degree=4), S.SPHERE_3D_Q4.resized(17, degree=2)] \
     + S.batched_ellipsoids(nprob=3, n_range=(7, 11), p_range=(2, 4))
@@ -207,6 +208,10 @@ def test_register_tile_shape_equals_shape0_and_oracle(w):
     G.sbm_set_tile_shape(P.handle, 2 if fp64 else 0, 2)
     y64, y32 = P.apply_f64(xd), P.apply_f32(xd.float())
     assert torch.equal(y32, y32_0), "shape 2 differs from shape 0 in FP32"
+    G.sbm_set_tile_shape(P.handle, 3, 3)
+    assert torch.equal(P.apply_f32(xd.float()), y32), "shape 3 differs from shape 2 in FP32"
+    assert torch.equal(P.apply_f64(xd), y64), "shape 3 differs from shape 2 in FP64"
+    G.sbm_set_tile_shape(P.handle, 2 if fp64 else 0, 2)
     assert torch.equal(y32, P.apply_f32(xd.float())), "repeated apply differs"
     assert _rel(y32.double().cpu().numpy(), ref32) <= F32_TOL
     if fp64:
