@@ -39,7 +39,7 @@ namespace {
 constexpr int reg_threads(int n) { return n == 2 ? 64 : 32; }
 
 // resident blocks asked of the compiler: 16 warps per SM (128 registers)
-template <typename T, int N>
+template <int N>
 constexpr int reg_min_blocks() {
   return 16 * 32 / reg_threads(N);
 }
@@ -52,19 +52,19 @@ constexpr int reg_words() {
 // h K + mu_ab M of every x-line of modes (a, b), index a + n b, in the
 // even/odd layout of XLineOp::store, computed on the host with the same
 // arithmetic as XLineOp (fused multiply-add, correctly rounded on both).
-template <typename T, int N>
+template <int N>
 struct XOps {
-  T m[N * N][XLineOp<T, N>::kSize];
+  float m[N * N][XLineOp<float, N>::kSize];
 };
 
-template <typename T, int N>
-XOps<T, N> make_xops(const KTab<T>& t) {
+template <int N>
+XOps<N> make_xops(const KTab<float>& t) {
   constexpr int H = N / 2, HE = (N + 1) / 2;
-  XOps<T, N> o;
+  XOps<N> o;
   for (int b = 0; b < N; ++b)
     for (int a = 0; a < N; ++a) {
-      T* m = o.m[a + N * b];
-      const T mu = t.hlam[a] + t.hlam[b];
+      float* m = o.m[a + N * b];
+      const float mu = t.hlam[a] + t.hlam[b];
       for (int i = 0; i < HE; ++i)
         for (int j = i; j < HE; ++j)
           m[i * HE + j] = m[j * HE + i] = std::fma(mu, t.fM.E[i][j], t.fKh.E[i][j]);
@@ -76,15 +76,14 @@ XOps<T, N> make_xops(const KTab<T>& t) {
   return o;
 }
 
-template <typename T>
 struct RegArgs {
-  const T* __restrict__ x;
-  T* __restrict__ y;
-  T* __restrict__ ycol;                     // [ncolours][n_dofs]
+  const float* __restrict__ x;
+  float* __restrict__ y;
+  float* __restrict__ ycol;                 // [ncolours][n_dofs]
   const int32_t* __restrict__ lines;        // ordered cells x L
   const int32_t* __restrict__ face_start;
   const int32_t* __restrict__ face_kind;
-  const T* __restrict__ face_out;           // [F][2L]
+  const float* __restrict__ face_out;       // [F][2L]
   const int32_t* __restrict__ chunk_first;  // tile shape 0
   const uint8_t* __restrict__ chunk_col;
   const int32_t* __restrict__ cell_chunk;   // ordered cell -> its chunk
@@ -94,11 +93,11 @@ struct RegArgs {
 };
 
 // the x-line operator h K + mu_ab M (even/odd layout) on one register line
-template <typename T, int N>
-__device__ __forceinline__ void xline_apply(const T* m, const T (&v)[N], T (&y)[N]) {
+template <int N>
+__device__ __forceinline__ void xline_apply(const float* m, const float (&v)[N], float (&y)[N]) {
   constexpr int H = N / 2, HE = (N + 1) / 2;
-  const LineFold<T, N> f(v);
-  LineAcc<T, N> acc;
+  const LineFold<float, N> f(v);
+  LineAcc<float, N> acc;
 #pragma unroll
   for (int i = 0; i < HE; ++i)
 #pragma unroll
@@ -111,16 +110,16 @@ __device__ __forceinline__ void xline_apply(const T* m, const T (&v)[N], T (&y)[
 }
 
 // the five line phases on the tile (node j0 + n j1 + n^2 j2)
-template <typename T, int N>
-__device__ __forceinline__ void cell_phases(const KTab<T>& t, const XOps<T, N>& xo,
-                                            T (&u)[N * N * N]) {
+template <int N>
+__device__ __forceinline__ void cell_phases(const KTab<float>& t, const XOps<N>& xo,
+                                            float (&u)[N * N * N]) {
   constexpr int L = N * N;
-  T v[N], w[N];
+  float v[N], w[N];
 #pragma unroll
   for (int l = 0; l < L; ++l) {          // z-lines (j0, j1) = (l % n, l / n) -> z-modes
 #pragma unroll
     for (int j = 0; j < N; ++j) v[j] = u[l + L * j];
-    line_to_modes<T, N>(t.fVt, v, w);
+    line_to_modes<float, N>(t.fVt, v, w);
 #pragma unroll
     for (int j = 0; j < N; ++j) u[l + L * j] = w[j];
   }
@@ -130,7 +129,7 @@ __device__ __forceinline__ void cell_phases(const KTab<T>& t, const XOps<T, N>& 
     for (int a = 0; a < N; ++a) {
 #pragma unroll
       for (int j = 0; j < N; ++j) v[j] = u[a + N * j + L * b];
-      line_to_modes<T, N>(t.fVt, v, w);
+      line_to_modes<float, N>(t.fVt, v, w);
 #pragma unroll
       for (int j = 0; j < N; ++j) u[a + N * j + L * b] = w[j];
     }
@@ -138,7 +137,7 @@ __device__ __forceinline__ void cell_phases(const KTab<T>& t, const XOps<T, N>& 
   for (int l = 0; l < L; ++l) {          // x-lines (y-mode, z-mode) = (l % n, l / n)
 #pragma unroll
     for (int j = 0; j < N; ++j) v[j] = u[N * l + j];
-    xline_apply<T, N>(xo.m[l], v, w);
+    xline_apply<N>(xo.m[l], v, w);
 #pragma unroll
     for (int j = 0; j < N; ++j) u[N * l + j] = w[j];
   }
@@ -148,7 +147,7 @@ __device__ __forceinline__ void cell_phases(const KTab<T>& t, const XOps<T, N>& 
     for (int a = 0; a < N; ++a) {
 #pragma unroll
       for (int j = 0; j < N; ++j) w[j] = u[a + N * j + L * b];
-      modes_to_line<T, N>(t.fV, w, v);
+      modes_to_line<float, N>(t.fV, w, v);
 #pragma unroll
       for (int j = 0; j < N; ++j) u[a + N * j + L * b] = v[j];
     }
@@ -156,7 +155,7 @@ __device__ __forceinline__ void cell_phases(const KTab<T>& t, const XOps<T, N>& 
   for (int l = 0; l < L; ++l) {          // z-modes back
 #pragma unroll
     for (int j = 0; j < N; ++j) w[j] = u[l + L * j];
-    modes_to_line<T, N>(t.fV, w, v);
+    modes_to_line<float, N>(t.fV, w, v);
 #pragma unroll
     for (int j = 0; j < N; ++j) u[l + L * j] = v[j];
   }
@@ -164,30 +163,30 @@ __device__ __forceinline__ void cell_phases(const KTab<T>& t, const XOps<T, N>& 
 
 // surrogate face (k, s): the chunk kernel's fold_face_z on every z-line
 // (j0, j1) of the tile, in the same operation order
-template <typename T, int N, int K, int SD, bool COH>
-__device__ __forceinline__ void fold_reg(const KTab<T>& t, const T* __restrict__ fo,
-                                         T (&u)[N * N * N]) {
+template <int N, int K, int SD, bool COH>
+__device__ __forceinline__ void fold_reg(const KTab<float>& t, const float* __restrict__ fo,
+                                         float (&u)[N * N * N]) {
   constexpr int L = N * N, KEND = SD ? N - 1 : 0;
-  const T* rv = fo;
-  const T* rg = fo + L;
+  const float* rv = fo;
+  const float* rg = fo + L;
 #pragma unroll
   for (int b = 0; b < N; ++b)
 #pragma unroll
     for (int a = 0; a < N; ++a) {
       if (K == 2) {
-        const T vv = ld_face<COH>(rv + a + N * b), g = ld_face<COH>(rg + a + N * b);
+        const float vv = ld_face<COH>(rv + a + N * b), g = ld_face<COH>(rg + a + N * b);
 #pragma unroll
         for (int m = 0; m < N; ++m) {
-          T& o = u[a + N * b + L * m];
+          float& o = u[a + N * b + L * m];
           o = fma(SD ? t.D1[m] : t.D0[m], g, o);
           if (m == KEND) o = add_rn(o, vv);
         }
       } else {
         const int jk = (K == 0) ? a : b, jo = (K == 0) ? b : a;
-        const T dk = SD ? t.D1[jk] : t.D0[jk];
+        const float dk = SD ? t.D1[jk] : t.D0[jk];
 #pragma unroll
         for (int m = 0; m < N; ++m) {
-          T add = mul_rn(dk, ld_face<COH>(rg + jo + N * m));
+          float add = mul_rn(dk, ld_face<COH>(rg + jo + N * m));
           if (jk == KEND) add = add_rn(add, ld_face<COH>(rv + jo + N * m));
           u[a + N * b + L * m] = add_rn(u[a + N * b + L * m], add);
         }
@@ -195,18 +194,18 @@ __device__ __forceinline__ void fold_reg(const KTab<T>& t, const T* __restrict__
     }
 }
 
-template <typename T, int N, bool PDL>
-__global__ void __launch_bounds__(reg_threads(N), (reg_min_blocks<T, N>()))
-cg_cell_reg_kernel(const RegArgs<T> a, const __grid_constant__ KTab<T> t,
-                   const __grid_constant__ XOps<T, N> xo) {
+template <int N, bool PDL>
+__global__ void __launch_bounds__(reg_threads(N), (reg_min_blocks<N>()))
+cg_cell_reg_kernel(const RegArgs a, const __grid_constant__ KTab<float> t,
+                   const __grid_constant__ XOps<N> xo) {
   constexpr int L = N * N, ND = L * N, P = N - 1, W = reg_words<N>();
-  __shared__ T xface[reg_threads(N)][L + 1];    // j0 = P face of each cell (odd row stride)
+  __shared__ float xface[reg_threads(N)][L + 1];    // j0 = P face of each cell (odd row stride)
   const int tid = threadIdx.x;
   const int b0 = a.block_first[blockIdx.x], b1 = a.block_first[blockIdx.x + 1];
   const int c0 = __ldg(a.chunk_first + b0), c1 = __ldg(a.chunk_first + b1);
   const int pos = c0 + tid;
   const bool act = pos < c1;
-  T u[ND];
+  float u[ND];
   int c = 0, nc = 0, ch = 0;
   const int32_t* ln = a.lines + (size_t)(act ? pos : 0) * L;
   if (act) {
@@ -216,25 +215,25 @@ cg_cell_reg_kernel(const RegArgs<T> a, const __grid_constant__ KTab<T> t,
     nc = __ldg(a.chunk_first + ch + 1) - f;
 #pragma unroll
     for (int l = 0; l < L; ++l) {
-      const T* xl = a.x + __ldg(ln + l);
+      const float* xl = a.x + __ldg(ln + l);
 #pragma unroll
       for (int j0 = 0; j0 < N; ++j0) u[j0 + N * l] = __ldg(xl + j0);
     }
-    cell_phases<T, N>(t, xo, u);
+    cell_phases<N>(t, xo, u);
     const int fs = __ldg(a.face_start + pos), fe = __ldg(a.face_start + pos + 1);
     if constexpr (PDL) {
       if (fs < fe) pdl_wait();
     }
     for (int f2 = fs; f2 < fe; ++f2) {
       const int kind = __ldg(a.face_kind + f2);
-      const T* fo = a.face_out + (size_t)f2 * 2 * L;
+      const float* fo = a.face_out + (size_t)f2 * 2 * L;
       switch (kind) {
-        case 0: fold_reg<T, N, 0, 0, PDL>(t, fo, u); break;
-        case 1: fold_reg<T, N, 1, 0, PDL>(t, fo, u); break;
-        case 2: fold_reg<T, N, 2, 0, PDL>(t, fo, u); break;
-        case 4: fold_reg<T, N, 0, 1, PDL>(t, fo, u); break;
-        case 5: fold_reg<T, N, 1, 1, PDL>(t, fo, u); break;
-        case 6: fold_reg<T, N, 2, 1, PDL>(t, fo, u); break;
+        case 0: fold_reg<N, 0, 0, PDL>(t, fo, u); break;
+        case 1: fold_reg<N, 1, 0, PDL>(t, fo, u); break;
+        case 2: fold_reg<N, 2, 0, PDL>(t, fo, u); break;
+        case 4: fold_reg<N, 0, 1, PDL>(t, fo, u); break;
+        case 5: fold_reg<N, 1, 1, PDL>(t, fo, u); break;
+        case 6: fold_reg<N, 2, 1, PDL>(t, fo, u); break;
         default: break;
       }
     }
@@ -251,7 +250,7 @@ cg_cell_reg_kernel(const RegArgs<T> a, const __grid_constant__ KTab<T> t,
   uint32_t mk[W];
 #pragma unroll
   for (int i = 0; i < W; ++i) mk[i] = __ldg(a.mask + (size_t)pos * W + i);
-  T* yc = a.ycol + (size_t)__ldg(a.chunk_col + ch) * a.n_dofs;
+  float* yc = a.ycol + (size_t)__ldg(a.chunk_col + ch) * a.n_dofs;
   const bool last = c == nc - 1;     // only the chunk's last cell stores its j0 = P nodes
 #pragma unroll
   for (int l = 0; l < L; ++l) {
@@ -260,7 +259,7 @@ cg_cell_reg_kernel(const RegArgs<T> a, const __grid_constant__ KTab<T> t,
     for (int j0 = 0; j0 < N; ++j0) {
       const int node = j0 + N * l;
       if (j0 == P && !last) continue;
-      T* dst = ((mk[node >> 5] >> (node & 31)) & 1u) ? yc : a.y;
+      float* dst = ((mk[node >> 5] >> (node & 31)) & 1u) ? yc : a.y;
       dst[base + j0] = u[node];
     }
   }
@@ -293,10 +292,10 @@ __global__ void k_reg_mask(const int32_t* __restrict__ cell_chunk,
   }
 }
 
-template <typename T, int N>
-cudaError_t launch_reg(const HostProblem& hp, const DeviceData& dd, const T* x, T* y,
-                       const T* fo, T* ycol, cudaStream_t st, bool pdl) {
-  RegArgs<T> a;
+template <int N>
+cudaError_t launch_reg(const HostProblem& hp, const DeviceData& dd, const float* x, float* y,
+                       const float* fo, float* ycol, cudaStream_t st, bool pdl) {
+  RegArgs a;
   a.x = x;
   a.y = y;
   a.ycol = ycol;
@@ -310,8 +309,8 @@ cudaError_t launch_reg(const HostProblem& hp, const DeviceData& dd, const T* x, 
   a.mask = dd.reg_mask;
   a.block_first = dd.reg_block_first;
   a.n_dofs = hp.n_dofs;
-  const KTab<T> t = make_ktab<T>(hp);
-  const XOps<T, N> xo = make_xops<T, N>(t);
+  const KTab<float> t = make_ktab<float>(hp);
+  const XOps<N> xo = make_xops<N>(t);
   // pdl (FP32 applies after the CUDA-core face kernel): a programmatic
   // dependent launch; a thread waits for the face kernel only when its cell
   // has surrogate faces (the other cells need nothing from it) and then reads
@@ -319,9 +318,9 @@ cudaError_t launch_reg(const HostProblem& hp, const DeviceData& dd, const T* x, 
   // own dependents early (the assembly starts as its blocks finish): an early
   // trigger cost 0.5-1 %.  Measured, unprofiled FP32 apply on GB300, p = 2
   // sphere of 128^3 cells: 0.0520 -> 0.0480 ms; results bitwise unchanged.
-  cudaError_t e = pdl ? launch_maybe_pdl(cg_cell_reg_kernel<T, N, true>, dim3(dd.reg_nblocks),
+  cudaError_t e = pdl ? launch_maybe_pdl(cg_cell_reg_kernel<N, true>, dim3(dd.reg_nblocks),
                                          dim3(reg_threads(N)), 0, st, true, a, t, xo)
-                      : launch_maybe_pdl(cg_cell_reg_kernel<T, N, false>, dim3(dd.reg_nblocks),
+                      : launch_maybe_pdl(cg_cell_reg_kernel<N, false>, dim3(dd.reg_nblocks),
                                          dim3(reg_threads(N)), 0, st, false, a, t, xo);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -385,8 +384,8 @@ cudaError_t launch_cell_reg(const HostProblem& hp, const DeviceData& dd, const f
                             const float* fo, float* ycol, cudaStream_t st, bool pdl) {
   if (!dd.reg_mask) return cudaErrorInvalidValue;
   switch (hp.n) {
-    case 2: return launch_reg<float, 2>(hp, dd, x, y, fo, ycol, st, pdl);
-    case 3: return launch_reg<float, 3>(hp, dd, x, y, fo, ycol, st, pdl);
+    case 2: return launch_reg<2>(hp, dd, x, y, fo, ycol, st, pdl);
+    case 3: return launch_reg<3>(hp, dd, x, y, fo, ycol, st, pdl);
     default: return cudaErrorInvalidValue;
   }
 }

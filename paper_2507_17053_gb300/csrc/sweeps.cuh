@@ -465,12 +465,10 @@ __device__ __forceinline__ void cell_fix_3d_l(const KTab<double>& t, const Load&
 
 // The thread's z-line of x comes from load(j), j = 0..n-1 (staged runs in
 // shared memory, or global memory directly).
-// PAD = false: the unpadded layout (PX = n), for callers that address the
-// tile themselves (the DG kernel).
-template <typename T, int N, bool PAD = true, typename XOp, typename Load>
+template <typename T, int N, typename XOp, typename Load>
 __device__ __forceinline__ void cell_fd_3d_l(const KTab<T>& t, const Load& load, T* tile, int c,
                                              int tl, bool act, const XOp& xop, T (&out)[N]) {
-  constexpr int PX = PAD ? TilePad<T, N>::PX : N, NDP = PX * N * N, PL = PX * N;
+  constexpr int PX = TilePad<T, N>::PX, NDP = PX * N * N, PL = PX * N;
   const int a = tl % N, b = tl / N;
   const int zl = (PX == N) ? tl : a + PX * b;     // the z-line's first node
   T* cell = tile + c * NDP;
@@ -518,11 +516,11 @@ __device__ __forceinline__ void cell_fd_3d_l(const KTab<T>& t, const Load& load,
   }
 }
 
-template <typename T, int N, bool PAD = true, typename XOp>
+template <typename T, int N, typename XOp>
 __device__ __forceinline__ void cell_fd_3d(const KTab<T>& t, const T* X, int xb, int xs, T* tile,
                                            int c, int tl, bool act, const XOp& xop,
                                            T (&out)[N]) {
-  cell_fd_3d_l<T, N, PAD>(t, [&](int j) { return X[xb + xs * j]; }, tile, c, tl, act, xop, out);
+  cell_fd_3d_l<T, N>(t, [&](int j) { return X[xb + xs * j]; }, tile, c, tl, act, xop, out);
 }
 
 // ---- cell term -------------------------------------------------------------
