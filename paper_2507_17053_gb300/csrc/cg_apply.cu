@@ -290,8 +290,13 @@ static cudaError_t apply_r(const HostProblem& hp, const DeviceData& dd, const Ch
         if ((err = resident_grid(cg_chunk_ord_kernel<T, D, N, R>, NT, smem, &cache0, &grid)) !=
             cudaSuccess)
           return err;
+        // 2D FP64 p = 6 starts after the faces: its blocks, spread over the SMs that
+        // the face kernel leaves, took 40.4 / 146 / 214 / 276 us as a dependent
+        // against 37.5 / 126 / 188 / 266 (disks of 100^2 / 300^2 / 400^2 / 500^2
+        // cells); p <= 5 gains 0 .. 25 %
+        const bool pdl = pdl_cell && !(D == 2 && N == 7 && std::is_same<T, double>::value);
         if ((err = launch_maybe_pdl(cg_chunk_ord_kernel<T, D, N, R>, dim3(std::min(grid, ct.n)),
-                                    dim3(NT), smem, st, pdl_cell, a, t, oa)) != cudaSuccess)
+                                    dim3(NT), smem, st, pdl, a, t, oa)) != cudaSuccess)
           return err;
       }
       nlaunch++;

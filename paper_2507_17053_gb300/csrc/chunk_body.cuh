@@ -506,6 +506,7 @@ __device__ __forceinline__ void chunk_loop_ord(const ChunkArgs<T>& a, const KTab
   T* XLs = Xbuf + 2 * CS::XS;
   int* Lbuf = reinterpret_cast<int*>(XLs + CS::XL);
   uint32_t* Bs = reinterpret_cast<uint32_t*>(Lbuf + 2 * L);
+  constexpr int NT = block_threads<T, D, N>(R);
   const int tid = threadIdx.x;
   int c, tl;
   cell_of_thread<T, D, N>(tid, c, tl);
@@ -530,7 +531,7 @@ __device__ __forceinline__ void chunk_loop_ord(const ChunkArgs<T>& a, const KTab
     for (int i = tid; i < L; i += blockDim.x) Lbuf[i] = __ldg(a.lines + (size_t)first * L + i);
     __syncthreads();
     if (tid == 0) s_ord_next = (int)atomicAdd(o.tickets, 1u);
-    gather_runs_async<T, L, SM>(xr, Lbuf, Xbuf, S, tid, blockDim.x);
+    gather_runs_async<T, L, SM>(xr, Lbuf, Xbuf, S, tid, NT);
   }
   cp_async_commit();
   __syncthreads();                            // s_ord_next written
@@ -555,7 +556,7 @@ __device__ __forceinline__ void chunk_loop_ord(const ChunkArgs<T>& a, const KTab
       for (int i = tid; i < L; i += blockDim.x) Ln[i] = __ldg(a.lines + (size_t)f2 * L + i);
       if (tid == 0) tk2 = atomicAdd(o.tickets, 1u);
       __syncthreads();
-      gather_runs_async<T, L, SM>(xr, Ln, Xbuf + (buf ^ 1) * CS::XS, S2, tid, blockDim.x);
+      gather_runs_async<T, L, SM>(xr, Ln, Xbuf + (buf ^ 1) * CS::XS, S2, tid, NT);
     }
     cp_async_commit();
     {
@@ -616,7 +617,7 @@ __device__ __forceinline__ void chunk_loop_ord(const ChunkArgs<T>& a, const KTab
     T old[N];
 #pragma unroll
     for (int k = 0; k < N; ++k) {
-      const int idx = tid + k * (int)blockDim.x;
+      const int idx = tid + k * NT;
       old[k] = T(0);
       if (idx < L * S && ((Bs[idx >> 5] >> (idx & 31)) & 1u)) {
         const int l = __float2int_rz(((float)idx + 0.5f) * invS);
@@ -625,7 +626,7 @@ __device__ __forceinline__ void chunk_loop_ord(const ChunkArgs<T>& a, const KTab
     }
 #pragma unroll
     for (int k = 0; k < N; ++k) {
-      const int idx = tid + k * (int)blockDim.x;
+      const int idx = tid + k * NT;
       if (idx < L * S) {
         const int l = __float2int_rz(((float)idx + 0.5f) * invS), kk = idx - l * S;
         const int cc = kk / P, m = kk - cc * P;
