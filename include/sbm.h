@@ -562,10 +562,11 @@ int sbm_device_status(sbm_problem* prob);
  * shapes and keeps the faster per precision:
  *   0  chunks of R consecutive cells of a mesh row (R (p+1)^(d-1) threads),
  *      x-line runs staged in shared memory; FP32 in 3D: the cells of these
- *      chunks in registers, one thread per cell (p <= 2) or p + 1 (p >= 3);
+ *      chunks in registers, one thread per cell (p <= 2) or p + 1 (p >= 3),
+ *      or shape 3 (p = 4, 5 and few cells);
  *   1  chunks of R/2 cells;
- *   2  (3D; FP32 p <= 4, FP64 p <= 3) the kernels of shape 0 (accepted, not
- *      timed);
+ *   2  (3D; FP32 p <= 4, FP64 p <= 3) FP32: the cells in registers as in
+ *      shape 0; FP64: shape 0 (accepted, not timed);
  *   3  (3D) shape 0's chunks without staged runs: each thread loads and
  *      stores its own lines.
  * and for shapes 0 and 3 each way of completing the DoFs several chunk

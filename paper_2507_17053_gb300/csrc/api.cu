@@ -881,8 +881,9 @@ int sbm_device_status(sbm_problem* prob) {
   return SBM_OK;
 }
 
-// time every tile shape of the single apply (but 2: the kernel of shape 0), in
-// FP64 and FP32, on the problem itself, and keep the faster of each
+// time every tile shape of the single apply that is a kernel of its own (2 is
+// the kernel of shape 0), in FP64 and FP32, on the problem itself, and keep the
+// faster of each
 int sbm_autotune(sbm_problem* prob, int* shape64, int* shape32) {
   if (!prob) return fail(SBM_ERR_ARG, "prob is NULL");
   if (!prob->on_device) return fail(SBM_ERR_STATE, "sbm_setup_face_data not called");
@@ -909,6 +910,7 @@ int sbm_autotune(sbm_problem* prob, int* shape64, int* shape32) {
       const int v = vo / 2;
       const bool o = vo % 2;
       if (v == 2 || (v == 3 && prob->hp.d != 3) ||
+          (v == 3 && !o && prec == 1 && f32_few_cells(prob->hp, prob->dd)) ||
           (o && (v == 1 || !prob->dd.chunks[0].ordered)))
         continue;
       prob->dd.variant[prec] = v;

@@ -351,6 +351,18 @@ static cudaError_t apply_r(const HostProblem& hp, const DeviceData& dd, const Ch
   return cudaSuccess;
 }
 
+// FP32 applies of shape 0 too small for the plane kernel, whose threads each run
+// n^2 lines: the time of one thread is a floor that more cells have to fill.
+// Measured on balls (us, chunk kernel / plane kernel / shape 3): p = 4 1 502
+// cells 15.5 / 15.8 / 14.3, 6 151 20.3 / 17.8 / 16.0, 11 956 27.2 / 20.4 / 23.0;
+// p = 5 519 21.0 / 23.6 / 14.3, 6 151 27.2 / 29.1 / 21.9, 11 956 37.9 / 31.9 /
+// 29.7, 20 719 52.8 / 39.3 / 41.8.  At p = 3 and 6 the plane kernel was never
+// behind the chunk kernel.
+bool f32_few_cells(const HostProblem& hp, const DeviceData& dd) {
+  const int cells = dd.col_start[dd.ncolours];
+  return hp.n == 5 ? cells < 9000 : hp.n == 6 && cells < 16000;
+}
+
 // variant 0: R cells per chunk; variant 1: R/2 (a second tile shape for the
 // autotuner); variant 2: the cells of variant 0's chunks one thread or n
 // threads each (FP32, whole applies; FP64 runs variant 0, which gives the same
@@ -365,14 +377,15 @@ static cudaError_t apply_t(const HostProblem& hp, const DeviceData& dd, const T*
   constexpr int RH = (R / 2) > 0 ? R / 2 : 1;
   const int v = (variant == 1 && RH < R) ? 1 : 0;
   // FP32 whole applies of shapes 0 and 2 run the register kernels, which give
-  // the same bits and were faster than the chunk kernel at every degree and size
-  // measured (us, chunk kernel / shape 3 / register kernels: p = 1 128^3 47.5 /
-  // 35.1 / 24.8, p = 2 96^3 55.6 / 42.3 / 24.4, p = 3 105 / 78.9 / 55.4, p = 4
-  // 195 / 153 / 114, p = 5 64^3 109 / 88.6 / 77, p = 6 48^3 60 / 48.9 / 46.1,
-  // p = 4 32^3 20.6 / 15.8 / 16.7: the autotuner still has shape 3)
-  const bool reg = std::is_same<T, float>::value && D == 3 && slab < 0 && nrhs == 1 &&
-                   (variant == 2 || (variant == 0 && !ordered));
-  const bool direct = variant == 3 && D == 3;
+  // the same bits and were faster than the chunk kernel (us, chunk kernel / shape
+  // 3 / register kernels: p = 1 128^3 47.5 / 35.1 / 24.8, p = 2 96^3 55.6 / 42.3 /
+  // 24.4, p = 3 105 / 78.9 / 55.4, p = 4 195 / 153 / 114, p = 5 64^3 109 / 88.6 /
+  // 77, p = 6 48^3 60 / 48.9 / 46.1), but for few cells at p = 4, 5: there shape 0
+  // is shape 3 (f32_few_cells)
+  const bool single32 = std::is_same<T, float>::value && D == 3 && slab < 0 && nrhs == 1;
+  const bool few = single32 && variant == 0 && f32_few_cells(hp, dd);
+  const bool reg = single32 && (variant == 2 || (variant == 0 && !ordered && !few));
+  const bool direct = D == 3 && (variant == 3 || (few && !ordered));
   const ChunkTable& ct = dd.chunks[v];
   // colour-ordered stores: whole single applies of chunking 0 by the chunk
   // kernels (shapes 0 and 3; shape 2 keeps the colour buffers)

@@ -268,9 +268,11 @@ cudaError_t launch_maybe_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size
 
 // FP32 whole applies of 3D CG problems on the chunks of shape 0, bitwise equal
 // to the chunk kernel: one thread per cell (n <= 3), n threads per cell (n >= 4).
-// cell_reg_available: what tile shape 2 is accepted for.
+// cell_reg_available: what tile shape 2 is accepted for; f32_few_cells: FP32
+// shape 0 runs the kernel of shape 3 (cg_apply.cu).
 bool cell_reg_available(const HostProblem& hp, bool fp32);
 bool cell_reg_used(const HostProblem& hp);
+bool f32_few_cells(const HostProblem& hp, const DeviceData& dd);
 cudaError_t build_cell_reg_tables(const HostProblem& hp, const std::vector<int32_t>& ch_first,
                                   DeviceData* dd);
 cudaError_t launch_cell_reg(const HostProblem& hp, const DeviceData& dd, const float* x, float* y,
