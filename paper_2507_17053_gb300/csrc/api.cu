@@ -119,9 +119,44 @@ static cudaError_t upload(T** dst, const T* src, size_t count) {
   return cudaMemcpy(*dst, src, count * sizeof(T), cudaMemcpyHostToDevice);
 }
 
+// In one allocation, owned by fix_buf: the 1D tables of the 3D applies (the
+// x-line operators; D0, M and S of the FP64 faces; M, S and W of the FP32 ones),
+// the DG neighbours and exponents.
+static cudaError_t upload_fixed(const HostProblem& hp, const std::vector<int32_t>& nbr,
+                                DeviceData* dd) {
+  std::vector<float> tab;
+  if (hp.d == 3 && hp.desc.extension == SBM_EXT_EXACT) {
+    const KTab<float> t = make_ktab<float>(hp);
+    for (int i = 0; i < hp.n; ++i) tab.insert(tab.end(), t.M[i], t.M[i] + hp.n);
+    for (int i = 0; i < hp.n; ++i) tab.insert(tab.end(), t.S[i], t.S[i] + hp.n);
+    tab.insert(tab.end(), t.W, t.W + hp.L);
+  }
+  const struct { const void* src; size_t bytes; } part[] = {
+      {hp.fx.xline.data(), hp.fx.xline.size() * sizeof(fix::Entry)},
+      {hp.fx.face.data(), hp.fx.face.size() * sizeof(fix::Entry)},
+      {nbr.data(), nbr.size() * sizeof(int32_t)},        // (rows of 2 d words, read in pairs)
+      {tab.data(), tab.size() * sizeof(float)}};
+  size_t off[5] = {0};
+  for (int i = 0; i < 4; ++i) off[i + 1] = off[i] + part[i].bytes;
+  const size_t be = hp.desc.dg && hp.d == 3 ? nbr.size() / 6 * sizeof(int32_t) : 0;
+  if (off[4] + be == 0) return cudaSuccess;
+  std::vector<unsigned char> h(off[4]);
+  for (int i = 0; i < 4; ++i)
+    if (part[i].bytes) std::memcpy(h.data() + off[i], part[i].src, part[i].bytes);
+  unsigned char* p = nullptr;
+  cudaError_t e = cudaMalloc((void**)&p, off[4] + be);
+  if (e != cudaSuccess) return e;
+  dd->fix_buf = p;
+  if (part[0].bytes) dd->xfix = (fix::Entry*)p;
+  if (part[1].bytes) dd->fix_tab = (fix::Entry*)(p + off[1]);
+  if (part[2].bytes) dd->nbr = (int32_t*)(p + off[2]);
+  if (part[3].bytes) dd->face_tab32 = (float*)(p + off[3]);
+  if (be) dd->dg_exp = (int32_t*)(p + off[4]);
+  return cudaMemcpy(p, h.data(), h.size(), cudaMemcpyHostToDevice);
+}
+
 static void free_device(DeviceData* dd) {
   cudaFree(dd->lines);
-  cudaFree(dd->xfix);
   cudaFree(dd->reg_cell_chunk);
   cudaFree(dd->reg_block_first);
   cudaFree(dd->reg_mask);
@@ -155,12 +190,7 @@ static void free_device(DeviceData* dd) {
   cudaFree(dd->face_phi);
   cudaFree(dd->face_phi32);
   cudaFree(dd->fix_pp);
-  cudaFree(dd->fix_p0);
-  cudaFree(dd->fix_exp);
-  cudaFree(dd->fix_tab);
-  cudaFree(dd->face_tab32);
-  cudaFree(dd->nbr);
-  cudaFree(dd->dg_exp);
+  cudaFree(dd->fix_buf);
   cudaFree(dd->stage_x);
   cudaFree(dd->stage_y);
   for (cudaEvent_t ev : dd->ev_in)
@@ -330,13 +360,7 @@ static int build_device(const HostProblem& hp, DeviceData* dd) {
         }
   }
   cudaError_t e;
-  if ((e = upload(&dd->nbr, nbr.data(), nbr.size())) != cudaSuccess) goto err;
-  if (hp.desc.dg && d == 3 &&
-      (e = cudaMalloc((void**)&dd->dg_exp, (size_t)Nc * sizeof(int32_t))) != cudaSuccess)
-    goto err;
-  if (d == 3 &&
-      (e = upload(&dd->xfix, hp.fx.xline.data(), hp.fx.xline.size())) != cudaSuccess)
-    goto err;
+  if ((e = upload_fixed(hp, nbr, dd)) != cudaSuccess) goto err;
   if ((e = upload(&dd->lines, lines_o.data(), lines_o.size())) != cudaSuccess) goto err;
   if ((e = upload(&dd->cell_rank, dd->order.data(), dd->order.size())) != cudaSuccess) goto err;
   if ((e = upload(&dd->face_start, fstart.data(), fstart.size())) != cudaSuccess) goto err;
@@ -394,18 +418,9 @@ static int build_device(const HostProblem& hp, DeviceData* dd) {
       goto err;
   }
   if ((e = device_face_phi(hp, fsrc, &dd->face_phi, &dd->face_phi32)) != cudaSuccess) goto err;
-  if (d == 3 && hp.desc.extension == SBM_EXT_EXACT) {
-    const KTab<float> t = make_ktab<float>(hp);
-    std::vector<float> tab;
-    for (int i = 0; i < n; ++i) tab.insert(tab.end(), t.M[i], t.M[i] + n);
-    for (int i = 0; i < n; ++i) tab.insert(tab.end(), t.S[i], t.S[i] + n);
-    tab.insert(tab.end(), t.W, t.W + L);
-    if ((e = upload(&dd->face_tab32, tab.data(), tab.size())) != cudaSuccess) goto err;
-  }
   if (d == 3 && hp.desc.extension == SBM_EXT_EXACT &&
-      ((e = device_face_fix((int64_t)fsrc.size(), L, n, dd->face_phi, make_ktab<double>(hp).W,
-                            &dd->fix_pp, &dd->fix_p0, &dd->fix_exp)) != cudaSuccess ||
-       (e = upload(&dd->fix_tab, hp.fx.face.data(), hp.fx.face.size())) != cudaSuccess))
+      (e = device_face_fix((int64_t)fsrc.size(), L, n, dd->face_phi, make_ktab<double>(hp).W,
+                           &dd->fix_pp, &dd->fix_p0, &dd->fix_exp)) != cudaSuccess)
     goto err;
   if (dd->nslab > 1) {
     // copy streams and events of the pipelined host-buffer apply

@@ -573,10 +573,22 @@ int setup_tables(sbm_batch* B) {
   const int nprob = (int)B->probs.size();
   std::vector<KTab<T>> kt(nprob);
   std::map<int, KTab<T>> unit;
+  std::map<int, FixedTables> fixed;
   for (int k = 0; k < nprob; ++k) {
     const HostProblem& hp = B->probs[k]->hp;
     kt[k] = make_ktab<T>(hp);
-    const KTab<T> u = unit_table<T>(hp);
+    KTab<T> u = unit_table<T>(hp);
+    if constexpr (std::is_same<T, double>::value) {
+      // a 2D problem's table too holds the 3D cell term's: the constant bank is
+      // shared with batches of 3D problems of the degree
+      if (hp.d == 2) {
+        auto [f, made] = fixed.try_emplace(hp.n);
+        if (made && !build_fixed_tables(hp.tab, 1.0, &f->second, 0.0, kFixCell))
+          return sbm_fail_detail(SBM_ERR_UNSUPPORTED, "fixed-point tables");
+        u.xVt = f->second.Vt;
+        u.xV = f->second.V;
+      }
+    }
     auto it = unit.find(hp.n);
     if (it == unit.end()) {
       unit[hp.n] = u;

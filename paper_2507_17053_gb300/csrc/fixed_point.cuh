@@ -52,6 +52,33 @@ struct alignas(8) Entry {
   int32_t h, l;                      // A 2^t = h 2^30 + l / 2
 };
 
+SBM_FIX Entry to_entry(int64_t I) {
+  const int64_t h = (I + ((int64_t)1 << 29)) >> 30;
+  return Entry{(int32_t)h, (int32_t)(2 * (I - h * ((int64_t)1 << 30)))};
+}
+
+// a b 2^t as an entry, rounded to nearest, of two finite doubles' bits;
+// |a b 2^t| < 2^61.  (In integers: in double precision the product, its error and
+// their conversions took nine operations of the slow pipe.)
+SBM_FIX Entry product(uint64_t a, uint64_t b, int t) {
+  const uint64_t frac = ((uint64_t)1 << 52) - 1;
+  const int ea = (int)(a >> 52) & 0x7ff, eb = (int)(b >> 52) & 0x7ff;
+  const uint64_t ma = (a & frac) | (ea ? frac + 1 : 0), mb = (b & frac) | (eb ? frac + 1 : 0);
+  const int sh = 2150 - (ea ? ea : 1) - (eb ? eb : 1) - t;
+  const uint64_t lo = ma * mb;
+#ifdef __CUDA_ARCH__
+  const uint64_t hi = __umul64hi(ma, mb);
+#else
+  const uint64_t hi = (uint64_t)(((unsigned __int128)ma * mb) >> 64);
+#endif
+  uint64_t r = 0;                              // the product is below 2^106
+  if (sh <= 0) r = sh > -64 ? lo << -sh : 0;
+  else if (sh < 64) r = ((hi << (64 - sh)) | (lo >> sh)) + ((lo >> (sh - 1)) & 1u);
+  else if (sh == 64) r = hi + (lo >> 63);
+  else if (sh < 107) r = (hi >> (sh - 64)) + ((hi >> (sh - 65)) & 1u);
+  return to_entry((int64_t)((a ^ b) >> 63 ? 0 - r : r));
+}
+
 // even and odd block of a centrosymmetric or (anti)symmetric-column matrix
 struct Block {
   Entry E[kMaxHalf][kMaxHalf];

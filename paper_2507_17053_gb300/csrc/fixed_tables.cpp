@@ -4,6 +4,8 @@
 
 #include <algorithm>
 #include <cmath>
+#include <mutex>
+#include <vector>
 
 #include "setup.hpp"
 
@@ -94,12 +96,18 @@ void mass_stiffness(const Tables1D& t, Pencil* P) {
   }
   for (int i = 0; i < n; ++i)
     for (int j = 0; j < n; ++j) P->M[i][j] = P->K[i][j] = DD();
+  DD inv[kMaxN][kMaxN];
+  for (int j = 0; j < n; ++j)
+    for (int m = 0; m < j; ++m) {
+      inv[j][m] = DD(1.0) / (x[j] - x[m]);
+      inv[m][j] = -inv[j][m];
+    }
   auto lagrange = [&](const DD& s, DD* v, DD* dv) {
     for (int j = 0; j < n; ++j) {
       DD a = 1.0, b;
       for (int m = 0; m < n; ++m) {
         if (m == j) continue;
-        const DD f = DD(1.0) / (x[j] - x[m]);
+        const DD f = inv[j][m];
         b = (b * (s - x[m]) + a) * f;
         a = a * (s - x[m]) * f;
       }
@@ -113,11 +121,13 @@ void mass_stiffness(const Tables1D& t, Pencil* P) {
     DD v[kMaxN], dv[kMaxN];
     lagrange(g[q], v, dv);
     for (int j = 0; j < n; ++j) P->S[q][j] = v[j];
-    for (int i = 0; i < n; ++i)
+    for (int i = 0; i < n; ++i) {
+      const DD wv = w[q] * v[i], wd = w[q] * dv[i];
       for (int j = 0; j < n; ++j) {
-        P->M[i][j] = P->M[i][j] + w[q] * v[i] * v[j];
-        P->K[i][j] = P->K[i][j] + w[q] * dv[i] * dv[j];
+        P->M[i][j] = P->M[i][j] + wv * v[j];
+        P->K[i][j] = P->K[i][j] + wd * dv[j];
       }
+    }
   }
 }
 
@@ -131,7 +141,7 @@ void refine(const Tables1D& t, Pencil* P) {
     P->lam[i] = t.lam[i];
     for (int j = 0; j < n; ++j) P->V[i][j] = t.V[i][j];
   }
-  for (int it = 0; it < 3; ++it) {
+  for (int it = 0; it < 2; ++it) {
     DD A[kMaxN][2 * kMaxN];                       // Gauss-Jordan: W = V^-1
     for (int i = 0; i < n; ++i)
       for (int j = 0; j < n; ++j) {
@@ -163,18 +173,19 @@ void refine(const Tables1D& t, Pencil* P) {
         R1[i][j] = a;
         R2[i][j] = b;
       }
+    DD T1[kMaxN][kMaxN], T2[kMaxN][kMaxN];
     for (int i = 0; i < n; ++i)
-      for (int j = 0; j < n; ++j) {
-        DD a, b;
-        for (int k = 0; k < n; ++k)
-          for (int l = 0; l < n; ++l) {
-            const DD ww = A[i][n + k] * A[j][n + l];
-            a = a + ww * R1[k][l];
-            b = b + ww * R2[k][l];
-          }
-        E1[i][j] = a;
-        E2[i][j] = b;
-      }
+      for (int j = 0; j < n; ++j)
+        for (int k = 0; k < n; ++k) {
+          T1[i][j] = T1[i][j] + A[i][n + k] * R1[k][j];
+          T2[i][j] = T2[i][j] + A[i][n + k] * R2[k][j];
+        }
+    for (int i = 0; i < n; ++i)
+      for (int j = 0; j < n; ++j)
+        for (int l = 0; l < n; ++l) {
+          E1[i][j] = E1[i][j] + T1[i][l] * A[j][n + l];
+          E2[i][j] = E2[i][j] + T2[i][l] * A[j][n + l];
+        }
     DD nv[kMaxN][kMaxN];
     for (int i = 0; i < n; ++i)
       for (int j = 0; j < n; ++j) {
@@ -199,134 +210,25 @@ void refine(const Tables1D& t, Pencil* P) {
 fix::Entry entry(const DD& A, int t) {
   const double s = std::ldexp(A.h, t);
   const int64_t i1 = std::llrint(s);
-  const int64_t I = i1 + std::llrint((s - (double)i1) + std::ldexp(A.l, t));
-  const int64_t h = (I + ((int64_t)1 << 29)) >> 30;
-  return fix::Entry{(int32_t)h, (int32_t)(2 * (I - h * ((int64_t)1 << 30)))};
+  return fix::to_entry(i1 + std::llrint((s - (double)i1) + std::ldexp(A.l, t)));
 }
 
-}  // namespace
+// t = 61 - ceil(log2) of the largest absolute sum
+int fit(double c) { return 61 - (int)std::ceil(std::log2(c * (1.0 + 1e-6))); }
 
-bool build_fixed_tables(const Tables1D& tb, double scale, FixedTables* out, double pen) {
-  const int n = tb.n, H = n / 2, HE = (n + 1) / 2;
+// What depends on the degree alone, made once per degree and process: the pencil
+// and the face tables ...
+struct Faces {
   Pencil P;
+  std::vector<fix::Entry> face;
+  int tM, eq, etm;
+};
+void make_faces(const Tables1D& tb, Faces* o) {
+  const int n = tb.n;
+  Pencil& P = o->P;
   P.n = n;
   mass_stiffness(tb, &P);
-  refine(tb, &P);
-  // scale = hm 2^eh, hm in (1/2, 1]
-  int eh;
-  double hm = std::frexp(scale, &eh);
-  if (hm == 0.5) {
-    hm = 1.0;
-    --eh;
-  }
-  auto X = [&](int a, int b, int i, int j) { return P.K[i][j] + (P.lam[a] + P.lam[b]) * P.M[i][j]; };
-  // modes scaled by 2^sm: rows of V^T of absolute sum in (1/2, 1]
-  double r[kMaxN];
-  int sm[kMaxN];
-  for (int k = 0; k < n; ++k) {
-    r[k] = 0.0;
-    for (int j = 0; j < n; ++j) r[k] += mag(P.V[j][k]);
-    sm[k] = (int)std::floor(-std::log2(r[k]) + 1e-7);
-    if (!(r[k] <= 1.0 + 1e-7)) return false;      // S_1 = S_2 = 0 below
-  }
-  // largest absolute row sums from the input to the phases' results
-  double B3 = 0.0, B4 = 0.0, B5 = 0.0;
-  for (int a = 0; a < n; ++a)
-    for (int b = 0; b < n; ++b)
-      for (int i = 0; i < n; ++i) {
-        double s = 0.0;
-        for (int j = 0; j < n; ++j) s += mag(X(a, b, i, j));
-        B3 = std::max(B3, s * r[a] * r[b]);
-      }
-  // (mirrored rows have equal sums)
-  for (int b = 0; b < n; ++b)
-    for (int i = 0; i < HE; ++i)
-      for (int y = 0; y < HE; ++y) {
-        double s = 0.0;
-        for (int j = 0; j < n; ++j)
-          for (int yy = 0; yy < n; ++yy) {
-            double u = 0.0;
-            for (int a = 0; a < n; ++a) u += P.V[y][a].h * P.V[yy][a].h * X(a, b, i, j).h;
-            s += std::fabs(u);
-          }
-        B4 = std::max(B4, s * r[b]);
-      }
-  for (int i = 0; i < HE; ++i)
-    for (int y = i; y < HE; ++y)
-      for (int z = y; z < HE; ++z) {   // and the axes can be exchanged
-        double s = 0.0;
-        for (int j = 0; j < n; ++j)
-          for (int yy = 0; yy < n; ++yy)
-            for (int zz = 0; zz < n; ++zz)
-              s += std::fabs(P.K[i][j].h * P.M[y][yy].h * P.M[z][zz].h +
-                             P.M[i][j].h * P.K[y][yy].h * P.M[z][zz].h +
-                             P.M[i][j].h * P.M[y][yy].h * P.K[z][zz].h);
-        B5 = std::max(B5, s);
-      }
-  auto scale_of = [](double B) { return -(int)std::ceil(std::log2(B) - 1e-7); };
-  const int S3 = scale_of(B3), S4 = scale_of(B4), S5 = scale_of(B5);
-  // t = 61 + S_i - S_{i-1} - K per phase, and what a result then sums
-  const int t1 = 61, t3 = 61 + S3 - fix::shift_x(n), t4 = 61 + S4 - S3 - fix::shift_y(n),
-            t5 = 61 + S5 - S4 - fix::shift_z(n);
-  if (t4 != t5) return false;                     // one table serves both
-  const double lim = std::ldexp(1.0, 61) * (1.0 - 1e-7);
-  out->Vt = out->V = fix::Block{};
-  for (int k = 0; k < n; ++k) {
-    double s = 0.0;
-    const bool odd = k >= HE;
-    for (int j = 0; j < (odd ? H : HE); ++j) {
-      s += std::ldexp(mag(P.V[j][k]), t1 + sm[k]);
-      const fix::Entry e = entry(P.V[j][k], t1 + sm[k]);
-      if (odd) out->Vt.O[k - HE][j] = e;
-      else out->Vt.E[k][j] = e;
-    }
-    if (!(s <= lim)) return false;
-  }
-  for (int j = 0; j < HE; ++j) {
-    double se = 0.0, so = 0.0;
-    for (int k = 0; k < n; ++k) {
-      const bool odd = k >= HE;
-      if (odd && j >= H) continue;
-      (odd ? so : se) += std::ldexp(mag(P.V[j][k]), t4);
-      const fix::Entry e = entry(P.V[j][k], t4);
-      if (odd) out->V.O[j][k - HE] = e;
-      else out->V.E[j][k] = e;
-    }
-    if (!(se <= lim && so <= lim)) return false;
-  }
-  // hm (K + (lam_a + lam_b) M) 2^(-sm_a - sm_b): the upper triangles of the
-  // even and the odd block, one slot per unordered pair of modes a <= b
-  const int packed = (HE * (HE + 1) / 2 + H * (H + 1) / 2) | 1;
-  out->xline.assign((size_t)(n * (n + 1) / 2) * packed, fix::Entry{0, 0});
-  size_t slot = 0;
-  for (int a = 0; a < n; ++a)
-    for (int b = a; b < n; ++b, slot += packed) {
-      const int t = t3 - sm[a] - sm[b];
-      auto E = [&](int i, int j) {
-        const DD v = (n & 1) && j == H ? X(a, b, i, j)
-                                       : (X(a, b, i, j) + X(a, b, i, n - 1 - j)) * DD(0.5);
-        return v * DD(hm);
-      };
-      auto O = [&](int i, int j) {
-        return (X(a, b, i, j) - X(a, b, i, n - 1 - j)) * DD(0.5) * DD(hm);
-      };
-      size_t w = slot;
-      for (int i = 0; i < HE; ++i) {
-        double s = 0.0;
-        for (int j = 0; j < HE; ++j) s += std::ldexp(mag(E(i, j)), t);
-        if (!(s <= lim)) return false;
-        for (int j = i; j < HE; ++j) out->xline[w++] = entry(E(i, j), t);
-      }
-      for (int i = 0; i < H; ++i) {
-        double s = 0.0;
-        for (int j = 0; j < H; ++j) s += std::ldexp(mag(O(i, j)), t);
-        if (!(s <= lim)) return false;
-        for (int j = i; j < H; ++j) out->xline[w++] = entry(O(i, j), t);
-      }
-    }
-  out->eoff = -59 - S5 + eh;
-  // faces: t = 61 - ceil(log2) of the largest absolute sum; the trace of D0
-  // is taken of 57-bit values and leaves at 60 bits (K = 3)
+  // the trace of D0 is taken of 57-bit values and leaves at 60 bits (K = 3)
   double cD = 0.0, cM = 0.0, cS = 0.0;
   for (int j = 0; j < n; ++j) {
     double m = 0.0, s = 0.0;
@@ -338,16 +240,182 @@ bool build_fixed_tables(const Tables1D& tb, double scale, FixedTables* out, doub
     cM = std::max(cM, m);
     cS = std::max(cS, s);
   }
-  auto fit = [](double c) { return 61 - (int)std::ceil(std::log2(c * (1.0 + 1e-6))); };
-  const int tD = fit(cD), tM = fit(cM), tS = fit(cS);
-  out->face.clear();
-  for (int j = 0; j < n; ++j) out->face.push_back(entry(P.D0[j], tD));
+  const int tD = fit(cD), tS = fit(cS);
+  o->tM = fit(cM);
+  for (int j = 0; j < n; ++j) o->face.push_back(entry(P.D0[j], tD));
   for (int i = 0; i < n; ++i)
-    for (int j = 0; j < n; ++j) out->face.push_back(entry(P.M[i][j], tM));
+    for (int j = 0; j < n; ++j) o->face.push_back(entry(P.M[i][j], o->tM));
   for (int q = 0; q < n; ++q)
-    for (int j = 0; j < n; ++j) out->face.push_back(entry(P.S[q][j], tS));
-  out->face_eq = 2 + 2 * (61 - tS);
-  out->face_etm = 2 - tD + 2 * (61 - tM);
+    for (int j = 0; j < n; ++j) o->face.push_back(entry(P.S[q][j], tS));
+  o->eq = 2 + 2 * (61 - tS);
+  o->etm = 2 - tD + 2 * (61 - o->tM);
+}
+
+// ... and the eigenbasis and scales of the cell term
+struct Cell {
+  Pencil P;
+  fix::Block Vt = {}, V = {};
+  int sm[kMaxN], t3, S5;
+  bool ok;
+};
+bool make_cell(const Tables1D& tb, Cell* o) {
+  const int n = tb.n, H = n / 2, HE = (n + 1) / 2;
+  Pencil& P = o->P;
+  refine(tb, &P);
+  // modes scaled by 2^sm: rows of V^T of absolute sum in (1/2, 1]
+  double r[kMaxN], lam[kMaxN], M[kMaxN][kMaxN], K[kMaxN][kMaxN];
+  int* sm = o->sm;
+  for (int k = 0; k < n; ++k) {
+    r[k] = 0.0;
+    for (int j = 0; j < n; ++j) r[k] += mag(P.V[j][k]);
+    sm[k] = (int)std::floor(-std::log2(r[k]) + 1e-7);
+    if (!(r[k] <= 1.0 + 1e-7)) return false;      // S_1 = S_2 = 0 below
+    lam[k] = P.lam[k].h;
+    for (int j = 0; j < n; ++j) {
+      M[k][j] = P.M[k][j].h;
+      K[k][j] = P.K[k][j].h;
+    }
+  }
+  // largest absolute row sums from the input to the phases' results
+  double B3 = 0.0, B4 = 0.0, B5 = 0.0;
+  for (int a = 0; a < n; ++a)
+    for (int b = a; b < n; ++b)
+      for (int i = 0; i < HE; ++i) {               // (mirrored rows have equal sums)
+        double s = 0.0;
+        for (int j = 0; j < n; ++j) s += std::fabs(K[i][j] + (lam[a] + lam[b]) * M[i][j]);
+        B3 = std::max(B3, s * r[a] * r[b]);
+      }
+  // (summed over the y-modes: V V^T = M, V lam V^T = K)
+  for (int b = 0; b < n; ++b)
+    for (int i = 0; i < HE; ++i)
+      for (int y = 0; y < HE; ++y) {
+        double s = 0.0;
+        for (int j = 0; j < n; ++j)
+          for (int yy = 0; yy < n; ++yy)
+            s += std::fabs((K[i][j] + lam[b] * M[i][j]) * M[y][yy] + M[i][j] * K[y][yy]);
+        B4 = std::max(B4, s * r[b]);
+      }
+  for (int i = 0; i < HE; ++i)
+    for (int y = i; y < HE; ++y)
+      for (int z = y; z < HE; ++z) {   // and the axes can be exchanged
+        double s = 0.0;
+        for (int j = 0; j < n; ++j)
+          for (int yy = 0; yy < n; ++yy) {
+            const double km = K[i][j] * M[y][yy] + M[i][j] * K[y][yy], mm = M[i][j] * M[y][yy];
+            for (int zz = 0; zz < n; ++zz) s += std::fabs(km * M[z][zz] + mm * K[z][zz]);
+          }
+        B5 = std::max(B5, s);
+      }
+  auto scale_of = [](double B) { return -(int)std::ceil(std::log2(B) - 1e-7); };
+  const int S3 = scale_of(B3), S4 = scale_of(B4), S5 = scale_of(B5);
+  // t = 61 + S_i - S_{i-1} - K per phase, and what a result then sums
+  const int t1 = 61, t4 = 61 + S4 - S3 - fix::shift_y(n),
+            t5 = 61 + S5 - S4 - fix::shift_z(n);
+  if (t4 != t5) return false;                     // one table serves both
+  o->t3 = 61 + S3 - fix::shift_x(n);
+  o->S5 = S5;
+  const double lim = std::ldexp(1.0, 61) * (1.0 - 1e-7);
+  for (int k = 0; k < n; ++k) {
+    double s = 0.0;
+    const bool odd = k >= HE;
+    for (int j = 0; j < (odd ? H : HE); ++j) {
+      s += std::ldexp(mag(P.V[j][k]), t1 + sm[k]);
+      const fix::Entry e = entry(P.V[j][k], t1 + sm[k]);
+      if (odd) o->Vt.O[k - HE][j] = e;
+      else o->Vt.E[k][j] = e;
+    }
+    if (!(s <= lim)) return false;
+  }
+  for (int j = 0; j < HE; ++j) {
+    double se = 0.0, so = 0.0;
+    for (int k = 0; k < n; ++k) {
+      const bool odd = k >= HE;
+      if (odd && j >= H) continue;
+      (odd ? so : se) += std::ldexp(mag(P.V[j][k]), t4);
+      const fix::Entry e = entry(P.V[j][k], t4);
+      if (odd) o->V.O[j][k - HE] = e;
+      else o->V.E[j][k] = e;
+    }
+    if (!(se <= lim && so <= lim)) return false;
+  }
+  return true;
+}
+
+const Faces& faces_of(const Tables1D& tb) {
+  static std::once_flag once[kMaxN + 1];
+  static Faces made[kMaxN + 1];
+  std::call_once(once[tb.n], [&] { make_faces(tb, &made[tb.n]); });
+  return made[tb.n];
+}
+const Cell& cell_of(const Tables1D& tb) {
+  static std::once_flag once[kMaxN + 1];
+  static Cell made[kMaxN + 1];
+  std::call_once(once[tb.n], [&] {
+    made[tb.n].P = faces_of(tb).P;
+    made[tb.n].ok = make_cell(tb, &made[tb.n]);
+  });
+  return made[tb.n];
+}
+
+// the cell term's part: Vt, V, xline, eoff
+bool cell_tables(const Tables1D& tb, double hm, int eh, FixedTables* out) {
+  const int n = tb.n, H = n / 2, HE = (n + 1) / 2;
+  const Cell& c = cell_of(tb);
+  if (!c.ok) return false;
+  const Pencil& P = c.P;
+  const double lim = std::ldexp(1.0, 61) * (1.0 - 1e-7);
+  out->Vt = c.Vt;
+  out->V = c.V;
+  // hm (K + (lam_a + lam_b) M) 2^(-sm_a - sm_b): the upper triangles of the
+  // even and the odd block, one slot per unordered pair of modes a <= b
+  const int packed = (HE * (HE + 1) / 2 + H * (H + 1) / 2) | 1;
+  out->xline.assign((size_t)(n * (n + 1) / 2) * packed, fix::Entry{0, 0});
+  size_t slot = 0;
+  for (int a = 0; a < n; ++a)
+    for (int b = a; b < n; ++b, slot += packed) {
+      const int t = c.t3 - c.sm[a] - c.sm[b];
+      const DD mu = P.lam[a] + P.lam[b];
+      DD X[fix::kMaxHalf][kMaxN];                 // the upper half of h K + mu M
+      for (int i = 0; i < HE; ++i)
+        for (int j = 0; j < n; ++j) X[i][j] = P.K[i][j] + mu * P.M[i][j];
+      size_t w = slot;
+      for (int o = 0; o < 2; ++o)
+        for (int i = 0; i < (o ? H : HE); ++i) {
+          double s = 0.0;
+          for (int j = 0; j < (o ? H : HE); ++j) {
+            const DD u = o ? X[i][j] - X[i][n - 1 - j] : X[i][j] + X[i][n - 1 - j];
+            const DD v = ((n & 1) && j == H ? X[i][j] : u * DD(0.5)) * DD(hm);
+            s += std::ldexp(mag(v), t);
+            if (j >= i) out->xline[w++] = entry(v, t);
+          }
+          if (!(s <= lim)) return false;
+        }
+    }
+  out->eoff = -59 - c.S5 + eh;
+  return true;
+}
+
+}  // namespace
+
+bool build_fixed_tables(const Tables1D& tb, double scale, FixedTables* out, double pen, int parts) {
+  const int n = tb.n, H = n / 2, HE = (n + 1) / 2;
+  *out = FixedTables{};
+  if (!parts) return true;
+  // scale = hm 2^eh, hm in (1/2, 1]
+  int eh;
+  double hm = std::frexp(scale, &eh);
+  if (hm == 0.5) {
+    hm = 1.0;
+    --eh;
+  }
+  if ((parts & kFixCell) && !cell_tables(tb, hm, eh, out)) return false;
+  const Faces& fa = faces_of(tb);
+  const Pencil& P = fa.P;
+  const int tM = fa.tM;
+  if (parts & kFixFaces) out->face = fa.face;
+  out->face_eq = fa.eq;
+  out->face_etm = fa.etm;
+  if (!(parts & kFixDg)) return true;
   // DG line operators: row i of K u + sum_s Own_s g_s, |g| <= 2 |u|, scaled to
   // leave 57-bit values at 59 bits (K = 3); hm goes into the entries.  The
   // penalty is part of them while it no more than doubles the largest row sum
@@ -373,7 +441,6 @@ bool build_fixed_tables(const Tables1D& tb, double scale, FixedTables* out, doub
     w[0] = DD(pen) + w[0];
     B1 = B1p;
   }
-  out->dg = fix::DgTab{};
   const int tR = fit(B1) - 1;
   auto folded = [&](const DD (&A)[kMaxN][kMaxN], int t, double f, fix::Block* o) {
     for (int i = 0; i < HE; ++i)

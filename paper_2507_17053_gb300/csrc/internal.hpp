@@ -128,7 +128,8 @@ cudaError_t device_chunk_tables(const int32_t* lines, int64_t nc, int L, int n, 
 cudaError_t device_face_phi(const HostProblem& hp, const std::vector<int64_t>& fsrc,
                             double** phi, float** phi32);
 // 3D exact extension: the fixed-point tables of the FP64 faces from the FP64
-// table phi ([F][Q][3][n]) and the face weights W ([Q]), allocated here.
+// table phi ([F][Q][3][n]) and the face weights W ([Q]), allocated here (freed
+// with pp).
 cudaError_t device_face_fix(int64_t F, int L, int n, const double* phi, const double* W,
                             fix::Entry** pp, fix::Entry** p0, int32_t** exp);
 
@@ -145,8 +146,9 @@ struct DeviceData {
   int32_t* face_start = nullptr; // [Nc + 1] per ordered cell, range into the ordered face list
   int32_t* face_kind = nullptr;  // [F] k | (s << 2)
   int32_t* face_cell = nullptr;  // [F] ordered cell position of the face's cell
-  // 3D: the x-line operators of the fixed-point FP64 cell term, slot by slot
+  // 3D CG: the x-line operators of the fixed-point FP64 cell term, slot by slot
   fix::Entry* xfix = nullptr;
+  void* fix_buf = nullptr;       // owns xfix, fix_tab, nbr, face_tab32 and dg_exp
   int nface = 0;
   double* face_out = nullptr;    // [F * 2L] per-face results of the face kernel (scratch)
   float* face_out32 = nullptr;
@@ -178,7 +180,7 @@ struct DeviceData {
   // 3D exact extension, FP64 faces (face_fixed.cuh), point index fastest:
   // [F][n^2][Q] the products phi_j1(xi_{q,1}) phi_j2(xi_{q,2}) of the two
   // non-first axes, index j1 + n j2; [F][n][Q] W_q phi_j0(xi_{q,0}); [F] the
-  // exponents; the 1D tables
+  // exponents (fix_pp owns the three); the 1D tables
   fix::Entry* fix_pp = nullptr;
   fix::Entry* fix_p0 = nullptr;
   int32_t* fix_exp = nullptr;

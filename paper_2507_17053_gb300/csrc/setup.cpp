@@ -485,8 +485,11 @@ int setup_prepare(const sbm_desc& desc, HostProblem* hp, std::string* err) {
     *err = "1D eigenbasis of the cell operator is inaccurate";
     return SBM_ERR_UNSUPPORTED;
   }
-  // (2D too: problems of one degree share one unit table in a batch)
-  if (!build_fixed_tables(P.tab, P.h, &P.fx, P.sigma_f * P.h)) {
+  // the parts that 3D FP64 applies read
+  const int fix_parts = d == 2 ? 0
+                               : (desc.dg ? kFixDg : kFixCell) |
+                                     (desc.extension == SBM_EXT_EXACT ? kFixFaces : 0);
+  if (!build_fixed_tables(P.tab, P.h, &P.fx, P.sigma_f * P.h, fix_parts)) {
     *err = "fixed-point tables of the cell operator are out of bounds";
     return SBM_ERR_UNSUPPORTED;
   }

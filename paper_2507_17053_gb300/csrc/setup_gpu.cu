@@ -665,14 +665,8 @@ cudaError_t device_chunk_tables(const int32_t* lines, int64_t nc, int L, int n, 
   return cudaDeviceSynchronize();
 }
 
-// a b 2^t as an entry (the product's rounding error included)
 __device__ __forceinline__ fix::Entry fix_product(double a, double b, int t) {
-  const double p = a * b, err = fma(a, b, -p);
-  const double s = ldexp(p, t);
-  const long long i1 = __double2ll_rn(s);
-  const long long I = i1 + __double2ll_rn((s - (double)i1) + ldexp(err, t));
-  const long long h = (I + (1ll << 29)) >> 30;
-  return fix::Entry{(int32_t)h, (int32_t)(2 * (I - h * (1ll << 30)))};
+  return fix::product((uint64_t)__double_as_longlong(a), (uint64_t)__double_as_longlong(b), t);
 }
 
 struct FaceWeights {
@@ -719,13 +713,14 @@ k_face_fix(int64_t F, int L, int n, const double* __restrict__ phi,
     const bool bad = s_bad != 0;
     if (q == 0) exp[f] = bad ? fix::kFaceExpBad : ef;
     if (q < L) {
+      const int t0 = bad ? 0 : 61 - t - ef;
       for (int j2 = 0; j2 < n; ++j2)
         for (int j1 = 0; j1 < n; ++j1)
           pp[((size_t)f * n * n + j1 + n * j2) * L + q] =
               bad ? fix::Entry{0, 0} : fix_product(ph[n + j1], ph[2 * n + j2], t);
       for (int j = 0; j < n; ++j)
         p0[((size_t)f * n + j) * L + q] =
-            bad ? fix::Entry{0, 0} : fix_product(W, ph[j], 61 - t - ef);
+            bad ? fix::Entry{0, 0} : fix_product(W, ph[j], t0);
     }
     __syncthreads();               // s_exp, s_bad are reused
   }
@@ -738,11 +733,11 @@ cudaError_t device_face_fix(int64_t F, int L, int n, const double* phi, const do
   if (F == 0) return cudaSuccess;
   FaceWeights fw = {};
   for (int q = 0; q < L; ++q) fw.W[q] = W[q];
-  cudaError_t e;
-  if ((e = cudaMalloc((void**)pp, (size_t)F * n * n * L * sizeof(fix::Entry))) != cudaSuccess ||
-      (e = cudaMalloc((void**)p0, (size_t)F * n * L * sizeof(fix::Entry))) != cudaSuccess ||
-      (e = cudaMalloc((void**)exp, (size_t)F * sizeof(int32_t))) != cudaSuccess)
-    return e;
+  const size_t npp = (size_t)F * n * n * L, np0 = (size_t)F * n * L;
+  cudaError_t e = cudaMalloc((void**)pp, (npp + np0) * sizeof(fix::Entry) + F * sizeof(int32_t));
+  if (e != cudaSuccess) return e;
+  *p0 = *pp + npp;
+  *exp = (int32_t*)(*p0 + np0);
   k_face_fix<<<(unsigned)std::min<int64_t>(F, 1 << 16), 64>>>(F, L, n, phi, fw, *pp, *p0, *exp);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   return cudaDeviceSynchronize();

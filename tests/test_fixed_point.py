@@ -163,6 +163,39 @@ static int conversions() {
   return bad;
 }
 
+// Products as entries against 128-bit arithmetic, over the exponents and at the ends.
+static int products() {
+  int bad = 0;
+  auto mant = [](double x, int* e) {
+    const double m = std::frexp(x, e);
+    return (__int128)std::ldexp(m, 53);
+  };
+  for (int trial = 0; trial < 20000; ++trial) {
+    double a = rnd(), b = rnd();
+    if (trial % 3 == 1) a = std::ldexp(a, (int)(1000 * rnd()));
+    if (trial % 5 == 1) b = std::ldexp(b, (int)(20 * rnd()));
+    if (trial % 7 == 1) a = std::rint(8 * a) / 8;
+    if (trial % 11 == 1) a = std::ldexp(a, -1040 - trial % 30);      // subnormal
+    int e, ea, eb;
+    std::frexp(a * b, &e);
+    // a result of up to 61 bits, or far below one unit
+    const int t = a == 0 || b == 0 ? 5 : (trial % 13 == 1 ? -20 - trial % 90 : 60) - e;
+    const __int128 p = mant(a, &ea) * mant(b, &eb);
+    const int sh = 106 - ea - eb - t;                                // a b 2^t = p 2^-sh
+    __int128 want = 0;
+    const __int128 m = p < 0 ? -p : p;
+    if (sh <= 0) want = m << -sh;
+    else if (sh < 120) want = (m + ((__int128)1 << (sh - 1))) >> sh;
+    if (p < 0) want = -want;
+    const fix::Entry q = fix::product(bits(a), bits(b), t);
+    if ((__int128)q.h * (1ll << 30) + q.l / 2 != want || q.l % 2) {
+      std::printf("product %a %a 2^%d\n", a, b, t);
+      bad = 1;
+    }
+  }
+  return bad;
+}
+
 // The faces' sums at their bounds (absolute sum of the products 2^61, values of +-2^57;
 // overflow stops the program) against 128-bit sums, and the 1D face tables.
 template <int N>
@@ -438,7 +471,7 @@ int dg_non_finite() {
 }
 
 int main() {
-  int bad = conversions();
+  int bad = conversions() | products();
   bad |= dg_non_finite<2>() | dg_non_finite<3>() | dg_non_finite<4>() | dg_non_finite<5>() |
          dg_non_finite<6>() | dg_non_finite<7>();
   for (double pen : {4.0, 49.0, 490.0, 4.9e3, 4.9e7, 1e10}) {

@@ -54,6 +54,25 @@ def test_batch_equals_single_applies(dtype):
         assert float((y - y2).abs().max() / y.abs().max()) <= tol
 
 
+def test_batch_tables_are_shared_by_2d_and_3d():
+    """A batch of 2D problems of a degree, created later, leaves the constant
+    tables that a 3D one of that degree reads as they were."""
+    ps = [G.Problem.from_workload(S.SPHERE_3D_Q4.resized(6, degree=p)) for p in range(1, 7)]
+    qs = [G.Problem.from_workload(S.DISK_2D_Q2.resized(9, degree=p)) for p in range(1, 7)]
+    vec = [torch.from_numpy(S.random_vector(3, p.n_dofs, "uniform")).cuda() for p in ps + qs]
+    ref = [p.apply_f64(x) for p, x in zip(ps + qs, vec)]
+    B = G.Batch(ps, 1, autotune=False)
+    for k in range(len(ps)):
+        B.set_tile_shape(k, 0)
+    C = G.Batch(qs, 1, autotune=False)
+    for k in range(len(qs)):
+        C.set_tile_shape(k, 0)
+    for b, xs, ys in ((B, vec[:6], ref[:6]), (C, vec[6:], ref[6:]), (B, vec[:6], ref[:6])):
+        out = [torch.empty_like(x) for x in xs]
+        b.apply(xs, out)
+        assert all(torch.equal(o, y) for o, y in zip(out, ys))
+
+
 def test_batch_tile_shape_3_equals_single_applies():
     """FP32 batches of 3D problems run tile shape 3 (the chunks without
     staged runs) when pinned: bitwise the single FP32 applies (any of tile
