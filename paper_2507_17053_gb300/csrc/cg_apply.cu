@@ -47,10 +47,19 @@ CellLaunch cell_launch_shape(int d, int n) {
 // Resident blocks asked of the compiler.  FP64 3D (fixed-point cell term),
 // blocks of about 250 threads: 6 up to p = 3 (40 registers), 4 above (64; two
 // blocks fewer per SM cost 10 % at p = 4 and 20 % at p = 5, 6); half-size
-// blocks (shape 1) twice as many.
+// blocks (shape 1) twice as many.  The others: none asked (0) gives 32 to 40
+// registers, 1 gives 40 to 72.  Measured with 0 / 1 (us, disks of 400^2 and
+// 900^2 cells): FP64 2D p = 3 56.1, 201 / 55.3, 202, p = 5 116, 500 / 114, 508, p
+// = 6 159, 729 / 156, 719; FP32 2D p = 2 13.8, 25.0 / 14.5, 26.8, p = 6 29.2, 100 /
+// 27.3, 105, half-size blocks p = 6 29.8, 103 / 27.1, 98.8; FP32 3D half-size
+// blocks (balls of 20^3 and 48^3 cells) p = 2 14.0, 15.6 / 13.8, 17.4, p = 5 23.1,
+// 54.1 / 15.4, 51.7.
 template <typename T, int D, int N, int R>
 constexpr int chunk_min_blocks() {
-  return !kFixed<T, D> ? 1 : (N <= 4 ? 6 : 4) * (R * N * N <= 128 ? 2 : 1);
+  constexpr bool half = R < ChunkShape<D, N>::R;
+  if (kFixed<T, D>) return (N <= 4 ? 6 : 4) * (R * N * N <= 128 ? 2 : 1);
+  if (std::is_same<T, double>::value) return N == 6 ? 0 : 1;
+  return half && N >= (D == 2 ? 6 : 4) ? 1 : 0;
 }
 
 template <typename T, int D, int N, int R>
@@ -198,6 +207,16 @@ static cudaError_t chunk_prepare(int* grid_cap) {
   return attr;
 }
 
+static int sm_count() {
+  static const int sms = [] {
+    int dev = 0, v = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+    return v;
+  }();
+  return sms;
+}
+
 // Which part of the operator one apply_r call runs: surrogate faces
 // [f0, f1), chunks [q0, q1), shared DoFs [m0, m1) of the assembly list (all:
 // f1 = q1 = m1 = -1).
@@ -320,8 +339,15 @@ static cudaError_t apply_r(const HostProblem& hp, const DeviceData& dd, const Ch
       int cap = 0;
       if ((err = chunk_prepare<T, D, N, R>(&cap)) != cudaSuccess) return err;
       const int grid = std::min(part.q1 - part.q0, cap);
+      // 2D FP64 p = 6 with 3/4 to 3 full-size blocks per SM starts after the faces:
+      // as a dependent its blocks fall unevenly on the SMs around the face kernel's,
+      // one more on some, 37.6 against 29.3 us (disk of 100^2 cells, 149 blocks) and
+      // 49.7 / 39.6 (148^2, 290); other counts and degrees gain 0 .. 20 %
+      const int64_t quarters = (int64_t)grid * NT / (64 * (int64_t)sm_count());
+      const bool pdl = pdl_cell && !(D == 2 && N == 7 && std::is_same<T, double>::value &&
+                                     quarters >= 3 && quarters < 12);
       if ((err = launch_maybe_pdl(cg_chunk_kernel<T, D, N, R>, dim3(grid, nrhs), dim3(NT), smem,
-                                  st, pdl_cell, a, t)) != cudaSuccess)
+                                  st, pdl, a, t)) != cudaSuccess)
         return err;
       nlaunch++;
     }
