@@ -64,16 +64,16 @@ def alu_roofline(dim, cfma, cops, cell_ms, probe):
 # from one ncu capture per (workload, tile shape, store mode) of the kernel as
 # it stood when captured (dram__bytes_read.sum + dram__bytes_write.sum), not
 # measured by this run; other shapes and modes: not captured
-CELL_TRAFFIC = {("sphere3d_cg_q4_n96", 0, 0): 129.524736e6 + 110.627328e6}
+CELL_TRAFFIC = {("sphere3d_cg_q4_n96", 0, 0): 129.524736e6 + 110.627328e6,
+                ("sphere3d_cg_q4_n96", 3, 0): 129.660928e6 + 118.488832e6}
 L2_BYTES = 129 * 1024 * 1024
 REF_BUDGET_S = 90.0              # wall-clock budget of the --impl reference run
 
 
 def cell_kernel_name(w, shape, ordered):
-    """The FP64 cell-term kernel that tile shape and store mode launch."""
+    """The FP64 cell-term kernel that tile shape and store mode launch (shape 2: shape 0's)."""
     n = w.degree + 1
-    if shape == 2:
-        return f"cg_cell_reg_kernel<double,{n}> (cell kernel, tile shape 2)"
+    shape = 0 if shape == 2 else shape
     name = ("cg_direct" if shape == 3 else "cg_chunk") + ("_ord" if ordered else "")
     dims = f"{n}" if shape == 3 else f"{w.dim},{n}"
     return (f"{name}_kernel<double,{dims}> (cell kernel, tile shape {shape}, "

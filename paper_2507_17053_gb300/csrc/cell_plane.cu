@@ -23,8 +23,8 @@
 // The results are bitwise those of tile shape 0; the assembly kernel of that
 // shape completes the DoFs several colours share.
 // Measured on GB300, FP32 applies with the best other tile shape -> this:
-// Q4 sphere of 96^3 cells 132 (one thread per cell, cell_reg.cu, 168 registers
-// and 12 warps per SM) -> 115 us, Q3 57.7 -> 55.7, Q5 of 64^3 88.6 (chunks
+// Q4 sphere of 96^3 cells 132 (one thread per cell, 168 registers and 12 warps
+// per SM) -> 116 us (few cells: f32_few_cells in cg_apply.cu), Q3 57.7 -> 55.7, Q5 of 64^3 88.6 (chunks
 // without staged runs) -> 77, Q6 ellipsoid of 48^3 48.9 -> 46.1 us.  The cell
 // term of the Q4 sphere takes 71 us for 133 MB: load latency (6 of 13 stall
 // cycles per instruction) and 1 180 instructions per warp of six cells.  In

@@ -248,7 +248,7 @@ static cudaError_t apply_r(const HostProblem& hp, const DeviceData& dd, const Ch
   // assembly after the cell kernel.  Measured (unprofiled applies, GB300):
   // FP32 p = 6 ellipsoid (shape 3) 62.7 -> 57.4 us, p = 3 / 4 spheres
   // (shapes 0, 3) 1-5 % faster, shape 2 1-8 % faster (cell_plane.cu); FP64 (with
-  // the fixed-point faces) disk of 1 801 DoFs 18.4 -> 13.4 us, p = 3 box of
+  // the fixed-point faces) disk of 1 801 DoFs 18.0 -> 14.1 us, p = 3 box of
   // 24^3 cells 29.2 -> 22.7, p = 6 ellipsoid 148 -> 137, p = 4 sphere 381 ->
   // 372 us.
   bool pdl_cell = false;

@@ -157,7 +157,8 @@ dg_apply_kernel(const DgArgs<T> a, const __grid_constant__ KTab<T> t) {
 // products of the two integrands, the test functions); four line phases.
 //
 // FP64 runs on the integer units (fixed_point.cuh): the exponent of a cell is
-// the largest of its own and its neighbours', from dg_exp_kernel; r_k of
+// the largest of its own and its neighbours', from dg_exp_kernel (the two sides
+// of a face can differ in it, and then round its terms differently); r_k of
 // 57-bit values leaves at 59 bits, so that the sum of the last phase stays
 // below 2^61.  The penalty is a part of w, and so of that scale, only while it
 // no more than doubles the largest row sum (pen_interior = 1 gives 1.1 to 1.7

@@ -18,11 +18,12 @@
 // of n^2 <= 49 products stay inside 64 bits because the inputs have 57 bits:
 //   |sum h ql| <= 2^62 + 2^36, |sum l qh| <= 49 2^30 2^26 < 2^61.7.
 // The rounding of a value is 2^-57 of the cell's largest one, 2^-60 in every
-// later phase, against 2^-53 of each product in double precision.
+// later phase, against 2^-53 of each product in double precision.  All points of
+// a face share the exponent of the largest extrapolation among them.
 //
 // The double form was bound by the double-precision pipe (95 % busy).
 // Measured on GB300, face kernel, double -> fixed point: Q4 sphere of 96^3
-// cells (21 914 faces) 162 -> 62 us, Q6 ellipsoid of 48^3 cells (4 246 faces)
+// cells (21 912 faces) 162 -> 62 us, Q6 ellipsoid of 48^3 cells (4 248 faces)
 // 193 -> 54 us; whole FP64 applies 484 -> 381 us and 291 -> 147 us, batch of 9
 // problems x 3 right-hand sides 1 130 -> 847 us.
 #pragma once

@@ -244,8 +244,9 @@ SBM_FIX void apply_line(const FE& E, const FO& O, const int64_t (&v)[N], int64_t
 //
 // E is the largest biased exponent of the cell (1 if all are subnormal).
 // Cells with E outside [kExpMin, kExpMax] (zeros, subnormals, near overflow)
-// take the careful conversions; kExpBad marks infinities and NaN (the cell's
-// results are NaN).
+// take the careful conversions (the apply of a zero vector, p = 1 .. 6, takes as long
+// as another in CG, up to 4 % longer in DG); kExpBad marks infinities and NaN
+// (the cell's results are NaN).
 constexpr int kExpMin = 128, kExpMax = 1900, kExpBad = 0x7ff;
 
 SBM_FIX bool plain_exp(int E) { return E >= kExpMin && E <= kExpMax; }

@@ -471,9 +471,9 @@ SolveStatus solve_cg(const ApplyFn<double>& apply, int64_t n, const double* b, d
 // matrix, phi_0 = 1, it is beta / |phi|; one dot product per step ends the
 // cycle on the device (ctl->done), where Givens rotations would be a chain of
 // j dependent operations.
-// Measured, disk of 1 801 DoFs, restart 100, 625 steps (18 us apply each):
-// whole solve 341 -> 26.6 ms (1 216 blocks per dot product, eleven stream
-// operations and a host round trip per step before).
+// Measured, disk of 1 801 DoFs, restart 100, 625 steps: whole solve 341 -> 26.6
+// ms with the apply at 18 us (1 216 blocks per dot product, eleven stream
+// operations and a host round trip per step before), 22.1 ms with it at 14.
 constexpr int GM_MAXB = 304;       // row blocks at most, 2 per SM
 constexpr int GM_SLICES = 8;       // blocks sharing the dot products of the same rows, at most
 constexpr int GM_RING = 4;         // columns in flight to the host
