@@ -129,7 +129,7 @@ def test_dg_neighbours_of_other_magnitudes(w):
 # ---- discontinuous Galerkin: interior-face penalties of every size -----------------
 
 DG_BOX = S._wl("box", 3, 2, 5, S.box((0.0,) * 3, (1.5,) * 3), dg=True, seed=5)
-PENALTIES = [1.0, 2.0, 30.0, 1e3, 1e6, 1e9]    # inside the line operators up to about 3
+PENALTIES = [1.0, 2.0, 30.0, 1e3, 1e6, 1e9]    # in the line operators up to 1.2 .. 2.2
 
 
 def _dg(p, pen=1.0):
